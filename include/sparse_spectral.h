@@ -385,7 +385,7 @@ ss_status solve_set_wait_limit(ss_stamp s, int64_t ns);
 
 /* Tile shape of this stamp's persistent solve: threads per block (128, 256,
  * 512 or 1024), resident blocks per SM (0 = as many as fit) and static work
- * chunks per block.  Takes effect at the next solve.  Default 1024, 1, 1. */
+ * chunks per block.  Takes effect at the next solve.  Default 512, 1, 1. */
 ss_status solve_set_config(ss_stamp s, int32_t block, int32_t blocks_per_sm, int32_t chunks_per_block);
 
 /* Allocation-free variant of solve() (the paper has no counterpart: this is a

@@ -119,6 +119,32 @@ ss_status ensure_ecoefdf_half(ss_stamp_s* s, cudaStream_t st) {
   return SS_OK;
 }
 
+// FP32 copies of the entry coefficients (the refined solve); the entries in
+// use are counted on the device (woff[n_slices] rows of 32), so nothing is
+// read back.
+__global__ void k_ecoef_f32(const double* __restrict__ in, const int32_t* __restrict__ rows, int per_entry,
+                            const int32_t* __restrict__ err, float* __restrict__ out) {
+  if (__ldg(err) != 0) return;   // a failed build: the offsets are incomplete
+  const int64_t n2 = (int64_t)__ldg(rows) * kSlice * per_entry / 2;   // pairs (32 rows: always whole)
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(in) + i);
+    reinterpret_cast<float2*>(out)[i] = make_float2((float)v.x, (float)v.y);
+  }
+}
+
+ss_status ensure_ecoef32(ss_stamp_s* s, bool half, cudaStream_t st) {
+  DevBuf<float>& dst = half ? s->ecoef32_h : s->ecoef32;
+  if (dst.get()) return SS_OK;
+  const int per = s->a_real ? 1 : 2;
+  const int64_t cap = half ? (int64_t)s->ecoef_h.n : s->n_ent + 1;
+  SS_TRY(dst.alloc((size_t)cap * per, st));
+  const int32_t* rows = half ? s->woff_h.get() + s->n_slices_h : s->slice_off.get() + s->n_slices;
+  k_ecoef_f32<<<4 * sm_count(), 256, 0, st>>>(
+      reinterpret_cast<const double*>(half ? s->ecoef_h.get() : s->ecoef64.get()), rows, per, s->err_dev.get(), dst.get());
+  SS_LAUNCH_CHECK();
+  return SS_OK;
+}
+
 OpView op_view(const ss_stamp_s* s) {
   OpView op;
   op.woff = s->slice_off.get();

@@ -36,6 +36,10 @@ struct OpView {
   uint32_t colmask;
   bool conj = false;       // half system: entry bit 31 set = the neighbour's value is conjugated
   uint32_t jmask = 0xffffffffu;   // step index = (entry >> colbits) & jmask
+  const float2* ecoef32 = nullptr;   // FP32 coefficient of every entry (realc: one float per entry), or null
+  uint32_t pad = 0;        // column of padding entries (an all-zero record)
+  bool diag0 = false;      // the diagonal is every row's first entry (half tables)
+  bool scaled = false;     // black rows hold -c / D off the diagonal (half tables with colours)
   bool realc = false;      // every entry coefficient has imaginary part exactly 0 (real a_hat)
 };
 
@@ -55,11 +59,12 @@ __device__ __forceinline__ float conj_if(float y, bool conj, uint32_t ent) {
 // Accumulate row `row` (lane of slice s) of L u in FP64 from the stored entry
 // coefficients: four FP64 FMAs per nonzero, two when the coefficients are real
 // (REAL: their imaginary parts are exactly 0, so the two dropped products add
-// exact zeros).  GB300 issues one FP64 FMA per SM clock, so the FP64 operator
-// counts its FP64 instructions.
-template <bool CG, bool REAL>
+// exact zeros).  GB300 retires two FP64 FMAs per SM clock, so the FP64 operator
+// counts its FP64 instructions.  SKIP leaves out the entries of column `self`
+// (the row's own record is read as zero).
+template <bool CG, bool REAL, bool SKIP>
 __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, int lane,
-                                                 const double2* __restrict__ rec) {
+                                                 const double2* rec, uint32_t self) {
   const int32_t w0 = __ldg(op.woff + s), w1 = __ldg(op.woff + s + 1);
   const int64_t base = (int64_t)w0 * kSlice + lane;
   const uint32_t* e = op.ent + base;
@@ -81,6 +86,7 @@ __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, in
     for (int q = 0; q < 4; ++q) {
       v[q] = ldv<CG>(rec + (ee[q] & op.colmask));
       v[q].y = conj_if(v[q].y, op.conj, ee[q]);
+      if (SKIP && (ee[q] & op.colmask) == self) v[q] = make_double2(0.0, 0.0);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -97,6 +103,7 @@ __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, in
     const uint32_t ee = __ldg(e + (int64_t)t * kSlice);
     double2 v = ldv<CG>(rec + (ee & op.colmask));
     v.y = conj_if(v.y, op.conj, ee);
+    if (SKIP && (ee & op.colmask) == self) v = make_double2(0.0, 0.0);
     if constexpr (REAL) {
       const double c = __ldg(cfr + (int64_t)t * kSlice);
       ar = fma(c, v.x, ar);
@@ -110,79 +117,11 @@ __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, in
   return make_double2(ar, ai);
 }
 
-template <bool CG = false>
-__device__ __forceinline__ double2 row_apply64(const OpView& op, int64_t s, int lane,
-                                               const double2* __restrict__ rec) {
-  return op.realc ? row_apply64_t<CG, true>(op, s, lane, rec) : row_apply64_t<CG, false>(op, s, lane, rec);
-}
-
-// Same in double-float (DF64 mode): the FP64 entry coefficient and u_l as
-// unevaluated float pairs, four double-float multiply-adds per nonzero on the
-// FP32 pipe (about 2^-48 relative per operation).  rec: float4 per column.
-template <bool CG, bool REAL>
-__device__ __forceinline__ float4 row_applydf_t(const OpView& op, int64_t s, int lane,
-                                                const float4* __restrict__ rec) {
-  const int32_t w0 = __ldg(op.woff + s), w1 = __ldg(op.woff + s + 1);
-  const int64_t base = (int64_t)w0 * kSlice + lane;
-  const uint32_t* e = op.ent + base;
-  const float4* cf = op.ecoefdf + base;
-  DF ar{0.f, 0.f}, ai{0.f, 0.f};
-  int t = 0;
-  const int w = w1 - w0;
-  for (; t + 4 <= w; t += 4) {
-    uint32_t ee[4];
-    float4 c[4], v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      ee[q] = __ldg(e + (int64_t)(t + q) * kSlice);
-      if constexpr (REAL) {
-        const float2 h = __ldg(reinterpret_cast<const float2*>(cf + (int64_t)(t + q) * kSlice));
-        c[q] = make_float4(h.x, h.y, 0.f, 0.f);
-      } else {
-        c[q] = __ldg(cf + (int64_t)(t + q) * kSlice);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      v[q] = ldv<CG>(rec + (ee[q] & op.colmask));
-      v[q].z = conj_if(v[q].z, op.conj, ee[q]);
-      v[q].w = conj_if(v[q].w, op.conj, ee[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      df_fma(ar, re_of(c[q]), re_of(v[q]));
-      df_fma(ai, re_of(c[q]), im_of(v[q]));
-      if constexpr (!REAL) {
-        df_fma(ar, df_neg(im_of(c[q])), im_of(v[q]));
-        df_fma(ai, im_of(c[q]), re_of(v[q]));
-      }
-    }
-  }
-  for (; t < w; ++t) {
-    const uint32_t ee = __ldg(e + (int64_t)t * kSlice);
-    float4 v = ldv<CG>(rec + (ee & op.colmask));
-    v.z = conj_if(v.z, op.conj, ee);
-    v.w = conj_if(v.w, op.conj, ee);
-    float4 c;
-    if constexpr (REAL) {
-      const float2 h = __ldg(reinterpret_cast<const float2*>(cf + (int64_t)t * kSlice));
-      c = make_float4(h.x, h.y, 0.f, 0.f);
-    } else {
-      c = __ldg(cf + (int64_t)t * kSlice);
-    }
-    df_fma(ar, re_of(c), re_of(v));
-    df_fma(ai, re_of(c), im_of(v));
-    if constexpr (!REAL) {
-      df_fma(ar, df_neg(im_of(c)), im_of(v));
-      df_fma(ai, im_of(c), re_of(v));
-    }
-  }
-  return cdf(ar, ai);
-}
-
-template <bool CG = false>
-__device__ __forceinline__ float4 row_applydf(const OpView& op, int64_t s, int lane, const float4* __restrict__ rec) {
-  return op.realc ? row_applydf_t<CG, true>(op, s, lane, rec) : row_applydf_t<CG, false>(op, s, lane, rec);
+template <bool CG = false, bool SKIP = false>
+__device__ __forceinline__ double2 row_apply64(const OpView& op, int64_t s, int lane, const double2* rec,
+                                               uint32_t self = 0) {
+  return op.realc ? row_apply64_t<CG, true, SKIP>(op, s, lane, rec, self)
+                  : row_apply64_t<CG, false, SKIP>(op, s, lane, rec, self);
 }
 
 // Same in FP32 (FP32 values, FP32 accumulation).  nk, the records' third
@@ -196,10 +135,10 @@ __device__ __forceinline__ float entry_scale(int32_t nk, float rec_z, int32_t pn
 
 // U index words per lane are loaded before their U gathers are issued, so a
 // row of width <= U costs one index round trip and one gather round trip.
-template <bool CG, bool WIDE, int U>
+template <bool CG, bool WIDE, bool SKIP, int U>
 __device__ __forceinline__ float2 row_apply32_t(const OpView& op, int64_t s, int lane, int32_t nk,
-                                                const float4* __restrict__ rec, const float2* ca,
-                                                const int32_t* pn) {
+                                                const float4* rec, const float2* ca, const int32_t* pn,
+                                                uint32_t self) {
   const int32_t w0 = __ldg(op.woff + s), w1 = __ldg(op.woff + s + 1);
   const uint32_t* e = op.ent + (int64_t)w0 * kSlice + lane;
   float ar = 0.f, ai = 0.f;
@@ -213,6 +152,7 @@ __device__ __forceinline__ float2 row_apply32_t(const OpView& op, int64_t s, int
     for (int q = 0; q < U; ++q) {
       v[q] = t + q < w ? ldv<CG>(rec + (ee[q] & op.colmask)) : make_float4(0.f, 0.f, 0.f, 0.f);
       v[q].y = conj_if(v[q].y, op.conj, ee[q]);
+      if (SKIP && (ee[q] & op.colmask) == self) v[q].x = v[q].y = 0.f;
     }
 #pragma unroll
     for (int q = 0; q < U; ++q) {
@@ -269,12 +209,12 @@ __device__ __forceinline__ float2 row_apply32_direct(const OpView& op, int64_t s
   return make_float2(ar, ai);
 }
 
-template <bool CG = false, int U = 4>
+template <bool CG = false, bool SKIP = false, int U = 4>
 __device__ __forceinline__ float2 row_apply32(const OpView& op, int64_t s, int lane, int64_t nk, bool wide,
-                                              const float4* __restrict__ rec, const float2* ca,
-                                              const int32_t* pn) {
-  return wide ? row_apply32_t<CG, true, U>(op, s, lane, norm_word(nk, true), rec, ca, pn)
-              : row_apply32_t<CG, false, U>(op, s, lane, norm_word(nk, false), rec, ca, pn);
+                                              const float4* rec, const float2* ca, const int32_t* pn,
+                                              uint32_t self = 0) {
+  return wide ? row_apply32_t<CG, true, SKIP, U>(op, s, lane, norm_word(nk, true), rec, ca, pn, self)
+              : row_apply32_t<CG, false, SKIP, U>(op, s, lane, norm_word(nk, false), rec, ca, pn, self);
 }
 
 }  // namespace ss

@@ -26,6 +26,8 @@ struct ss_batch_s {
   ss::DevBuf<double2> ca64, ecoef64;
   ss::DevBuf<float2> ca32;
   std::vector<int32_t> woff_h, slice_inst_h;
+  ss::DevBuf<uint32_t> cmask;         // the instances' colour masks (zero: a set without colours)
+  std::vector<uint32_t> cmask_h;      // host copy; empty when no instance has colours
   ss::SolvePlan plan;
   ss::SolveWork work;
   // tile shape
@@ -141,15 +143,16 @@ inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t
 
 ss_status replan(ss_batch_s* b, int mode, cudaStream_t st) {
   int grid_max = 0;
-  SS_TRY(max_grid(mode, b->block, &grid_max));
+  SS_TRY(max_grid(mode, false, false, b->block, &grid_max));
   int grid = grid_max;
   if (b->blocks_per_sm > 0) grid = std::min(grid_max, b->blocks_per_sm * sm_count());
   const int64_t by_size = std::max<int64_t>(1, b->n_slices / 8);
   const int target = (int)std::min<int64_t>((int64_t)grid * b->chunks_per_block, by_size);
-  SS_TRY(plan_chunks(b->plan, b->woff_h, b->slice_inst_h, target));
+  SS_TRY(plan_chunks(b->plan, b->woff_h, b->slice_inst_h, b->cmask_h, target));
+  b->plan.black = b->cmask_h.empty() ? nullptr : b->cmask.get();
   b->plan.block = b->block;
-  b->plan.grid = std::min<int>(grid, (int)b->plan.chunk.size());
-  SS_TRY(work_upload(b->work, b->plan, st));
+  b->plan.grid = std::min<int>(grid, std::max(b->plan.n_chunks[0], b->plan.n_chunks[1]));
+  SS_TRY(work_upload(b->work, b->plan, true, st));
   b->planned = true;
   b->planned_mode = mode;
   if (b->graph) {
@@ -170,13 +173,14 @@ OpView batch_op(const ss_batch_s* b) {
   op.jmask = (1u << b->jbits) - 1u;
   op.conj = b->conj;
   op.realc = b->realc;
+  op.scaled = b->conj;   // half tables (those without colours have no black rows)
   return op;
 }
 
 ss_status run_once(ss_batch_s* b, double tol, int max_iter, ss_precision prec, bool use_graph, cudaStream_t st) {
   const int mode = prec == SS_FP64 ? 0 : 1;
   if (!b->planned || b->planned_mode != mode) SS_TRY(replan(b, mode, st));
-  SS_TRY(work_upload(b->work, b->plan, st));   // f/u pointers may have changed
+  SS_TRY(work_upload(b->work, b->plan, false, st));   // f/u pointers may have changed
   if (!b->work.ev[0]) {
     SS_CUDA(cudaEventCreate(&b->work.ev[0]));
     SS_CUDA(cudaEventCreate(&b->work.ev[1]));
@@ -244,19 +248,21 @@ struct SysIn {
   const double2* ecoef;
   int colbits, jbits;
   uint32_t colmask;
+  const uint32_t* black;                  // colour masks, or null
+  const std::vector<uint32_t>* black_host;
 };
 
 SysIn full_in(const ss_stamp_s* s) {
   return SysIn{s->size, s->rows_pad, s->n_slices, s->n_ent, s->zero_idx, s->norm.get(), s->slice_off.get(),
                &s->woff_host, s->ent.get(), s->ecoef64.get(), colbits_of(s->jbits), s->jbits,
-               colmask_of(s->jbits)};
+               colmask_of(s->jbits), s->colours ? s->cmask.get() : nullptr, &s->cmask_host};
 }
 
 SysIn half_in(const ss_stamp_s* s) {
   const int64_t n_ent_h = s->woff_h_host.empty() ? 0 : (int64_t)s->woff_h_host.back() * kSlice;
   return SysIn{s->n_plus, s->rows_pad_h, s->n_slices_h, n_ent_h, -1, s->norm_h.get(), s->woff_h.get(),
                &s->woff_h_host, s->ent_h.get(), s->ecoef_h.get(), s->colbits_h, s->jbits,
-               (uint32_t)((1u << s->colbits_h) - 1u)};
+               (uint32_t)((1u << s->colbits_h) - 1u), s->colours ? s->cmask_h.get() : nullptr, &s->cmask_h_host};
 }
 
 }  // namespace
@@ -298,6 +304,13 @@ static ss_status batch_create_impl(ss_batch_s* b, int32_t n, const ss_stamp* sta
   DevBuf<int8_t> wide_rows;
   SS_TRY(wide_rows.alloc(b->rows_total, st));
   SS_CUDA(cudaMemsetAsync(wide_rows.get(), 0, b->rows_total, st));
+  bool colours = false;
+  for (int i = 0; i < n; ++i) colours = colours || in[i].black;
+  if (colours) {
+    SS_TRY(b->cmask.alloc(slices, st));
+    SS_CUDA(cudaMemsetAsync(b->cmask.get(), 0, slices * sizeof(uint32_t), st));
+  }
+  b->cmask_h.assign(colours ? slices : 0, 0u);
   b->woff_h.assign(slices + 1, 0);
   b->slice_inst_h.assign(slices, 0);
   b->plan.inst.assign(n, SolveInst{});
@@ -330,6 +343,11 @@ static ss_status batch_create_impl(ss_batch_s* b, int32_t n, const ss_stamp* sta
     SS_CUDA(cudaMemcpyAsync(b->pn.get() + c0, s->pn32.get(), s->s_a * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     const std::vector<int32_t>& w = *x.woff_host;
     if ((int64_t)w.size() != x.n_slices + 1) SS_FAIL(SS_ERR_INVALID, "batch_create: stamp %d has no slice table", i);
+    if (x.black) {
+      if ((int64_t)x.black_host->size() != x.n_slices) SS_FAIL(SS_ERR_INVALID, "batch_create: stamp %d has no colour masks", i);
+      SS_CUDA(cudaMemcpyAsync(b->cmask.get() + s0, x.black, x.n_slices * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
+      std::copy(x.black_host->begin(), x.black_host->end(), b->cmask_h.begin() + s0);
+    }
     for (int64_t q = 0; q <= x.n_slices; ++q) b->woff_h[s0 + q] = w[q] + (int32_t)(e0 / kSlice);
     for (int64_t q = 0; q < x.n_slices; ++q) b->slice_inst_h[s0 + q] = i;
     SolveInst& si = b->plan.inst[i];
@@ -349,7 +367,7 @@ static ss_status batch_create_impl(ss_batch_s* b, int32_t n, const ss_stamp* sta
   SS_TRY(work_alloc(b->work, b->rows_total, b->norm.get(), wide_rows.get(), false, st));
   SS_CUDA(cudaStreamSynchronize(st));
   b->norm.settle(); b->woff.settle(); b->slice_inst.settle(); b->ent.settle();
-  b->ca64.settle(); b->ca32.settle(); b->pn.settle(); b->ecoef64.settle();
+  b->ca64.settle(); b->ca32.settle(); b->pn.settle(); b->ecoef64.settle(); b->cmask.settle();
   return SS_OK;
 }
 
@@ -584,7 +602,7 @@ extern "C" ss_status batch_config(ss_batch b, int32_t* block, int32_t* blocks_pe
   if (blocks_per_sm) *blocks_per_sm = b->blocks_per_sm;
   if (chunks_per_block) *chunks_per_block = b->chunks_per_block;
   if (grid) *grid = t->plan.grid;
-  if (n_chunks) *n_chunks = (int32_t)t->plan.chunk.size();
+  if (n_chunks) *n_chunks = t->plan.n_chunks[0];
   return SS_OK;
 }
 

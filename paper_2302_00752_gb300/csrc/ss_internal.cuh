@@ -278,7 +278,14 @@ struct ss_stamp_s {
   ss::DevBuf<double2> ecoef_h;        // FP64 entry coefficients of the half table
   ss::DevBuf<int64_t> norm_h;         // [rows_pad_h + 1] |k|^2 of the compact rows (0 on padding)
   ss::DevBuf<float4> ecoefdf_h;       // the half table's coefficients as double-float (first DF64 solve)
+  ss::DevBuf<float> ecoef32, ecoef32_h;   // FP32 copies of both (first refined solve; real: one float per entry)
   std::vector<int32_t> woff_h_host;   // host copy of woff_h, filled on demand (stamp_host_tables)
+  // two-colour masks of the solver (solve.cu): bit = the row is black (a row
+  // of level N, N - 2, ... with no neighbour among the other black rows; also
+  // padding); only when `colours`
+  bool colours = false;
+  ss::DevBuf<uint32_t> cmask, cmask_h;          // [n_slices], [n_slices_h]
+  std::vector<uint32_t> cmask_host, cmask_h_host;   // host copies (stamp_host_tables)
   // error words of the build not yet read (stamp_build_pending); the half
   // system is tentative until they are (stamp_check_pending)
   bool check_pending = false;
@@ -314,6 +321,8 @@ ss_status launch_apply32(const ss_stamp_s* s, const float2* u, float2* y, cudaSt
 // Double-float copy of the FP64 entry coefficients (built once per operator).
 ss_status ensure_ecoefdf(ss_stamp_s* s, cudaStream_t st);
 ss_status ensure_ecoefdf_half(ss_stamp_s* s, cudaStream_t st);
+// FP32 copy of the full or half table's entry coefficients (asynchronous).
+ss_status ensure_ecoef32(ss_stamp_s* s, bool half, cudaStream_t st);
 
 int sm_count();
 

@@ -701,14 +701,42 @@ __global__ void k_slice_widths(const int32_t* __restrict__ cnt, int64_t size, in
   }
 }
 
+// Levels of the set as row ranges: start[t] is the first row of level t + 1.
+constexpr int kColourLevels = 16;
+struct LevelStarts {
+  int n = 0;   // N, 0: no colours
+  int32_t start[kColourLevels];
+};
+
+// Row i lies in level N, N - 2, ...
+__device__ __forceinline__ bool black_level(const LevelStarts& L, int32_t i) {
+  int lvl = 0;
+  for (int t = 0; t < L.n; ++t) lvl += i >= L.start[t];
+  return ((L.n - lvl) & 1) == 0;
+}
+
+// The same for k and -k (their linear forms are lin(bias) +- c), different for
+// any other pair up to a 64-bit coincidence.
+__device__ __forceinline__ uint64_t sym_label(uint64_t lin, uint64_t lin_bias) {
+  const uint64_t c = lin - lin_bias, m = 0ull - c;
+  return c < m ? c : m;
+}
+
 // Entries of a row in step order, then padding (dummy column rows_pad, zero
 // coefficient).  Also stores the FP64 coefficient of every entry,
 // (|k|^2 + |l|^2 - |p_j|^2) * 2 pi^2 a_hat_j = 4 pi^2 (k.l) a_hat_j (eq. GF), so
 // that the FP64 operator spends four FP64 FMAs per nonzero.
+// With levels given, also the solver's colour mask of the slice: black rows lie
+// in level N, N - 2, ... and have no black neighbour.  Of two neighbours in
+// those levels the one with the smaller label turns red (both when the labels
+// agree), so k and -k keep one colour and what stays black is independent.
+// The level of a neighbour follows from its index (rows are ordered by level):
+// no extra gather, and the labels are read only for such pairs.
 __global__ void k_fill_slices(NbrView nb, int64_t size, int64_t rows_pad, int s_a, int j0,
                               const int32_t* __restrict__ woff, int colbits, const int64_t* __restrict__ norm,
                               const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64, uint32_t* ent,
-                              double2* ecoef, bool real) {
+                              double2* ecoef, bool real, const uint64_t* __restrict__ hl, uint64_t lin_bias,
+                              int64_t zero_idx, LevelStarts lv, uint32_t* cmask) {
   double* ecoef_re = reinterpret_cast<double*>(ecoef);   // real coefficients: one double per entry
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= rows_pad) return;
@@ -717,6 +745,7 @@ __global__ void k_fill_slices(NbrView nb, int64_t size, int64_t rows_pad, int s_
   const int64_t base = (int64_t)woff[s] * kSlice + lane;
   const int w = woff[s + 1] - woff[s];
   int t = 0;
+  bool blk = lv.n > 0 && (i >= size || (i != zero_idx && black_level(lv, (int32_t)i)));
   if (i < size) {
     const int64_t nk = norm[i];
     for (int ub = 0; ub < nb.Ls + nb.Hs; ub += kNbrBatch) {
@@ -739,8 +768,14 @@ __global__ void k_fill_slices(NbrView nb, int64_t size, int64_t rows_pad, int s_
         const double sc = (double)(nk + nv[q] - pnorm[j]);
         if (real) ecoef_re[e] = sc * ca64[j].x;
         else ecoef[e] = make_double2(sc * ca64[j].x, sc * ca64[j].y);
+        if (blk && v[q] != i && black_level(lv, v[q]))
+          blk = sym_label(__ldg(hl + v[q]), lin_bias) < sym_label(__ldg(hl + i), lin_bias);
       }
     }
+  }
+  if (lv.n > 0) {   // rows_pad is a whole number of warps
+    const uint32_t m = __ballot_sync(0xffffffffu, blk);
+    if (lane == 0) cmask[s] = m;
   }
   const uint32_t pad = (uint32_t)rows_pad | ((uint32_t)j0 << colbits);
   for (; t < w; ++t) {
@@ -1181,12 +1216,17 @@ __global__ void k_half_widths(const int32_t* __restrict__ plus_rows, int64_t n_p
   if ((threadIdx.x & 31) == 0) slice_w[i / kSlice] = m;
 }
 
+// Entries of the half table: the diagonal first, the others in step order.
+// With colours the black rows hold -c / D off the diagonal: the solver's black
+// half pass v_B = -D_B^-1 C^H u_R is then the row product alone, without the
+// diagonal's entry and without a division or product per row and iteration.
 __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plus, int64_t rows_pad_h,
                             const int32_t* __restrict__ woff, const uint32_t* __restrict__ ent,
                             const double2* __restrict__ ecoef, uint32_t colmask, int colbits, int64_t pad_col,
                             int colbits_h, int j0, const int32_t* __restrict__ hpos,
                             const int32_t* __restrict__ woff_h, uint32_t* ent_h, double2* ecoef_h, bool real,
-                            const int32_t* __restrict__ err) {
+                            const int32_t* __restrict__ err, const uint32_t* __restrict__ cmask, uint32_t* cmask_h,
+                            const int64_t* __restrict__ norm_h, double dscale) {
   const double* ecoef_re = reinterpret_cast<const double*>(ecoef);
   double* ecoef_h_re = reinterpret_cast<double*>(ecoef_h);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1197,11 +1237,20 @@ __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plu
   const int64_t base_h = (int64_t)woff_h[sh] * kSlice + (i % kSlice);
   const int w_h = woff_h[sh + 1] - woff_h[sh];
   int t = 0;
+  bool blk = false;
+  if (cmask) {   // the rows' colours (null: none)
+    const int64_t g = i < n_plus ? plus_rows[i] : -1;
+    blk = g < 0 || ((__ldg(cmask + g / kSlice) >> (g % kSlice)) & 1u);
+    const uint32_t m = __ballot_sync(0xffffffffu, blk);
+    if (i % kSlice == 0) cmask_h[sh] = m;
+  }
   if (i < n_plus) {
     const int64_t g = plus_rows[i];
     const int64_t s = g / kSlice;
     const int64_t base = (int64_t)woff[s] * kSlice + (g % kSlice);
     const int w = woff[s + 1] - woff[s];
+    const double sc = blk ? -1.0 / (dscale * (double)norm_h[i]) : 1.0;
+    t = 1;   // entry 0: the diagonal
     for (int tf0 = 0; tf0 < w; tf0 += kNbrBatch) {
       // entry words, then the gathered positions, loaded before use
       uint32_t ev[kNbrBatch];
@@ -1221,10 +1270,16 @@ __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plu
         const int64_t e = base + (int64_t)(tf0 + q) * kSlice;
         const uint32_t col = h >= 0 ? (uint32_t)h : (uint32_t)(-2 - h);
         const uint32_t j = ev[q] >> colbits;
-        ent_h[base_h + (int64_t)t * kSlice] = col | (j << colbits_h) | (h < 0 ? 0x80000000u : 0u);
-        if (real) ecoef_h_re[base_h + (int64_t)t * kSlice] = ecoef_re[e];
-        else ecoef_h[base_h + (int64_t)t * kSlice] = ecoef[e];
-        ++t;
+        const bool dg = (int)j == j0;
+        const int64_t eh = base_h + (dg ? 0 : (int64_t)t++ * kSlice);
+        const double m = dg ? 1.0 : sc;
+        ent_h[eh] = col | (j << colbits_h) | (h < 0 ? 0x80000000u : 0u);
+        if (real) {
+          ecoef_h_re[eh] = m * ecoef_re[e];
+        } else {
+          const double2 c = ecoef[e];
+          ecoef_h[eh] = make_double2(m * c.x, m * c.y);
+        }
       }
     }
   }
@@ -1258,7 +1313,8 @@ static ss_status build_half(ss_stamp_s* S, cudaStream_t st) {
   SS_TRY(S->hpos.alloc(S->size, st));
   SS_TRY(S->plus_rows.alloc(S->rows_pad_h, st));
   SS_TRY(S->norm_h.alloc(S->rows_pad_h + 1, st));
-  SS_TRY(S->woff_h.alloc(S->n_slices_h + 1, st));
+  SS_TRY(S->woff_h.alloc(2 * S->n_slices_h + 1, st));   // and the colour masks
+  S->cmask_h.view(reinterpret_cast<uint32_t*>(S->woff_h.get() + S->n_slices_h + 1), S->n_slices_h);
   // Entries of the half table: every compact slice is at most as wide as the
   // widest row it holds; the plus rows of one full slice are consecutive
   // compact rows, so they fall in at most two compact slices and the half
@@ -1298,7 +1354,9 @@ static ss_status build_half(ss_stamp_s* S, cudaStream_t st) {
     k_half_fill<<<nblk(S->rows_pad_h), 256, 0, st>>>(S->plus_rows.get(), n_plus, S->rows_pad_h, S->slice_off.get(),
                                                      S->ent.get(), S->ecoef64.get(), colmask, colbits_of(S->jbits),
                                                      S->rows_pad, S->colbits_h, S->j0, S->hpos.get(), S->woff_h.get(),
-                                                     S->ent_h.get(), S->ecoef_h.get(), S->a_real, S->err_dev.get());
+                                                     S->ent_h.get(), S->ecoef_h.get(), S->a_real, S->err_dev.get(),
+                                                     S->colours ? S->cmask.get() : nullptr, S->cmask_h.get(),
+                                                     S->norm_h.get(), 2.0 * kTwoPiSq * S->a0);
   }
   SS_LAUNCH_CHECK();
   S->woff_h_host.clear();   // host copy on demand (stamp_host_tables)
@@ -1375,7 +1433,8 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
                                                       d_wmax.get());
   }
   SS_LAUNCH_CHECK();
-  SS_TRY(S->slice_off.alloc(S->n_slices + 1, st));
+  SS_TRY(S->slice_off.alloc(2 * S->n_slices + 1, st));   // and the colour masks
+  S->cmask.view(reinterpret_cast<uint32_t*>(S->slice_off.get() + S->n_slices + 1), S->n_slices);
   SS_TRY(scan_lookback(LbRead{slice_w.get()}, LbWrite{S->slice_off.get()}, S->n_slices + 1, d_total.get(),
                        S->err_dev.get(), st));
   int64_t total_w = 0;
@@ -1394,8 +1453,27 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   S->n_ent = total_w * kSlice;
   SS_TRY(S->ent.alloc(S->n_ent + 1, st));
   SS_TRY(S->ecoef64.alloc(S->n_ent + 1, st));
+  LevelStarts lv;
+  S->colours = false;
+  if (!S->adr && S->N >= 1 && S->N <= kColourLevels) {
+    int64_t red = 0;   // rows of the other levels, apart from k = 0
+    for (int t = 0; t <= S->N; ++t)
+      if ((S->N - t) & 1) {
+        const int64_t a = S->level_start[t], b = S->level_start[t + 1];
+        red += b - a - (S->zero_idx >= a && S->zero_idx < b);
+      }
+    if (red > 0) {
+      S->colours = true;
+      lv.n = S->N;
+      for (int t = 0; t < S->N; ++t) lv.start[t] = (int32_t)S->level_start[t + 1];
+    }
+  }
+  S->cmask_host.clear();
+  S->cmask_h_host.clear();
   S->ecoefdf.release();   // rebuilt from ecoef64 by the next DF64 solve
   S->ecoefdf_h.release();
+  S->ecoef32.release();
+  S->ecoef32_h.release();
   if (S->adr) {
     SS_TRY(S->diag64.alloc(S->rows_pad + 1, st));
     SS_DISPATCH_WT(S->key.WT, (k_fill_slices_adr<WT><<<nblk(S->rows_pad + 1), 256, 0, st>>>(
@@ -1408,7 +1486,8 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
       k_fill_slices<<<nblk(S->rows_pad), 256, 0, st>>>(nb, S->size, S->rows_pad, s_a, S->j0,
                                                        S->slice_off.get(), colbits_of(S->jbits), S->norm.get(),
                                                        S->pnorm.get(), S->ca64.get(), S->ent.get(), S->ecoef64.get(),
-                                                       S->a_real);
+                                                       S->a_real, S->hl.get(), P.lin_bias, S->zero_idx, lv,
+                                                       S->cmask.get());
     }
   }
   SS_LAUNCH_CHECK();
@@ -1647,6 +1726,8 @@ static void rebind(ss_stamp_s* S, cudaStream_t st) {
   S->ecoef64.s = st;
   S->ecoefdf.s = st;
   S->ecoefdf_h.s = st;
+  S->ecoef32.s = st;
+  S->ecoef32_h.s = st;
   S->nw32.s = st;
   S->rec64.s = st;
   S->diag64.s = st;
@@ -1724,11 +1805,17 @@ ss_status stamp_host_tables(ss_stamp_s* S, cudaStream_t st) {
   int32_t e[4] = {0, 0, 0, 0};
   if (need_full) S->woff_host.resize(S->n_slices + 1);
   if (need_half) S->woff_h_host.resize(S->n_slices_h + 1);
+  const bool mf = need_full && S->colours, mh = need_half && S->colours;
+  S->cmask_host.resize(S->colours ? S->n_slices : 0);
+  S->cmask_h_host.resize(S->colours && S->half_ok ? S->n_slices_h : 0);
   SS_TRY(read_back(st, {{e, S->err_dev.get(), sizeof(e)},
                         {need_full ? S->woff_host.data() : nullptr, S->slice_off.get(),
                          need_full ? (S->n_slices + 1) * sizeof(int32_t) : 0},
                         {need_half ? S->woff_h_host.data() : nullptr, S->woff_h.get(),
-                         need_half ? (S->n_slices_h + 1) * sizeof(int32_t) : 0}}));
+                         need_half ? (S->n_slices_h + 1) * sizeof(int32_t) : 0},
+                        {mf ? S->cmask_host.data() : nullptr, S->cmask.get(), mf ? S->n_slices * sizeof(uint32_t) : 0},
+                        {mh ? S->cmask_h_host.data() : nullptr, S->cmask_h.get(),
+                         mh ? S->n_slices_h * sizeof(uint32_t) : 0}}));
   SS_TRY(stamp_check_pending(S, e));
   if (!S->half_ok) S->woff_h_host.clear();
   return SS_OK;
