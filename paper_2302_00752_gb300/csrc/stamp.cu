@@ -708,11 +708,24 @@ struct LevelStarts {
   int32_t start[kColourLevels];
 };
 
-// Row i lies in level N, N - 2, ...
-__device__ __forceinline__ bool black_level(const LevelStarts& L, int32_t i) {
+// Rows [first, first + n) of row i's level when that is level N, N - 2, ...,
+// else no rows.
+__device__ __forceinline__ void black_level(const LevelStarts& L, int32_t i, int32_t size, int32_t* first, uint32_t* n) {
   int lvl = 0;
-  for (int t = 0; t < L.n; ++t) lvl += i >= L.start[t];
-  return ((L.n - lvl) & 1) == 0;
+  int32_t a = 0, b = size;
+#pragma unroll
+  for (int t = 0; t < kColourLevels; ++t) {   // unrolled: a dynamic index would copy the argument to local memory
+    if (t >= L.n) continue;
+    const int32_t s = L.start[t];
+    if (i >= s) {
+      a = s;
+      ++lvl;
+    } else {
+      b = min(b, s);
+    }
+  }
+  *first = a;
+  *n = ((L.n - lvl) & 1) == 0 ? (uint32_t)(b - a) : 0u;
 }
 
 // The same for k and -k (their linear forms are lin(bias) +- c), different for
@@ -720,6 +733,21 @@ __device__ __forceinline__ bool black_level(const LevelStarts& L, int32_t i) {
 __device__ __forceinline__ uint64_t sym_label(uint64_t lin, uint64_t lin_bias) {
   const uint64_t c = lin - lin_bias, m = 0ull - c;
   return c < m ? c : m;
+}
+
+// Row i has the larger label than each of its neighbours of the same level
+// (rows [own0, own0 + own_n)); called for the few rows that have one.
+__device__ __noinline__ bool black_wins(NbrView nb, int64_t i, int32_t own0, uint32_t own_n,
+                                        const uint64_t* __restrict__ hl, uint64_t lin_bias) {
+  const uint64_t mine = sym_label(__ldg(hl + i), lin_bias);
+  for (int u = 0; u < nb.Ls + nb.Hs; u += 4) {
+    const int4 x = nbr_chunk(nb, i, u);
+    for (int q = 0; q < 4; ++q) {
+      const int32_t v = int4_at(x, q);
+      if ((uint32_t)(v - own0) < own_n && v != (int32_t)i && sym_label(__ldg(hl + v), lin_bias) >= mine) return false;
+    }
+  }
+  return true;
 }
 
 // Entries of a row in step order, then padding (dummy column rows_pad, zero
@@ -730,50 +758,94 @@ __device__ __forceinline__ uint64_t sym_label(uint64_t lin, uint64_t lin_bias) {
 // in level N, N - 2, ... and have no black neighbour.  Of two neighbours in
 // those levels the one with the smaller label turns red (both when the labels
 // agree), so k and -k keep one colour and what stays black is independent.
-// The level of a neighbour follows from its index (rows are ordered by level):
-// no extra gather, and the labels are read only for such pairs.
-__global__ void k_fill_slices(NbrView nb, int64_t size, int64_t rows_pad, int s_a, int j0,
-                              const int32_t* __restrict__ woff, int colbits, const int64_t* __restrict__ norm,
-                              const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64, uint32_t* ent,
-                              double2* ecoef, bool real, const uint64_t* __restrict__ hl, uint64_t lin_bias,
-                              int64_t zero_idx, LevelStarts lv, uint32_t* cmask) {
-  double* ecoef_re = reinterpret_cast<double*>(ecoef);   // real coefficients: one double per entry
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows_pad) return;
-  const int64_t s = i / kSlice;
-  const int lane = (int)(i % kSlice);
+// A step changes the level by at most one, so such a neighbour lies in the
+// row's own level: one range check per entry, and the labels are read only for
+// pairs that pass it.
+//
+// One warp per slice: it stages neighbour words of its 32 rows in shared memory
+// (coalesced 16-byte loads), every lane turns its row's words into a bit mask,
+// and the entries are formed column by column - the next set bit of every row
+// - so that a column costs the FP64 pipe (a conversion and a product per entry,
+// 16 clocks of the SM per warp instruction) once, not once per step that some
+// row of the slice has: on the last level four columns instead of up to s_a.
+// k_fill_dense serves rows of at most 64 words (s_a <= 57), one mask per row;
+// k_fill_slices any row, 64 words at a time.  d = 100 (1.15 M rows of 44 words,
+// 7.6 M entries): 76 and 146 us; a thread per row that walked its words in step
+// order took 125 us.
+constexpr int kFillWarps = 4, kFillWords = 64;
+
+__global__ void __launch_bounds__(32 * kFillWarps) k_fill_slices(
+    NbrView nb, int64_t size, int64_t rows_pad, int j0, const int32_t* __restrict__ woff, int colbits,
+    const int64_t* __restrict__ norm, const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64,
+    uint32_t* __restrict__ ent, double2* __restrict__ ecoef, bool real, const uint64_t* __restrict__ hl,
+    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask) {
+  constexpr int kStride = kFillWords / 4 + 1;   // 16-byte words of a staged row (odd: no bank conflicts)
+  __shared__ int4 s_words[kFillWarps][32 * kStride];
+  double* ecoef_re = reinterpret_cast<double*>(ecoef);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t s = (int64_t)blockIdx.x * kFillWarps + warp, row0 = s * kSlice;
+  if (row0 >= rows_pad) return;   // whole warps
+  const int rows = (int)(size - row0 < kSlice ? size - row0 : kSlice);   // at least one
+  int4* w4 = s_words[warp];
+  const int32_t* mine = reinterpret_cast<const int32_t*>(w4 + lane * kStride);
+  const int64_t i = row0 + lane;
+  int32_t own0 = 0;
+  uint32_t own_n = 0;   // the row's level when it is a black one
+  if (lv.n > 0 && i < size && i != zero_idx) black_level(lv, (int32_t)i, (int32_t)size, &own0, &own_n);
+  bool near = false;    // some neighbour lies in that level
   const int64_t base = (int64_t)woff[s] * kSlice + lane;
   const int w = woff[s + 1] - woff[s];
-  int t = 0;
-  bool blk = lv.n > 0 && (i >= size || (i != zero_idx && black_level(lv, (int32_t)i)));
-  if (i < size) {
-    const int64_t nk = norm[i];
-    for (int ub = 0; ub < nb.Ls + nb.Hs; ub += kNbrBatch) {
-      int4 x[kNbrBatch / 4];
+  const int64_t nk = i < size ? norm[i] : 0;
+  const int U = nb.Ls + nb.Hs;
+  int t = 0;            // entries of the row so far
+  for (int u0 = 0; u0 < U; u0 += kFillWords) {
+    const int n4 = min(kFillWords, U - u0) / 4;
+    __syncwarp();
+    for (int r = lane / n4, c = lane % n4, x = lane; x < rows * n4; x += 32) {
+      w4[r * kStride + c] = nbr_chunk(nb, row0 + r, u0 + 4 * c);
+      for (c += 32; c >= n4; c -= n4) ++r;
+    }
+    __syncwarp();
+    uint64_t mask = 0;   // bit u: word u0 + u names a neighbour
+    if (lane < rows) {
+      for (int c = 0; c < n4; ++c) {
+        const int4 x = w4[lane * kStride + c];
 #pragma unroll
-      for (int q = 0; q < kNbrBatch / 4; ++q)
-        x[q] = ub + 4 * q < nb.Ls + nb.Hs ? nbr_chunk(nb, i, ub + 4 * q) : make_int4(-1, -1, -1, -1);
-      int32_t v[kNbrBatch];
-      int64_t nv[kNbrBatch];
+        for (int q = 0; q < 4; ++q) {
+          const int32_t v = int4_at(x, q);
+          mask |= (uint64_t)(v >= 0) << (4 * c + q);
+          near |= ((uint32_t)(v - own0) < own_n) & (v != (int32_t)i);
+        }
+      }
+    }
+    while (__any_sync(0xffffffffu, mask != 0)) {
+      int32_t v[4];
+      int j[4];
+      int64_t nv[4], pj[4];
 #pragma unroll
-      for (int q = 0; q < kNbrBatch; ++q) v[q] = int4_at(x[q / 4], q % 4);
+      for (int q = 0; q < 4; ++q) {
+        const int u = __ffsll((long long)mask) - 1;   // -1: the row's bits are used up
+        mask &= mask - 1;
+        v[q] = u < 0 ? -1 : mine[u];
+        j[q] = u < 0 ? 0 : nbr_step(nb, u0 + u);
+        nv[q] = v[q] >= 0 ? __ldg(norm + v[q]) : 0;
+        pj[q] = __ldg(pnorm + j[q]);
+      }
 #pragma unroll
-      for (int q = 0; q < kNbrBatch; ++q) nv[q] = v[q] >= 0 ? __ldg(norm + v[q]) : 0;
-#pragma unroll
-      for (int q = 0; q < kNbrBatch; ++q) {
+      for (int q = 0; q < 4; ++q) {
         if (v[q] < 0) continue;
-        const int j = nbr_step(nb, ub + q);
         const int64_t e = base + (int64_t)t++ * kSlice;
-        ent[e] = (uint32_t)v[q] | ((uint32_t)j << colbits);
-        const double sc = (double)(nk + nv[q] - pnorm[j]);
-        if (real) ecoef_re[e] = sc * ca64[j].x;
-        else ecoef[e] = make_double2(sc * ca64[j].x, sc * ca64[j].y);
-        if (blk && v[q] != i && black_level(lv, v[q]))
-          blk = sym_label(__ldg(hl + v[q]), lin_bias) < sym_label(__ldg(hl + i), lin_bias);
+        ent[e] = (uint32_t)v[q] | ((uint32_t)j[q] << colbits);
+        const double sc = (double)(nk + nv[q] - pj[q]);
+        const double2 c = __ldg(ca64 + j[q]);
+        if (real) ecoef_re[e] = sc * c.x;
+        else ecoef[e] = make_double2(sc * c.x, sc * c.y);
       }
     }
   }
-  if (lv.n > 0) {   // rows_pad is a whole number of warps
+  bool blk = i >= size || own_n > 0;
+  if (near) blk = black_wins(nb, i, own0, own_n, hl, lin_bias);
+  if (lv.n > 0) {
     const uint32_t m = __ballot_sync(0xffffffffu, blk);
     if (lane == 0) cmask[s] = m;
   }
@@ -782,6 +854,89 @@ __global__ void k_fill_slices(NbrView nb, int64_t size, int64_t rows_pad, int s_
     ent[base + (int64_t)t * kSlice] = pad;
     if (real) ecoef_re[base + (int64_t)t * kSlice] = 0.0;
     else ecoef[base + (int64_t)t * kSlice] = make_double2(0.0, 0.0);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kFillWarps) k_fill_dense(
+    NbrView nb, int64_t size, int64_t rows_pad, int s_a, int j0, const int32_t* __restrict__ woff, int colbits,
+    const int64_t* __restrict__ norm, const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64,
+    uint32_t* __restrict__ ent, double2* __restrict__ ecoef, bool real, const uint64_t* __restrict__ hl,
+    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask) {
+  extern __shared__ int4 sm_words[];   // per warp: 32 rows of Ls lo words, then 32 rows of Hs hi words
+  __shared__ double2 s_ca[kFillWords];
+  __shared__ int64_t s_pn[kFillWords];
+  double* ecoef_re = reinterpret_cast<double*>(ecoef);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int j = threadIdx.x; j < s_a; j += blockDim.x) {
+    s_ca[j] = ca64[j];
+    s_pn[j] = pnorm[j];
+  }
+  const int U = nb.Ls + nb.Hs;
+  int4* w4 = sm_words + warp * 8 * U;
+  const int64_t s = (int64_t)blockIdx.x * kFillWarps + warp;
+  const bool live = s * kSlice < rows_pad;
+  const int64_t row0 = s * kSlice;
+  const int rows = live ? (int)(size - row0 < kSlice ? size - row0 : kSlice) : 0;
+  const int4* lo4 = reinterpret_cast<const int4*>(nb.lo + row0 * nb.Ls);
+  const int4* hi4 = reinterpret_cast<const int4*>(nb.hi + row0 * nb.Hs);
+  const int nl = rows * nb.Ls / 4, nh = rows * nb.Hs / 4;
+  for (int x = lane; x < nl; x += 32) w4[x] = __ldg(lo4 + x);
+  int4* h4 = w4 + 8 * nb.Ls;
+  for (int x = lane; x < nh; x += 32) h4[x] = __ldg(hi4 + x);
+  __syncthreads();
+  if (!live) return;
+  const int64_t i = row0 + lane;
+  int32_t own0 = 0;
+  uint32_t own_n = 0;   // the row's level when it is a black one
+  if (lv.n > 0 && i < size && i != zero_idx) black_level(lv, (int32_t)i, (int32_t)size, &own0, &own_n);
+  bool near = false;    // some neighbour lies in that level
+  uint64_t mask = 0;    // bit u: word u names a neighbour
+  if (i < size) {
+    for (int u = 0; u < U; u += 4) {
+      const int4 x = u < nb.Ls ? w4[(lane * nb.Ls + u) >> 2] : h4[(lane * nb.Hs + u - nb.Ls) >> 2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int32_t v = int4_at(x, q);
+        mask |= (uint64_t)(v >= 0) << (u + q);
+        near |= ((uint32_t)(v - own0) < own_n) & (v != (int32_t)i);
+      }
+    }
+  }
+  bool blk = i >= size || own_n > 0;
+  if (near) blk = black_wins(nb, i, own0, own_n, hl, lin_bias);
+  if (lv.n > 0) {
+    const uint32_t m = __ballot_sync(0xffffffffu, blk);
+    if (lane == 0) cmask[s] = m;
+  }
+  const int32_t* lw = reinterpret_cast<const int32_t*>(w4) + lane * nb.Ls;
+  const int32_t* hw = reinterpret_cast<const int32_t*>(h4) + lane * nb.Hs;
+  const int64_t base = (int64_t)woff[s] * kSlice + lane;
+  const int w = woff[s + 1] - woff[s];
+  const int64_t nk = i < size ? norm[i] : 0;
+  const uint32_t pad = (uint32_t)rows_pad | ((uint32_t)j0 << colbits);
+  for (int t = 0; t < w; t += 4) {
+    int32_t v[4];
+    int j[4];
+    int64_t nv[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int u = __ffsll((long long)mask) - 1;   // -1: the row's entries are used up
+      mask &= mask - 1;
+      v[q] = u < 0 ? -1 : (u < nb.Ls ? lw[u] : hw[u - nb.Ls]);
+      j[q] = u < 0 ? j0 : (u < nb.Ls ? u : u - nb.Ls + nb.L);
+      nv[q] = v[q] >= 0 ? __ldg(norm + v[q]) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (t + q >= w) break;   // warp-uniform
+      const int64_t e = base + (int64_t)(t + q) * kSlice;
+      const bool ok = v[q] >= 0;
+      ent[e] = ok ? (uint32_t)v[q] | ((uint32_t)j[q] << colbits) : pad;
+      const double sc = ok ? (double)(nk + nv[q] - s_pn[j[q]]) : 0.0;
+      const double2 c = s_ca[j[q]];
+      if (real) ecoef_re[e] = sc * c.x;
+      else ecoef[e] = make_double2(sc * c.x, sc * c.y);
+    }
   }
 }
 
@@ -1483,11 +1638,17 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   } else {
     {
       ProfScope prof_("k_fill_slices", st);
-      k_fill_slices<<<nblk(S->rows_pad), 256, 0, st>>>(nb, S->size, S->rows_pad, s_a, S->j0,
-                                                       S->slice_off.get(), colbits_of(S->jbits), S->norm.get(),
-                                                       S->pnorm.get(), S->ca64.get(), S->ent.get(), S->ecoef64.get(),
-                                                       S->a_real, S->hl.get(), P.lin_bias, S->zero_idx, lv,
-                                                       S->cmask.get());
+      const unsigned fb = (unsigned)((S->n_slices + kFillWarps - 1) / kFillWarps);
+      if (nb.Ls + nb.Hs <= kFillWords)
+        k_fill_dense<<<fb, 32 * kFillWarps, (size_t)kFillWarps * 8 * (nb.Ls + nb.Hs) * sizeof(int4), st>>>(
+            nb, S->size, S->rows_pad, s_a, S->j0, S->slice_off.get(), colbits_of(S->jbits), S->norm.get(),
+            S->pnorm.get(), S->ca64.get(), S->ent.get(), S->ecoef64.get(), S->a_real, S->hl.get(), P.lin_bias,
+            S->zero_idx, lv, S->cmask.get());
+      else
+        k_fill_slices<<<fb, 32 * kFillWarps, 0, st>>>(
+            nb, S->size, S->rows_pad, S->j0, S->slice_off.get(), colbits_of(S->jbits), S->norm.get(), S->pnorm.get(),
+            S->ca64.get(), S->ent.get(), S->ecoef64.get(), S->a_real, S->hl.get(), P.lin_bias, S->zero_idx, lv,
+            S->cmask.get());
     }
   }
   SS_LAUNCH_CHECK();
