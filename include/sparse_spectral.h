@@ -194,8 +194,8 @@ ss_status sft_recover_samples(const ss_lattice* lat, const void* samples, ss_pre
 /* lattice_sample followed by sft_recover_samples (library-owned sample and
  * FFT buffers).  In FP64 on a 7-smooth M up to 2^22 both transforms (the
  * inverse one that samples g and the forward one that recovers it) run in the
- * library's double-float FFT instead of cuFFT.  That FFT rounds at about
- * 2^-46 relative.  The thresholding and output are as in sft_recover_samples.
+ * library's fixed-point FFT instead of cuFFT.  Its rounding is about 2^-56 of
+ * sum |coef| in every bin.  The thresholding and output are as in sft_recover_samples.
  * Synchronises `stream`. */
 ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_precision prec, const int32_t* cand,
                       int64_t n_cand, int64_t s_max, double tau, int32_t* freq_out, double* val_out,
@@ -213,7 +213,9 @@ ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_precision prec
  * [s_max][d], val_out device FP64 complex [s_max], the count in *n_out; more
  * than s_max terms is SS_ERR_INVALID; a k that does not map back to its bin
  * (k.z mod M != b: the lattice is not reconstructing for the support) is
- * SS_ERR_NOT_RECONSTRUCTING.  Costs d + 1 samplings and FFTs of length M.
+ * SS_ERR_NOT_RECONSTRUCTING.  Costs d + 1 samplings and FFTs of length M (in
+ * FP64 where sft_recover takes the fixed-point FFT: one complex transform each
+ * way for two of them).
  * Synchronises `stream`. */
 ss_status sft_identify(const ss_lattice* lat, const ss_trig* g, ss_precision prec, int32_t P, int64_t s_max,
                        double tau, int32_t* freq_out, double* val_out, int64_t* n_out, void* stream);
@@ -483,7 +485,7 @@ typedef struct {
  * S^N[a_hat](supp f_hat) (stamp_build), f_hat scattered onto S and the solve
  * of L_{N,s} u = f_hat (solve with tol, max_iter, solve_prec).  a and f
  * share one complex transform in two cases: FP64 on a 7-smooth M up to 2^22,
- * where sft_recover takes the double-float FFT and one transform runs each
+ * where sft_recover takes the fixed-point FFT and one transform runs each
  * way; and FP32 on an M that is not 7-smooth, where cuFFT takes Bluestein's
  * method and one forward C2C carries s_a / s_a' + i s_f / s_f'.  The scales
  * s_a', s_f' (and their FP64 counterparts) are powers of two near the two

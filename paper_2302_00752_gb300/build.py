@@ -17,7 +17,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsparse_spectral.so")
 PEAKS_LIB = os.path.join(HERE, "libss_peaks.so")   # rate microbenchmarks (benchmark only)
 SOURCES = ["api.cu", "scan.cu", "stamp.cu", "apply.cu", "lattice.cu", "sft.cu", "solve.cu", "batch.cu", "proxy.cu",
-           "pipeline.cu", "fft_df.cu", "fft_pruned.cu"]
+           "pipeline.cu", "fft_fx.cu", "fft_pruned.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,6 +1,6 @@
 // Complex double-float values and the small DFT kernels shared by the
-// double-float transforms (fft_df.cu: full length-M transform; fft_pruned.cu:
-// sparse-input evaluation and pruned-output transform).  A value is
+// double-float transforms (fft_pruned.cu: sparse-input evaluation and
+// pruned-output transform).  A value is
 // (re, im) with each part an unevaluated float pair (df.cuh).
 #pragma once
 

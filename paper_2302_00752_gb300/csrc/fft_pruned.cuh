@@ -1,6 +1,6 @@
 // Pruned DFTs of a 7-smooth length M for the coefficient recovery on long
 // lattices (FP64: double-float arithmetic, beyond the full transform of
-// fft_df.cu; FP32: FP32 arithmetic)
+// fft_fx.cu; FP32: FP32 arithmetic)
 // (Section "Previous results on SFTs": one length-M 1D FFT of the lattice
 // samples; only the bins k.z mod M of the candidate set are read).
 //
@@ -19,7 +19,7 @@
 // w^r = T1[r >> b] T0[r & (2^b - 1)].
 #pragma once
 
-#include "fft_df.cuh"
+#include "fft_fx.cuh"
 #include "ss_internal.cuh"
 
 namespace ss {

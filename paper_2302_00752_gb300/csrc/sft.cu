@@ -26,7 +26,7 @@
 #include <mutex>
 
 #include "df.cuh"
-#include "fft_df.cuh"
+#include "fft_fx.cuh"
 #include "fft_pruned.cuh"
 #include "lattice.cuh"
 
@@ -341,7 +341,8 @@ __global__ void k_merge_sum(const int32_t* __restrict__ sgn, const double2* __re
 // One warp per term.
 __global__ void k_compact_terms(const int32_t* __restrict__ freq, int64_t n, LatticeDev L,
                                 const int32_t* __restrict__ flag, const int32_t* __restrict__ pos,
-                                const double2* __restrict__ merged, int64_t* q, int64_t* step, double2* coef_out) {
+                                const double2* __restrict__ merged, int64_t* q, int64_t* step, double2* coef_out,
+                                int32_t* lead) {
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (t >= n || !flag[t]) return;   // warp-uniform
   const int64_t k = pos[t];
@@ -351,6 +352,7 @@ __global__ void k_compact_terms(const int32_t* __restrict__ freq, int64_t n, Lat
   q[k] = r;
   step[k] = (int64_t)(((uint64_t)r * (uint64_t)kSampThreads) % (uint64_t)L.M);
   coef_out[k] = merged[t];
+  if (lead) lead[k] = (int32_t)t;
 }
 
 
@@ -486,11 +488,12 @@ struct SftPlan {
   DevBuf<float2> t3[3];                                    // FP32 three-level tables
   int64_t n2 = 0;
   bool df = false;                                         // full table in double-float form
-  // double-float complex FFT (FP64 recovery of two real sums at once)
-  bool has_dff = false;
-  DfFftPlan dff;
-  DevBuf<float4> dfz, dftmp;
-  DevBuf<double> dfscale;   // the two sums' scales of the last round trip
+  // fixed-point complex FFT (FP64 recovery of two real sums at once)
+  bool has_fx = false;
+  FxFftPlan fx;
+  DevBuf<longlong2> fxz, fxtmp;
+  DevBuf<int4> fxtab;
+  DevBuf<double> fxscale;   // the two sums' scales and floors of the last round trip
   // pruned transforms (on a 7-smooth M above the full table's limit;
   // double-float arithmetic in FP64, FP32 in FP32): two-level twiddle table,
   // the complex sample vector s_a / sigma_a + i s_f / sigma_f and the two
@@ -582,11 +585,13 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
       k_twiddles_df<<<nblk(M), 256, 0, st>>>(M, reinterpret_cast<float4*>(p->full.get()));
     SS_LAUNCH_CHECK();
     p->df = !native_fp64_sampling();
-    if (p->df && df_fft_plan(M, &p->dff)) {
-      SS_TRY(p->dfz.alloc(M, st));
-      SS_TRY(p->dftmp.alloc(M, st));
-      SS_TRY(p->dfscale.alloc(2, st));
-      p->has_dff = true;
+    if (p->df && fx_fft_plan(M, &p->fx)) {
+      SS_TRY(p->fxz.alloc(M, st));
+      SS_TRY(p->fxtmp.alloc(M, st));
+      SS_TRY(p->fxtab.alloc(M + p->fx.L1 + p->fx.L2, st));
+      SS_TRY(p->fxscale.alloc(4, st));
+      SS_TRY(fx_fft_table(p->fx, p->fxtab.get(), st));
+      p->has_fx = true;
     }
   }
   if (M > kFullTableMax && !(prec == SS_FP64 && native_fp64_sampling()) && pruned_supported(M)) {
@@ -602,7 +607,7 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
   // the plan is cached across calls and streams
   SS_CUDA(cudaStreamSynchronize(st));
   p->samples.settle(); p->spectrum.settle(); p->lo.settle(); p->hi.settle(); p->full.settle();
-  p->dfz.settle(); p->dftmp.settle(); p->dfscale.settle();
+  p->fxz.settle(); p->fxtmp.settle(); p->fxtab.settle(); p->fxscale.settle();
   p->prt.t0.settle(); p->prt.t1.settle(); p->prz.settle(); p->prscale.settle();
   for (auto& t : p->t3) t.settle();
   g_plans.push_front(p);
@@ -704,8 +709,15 @@ __global__ void k_bin_terms(const int64_t* __restrict__ q, const double2* __rest
 // scale[w] = the power of two at or below sum_t |c_t| of sum w (1 if zero):
 // the two sums share one transform at comparable magnitudes, so each keeps its
 // own relative rounding error; powers of two scale exactly.
+// UNITS (fixed-point spectra, scale[4]): scale[2 + w] is what a bin of sum w
+// that rounds to zero units is read as: a quarter of a unit, so that a
+// threshold of zero keeps every candidate of a nonzero sum, 0 for a sum that
+// is zero, NaN where a coefficient of either sum is not finite or a scale has
+// no reciprocal (integers would hide it).
 constexpr int kScaleThreads = 512;
+template <bool UNITS = false>
 __device__ void pair_scale(const double2* const c[2], const int64_t n[2], double* scale) {
+  double total[2];
   __shared__ double s_part[kScaleThreads];
   for (int w = 0; w < 2; ++w) {
     double acc = 0.0;
@@ -716,19 +728,24 @@ __device__ void pair_scale(const double2* const c[2], const int64_t n[2], double
       if (threadIdx.x < o) s_part[threadIdx.x] += s_part[threadIdx.x + o];
       __syncthreads();
     }
+    total[w] = s_part[0];
     if (threadIdx.x == 0) scale[w] = s_part[0] > 0.0 ? ldexp(1.0, ilogb(s_part[0])) : 1.0;
     __syncthreads();
   }
+  if (!UNITS || threadIdx.x) return;
+  const double bad = 0.0 * (total[0] + 1.0 / scale[0]) + 0.0 * (total[1] + 1.0 / scale[1]);
+  for (int w = 0; w < 2; ++w) scale[2 + w] = bad + (total[w] > 0.0 ? 0.25 : 0.0);
 }
 
 // term counts on the device (merged sums)
+template <bool UNITS>
 __global__ void __launch_bounds__(kScaleThreads) k_pair_scale(const double2* __restrict__ ca,
                                                               const int64_t* __restrict__ na_dev,
                                                               const double2* __restrict__ cf,
                                                               const int64_t* __restrict__ nf_dev, double* scale) {
   const double2* c[2] = {ca, cf};
   const int64_t n[2] = {*na_dev, *nf_dev};
-  pair_scale(c, n, scale);
+  pair_scale<UNITS>(c, n, scale);
 }
 
 // term counts from the host (the sums as given)
@@ -778,7 +795,7 @@ __global__ void k_extract_pair32(const int32_t* __restrict__ cand, int64_t n, La
 __global__ void k_bin_pair(const int64_t* __restrict__ qa, const double2* __restrict__ ca,
                            const int64_t* __restrict__ na_dev, const int64_t* __restrict__ qf,
                            const double2* __restrict__ cf, const int64_t* __restrict__ nf_dev,
-                           const double* __restrict__ scale, int64_t M, float4* __restrict__ Z) {
+                           const double* __restrict__ scale, int64_t M, longlong2* __restrict__ Z) {
   const int64_t na = *na_dev, n = na + *nf_dev;
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -810,36 +827,39 @@ __global__ void k_bin_pair(const int64_t* __restrict__ qa, const double2* __rest
   if (lane) return;
   const double ia = 1.0 / scale[0], jf = 1.0 / scale[1];   // exact: powers of two
   are *= ia; aim *= ia; fre *= jf; fim *= jf;
+  const double un = ldexp(1.0, kFxFrac);
   if (b == 0 || 2 * b == M) {
-    const DF zr = df_split(are), zi = df_split(fre);
-    Z[b] = make_float4(zr.hi, zr.lo, zi.hi, zi.lo);
+    Z[b] = make_longlong2(__double2ll_rn(un * are), __double2ll_rn(un * fre));
     return;
   }
   are *= 0.5; aim *= 0.5; fre *= 0.5; fim *= 0.5;
-  DF x = df_split(are - fim), y = df_split(aim + fre);
-  Z[b] = make_float4(x.hi, x.lo, y.hi, y.lo);
-  x = df_split(are + fim);
-  y = df_split(fre - aim);
-  Z[M - b] = make_float4(x.hi, x.lo, y.hi, y.lo);
+  Z[b] = make_longlong2(__double2ll_rn(un * (are - fim)), __double2ll_rn(un * (aim + fre)));
+  Z[M - b] = make_longlong2(__double2ll_rn(un * (are + fim)), __double2ll_rn(un * (fre - aim)));
 }
 
 // Recovery from the forward transform Zh of s_a + i s_f: with x = Zh[b] and
 // y = Zh[M - b], the bin of the real sum a is (x + conj(y)) / 2 and that of f
 // is (x - conj(y)) / (2 i), each scaled by 1 / M.
+// floor: pair_scale's scale[2 + WHICH].
 template <int WHICH>
-__global__ void k_extract_pair(const int32_t* __restrict__ cand, int64_t n, LatticeDev L, const float4* __restrict__ Zh,
-                               const double* __restrict__ scale, double2* val, double* mag,
-                               unsigned long long* maxbits) {
+__device__ __forceinline__ double2 pair_bin(const longlong2 x, const longlong2 y, double floor) {
+  const int64_t re = WHICH == 0 ? x.x + y.x : x.y + y.y, im = WHICH == 0 ? x.y - y.y : y.x - x.x;
+  const double f = (re | im) == 0 ? floor : 0.0 * floor;
+  return make_double2((double)re + f, (double)im);
+}
+
+// unit: value of one unit of Zh (2^(shift - kFxFrac)).
+template <int WHICH>
+__global__ void k_extract_pair(const int32_t* __restrict__ cand, int64_t n, LatticeDev L,
+                               const longlong2* __restrict__ Zh, double unit, const double* __restrict__ scale,
+                               double2* val, double* mag, unsigned long long* maxbits) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t b = residue_of(cand + i * L.d, L.d, L);
   const int64_t nb = (L.M - b) % L.M;
-  const float4 xs = Zh[b], ys = Zh[nb];
-  const double xr = (double)xs.x + (double)xs.y, xi = (double)xs.z + (double)xs.w;
-  const double yr = (double)ys.x + (double)ys.y, yi = (double)ys.z + (double)ys.w;
-  const double sc = 0.5 / (double)L.M * scale[WHICH];
-  const double2 v = WHICH == 0 ? make_double2((xr + yr) * sc, (xi - yi) * sc)
-                               : make_double2((xi + yi) * sc, (yr - xr) * sc);
+  const double sc = 0.5 / (double)L.M * unit * scale[WHICH];
+  const double2 z = pair_bin<WHICH>(Zh[b], Zh[nb], scale[2 + WHICH]);
+  const double2 v = make_double2(z.x * sc, z.y * sc);
   val[i] = v;
   const double m = hypot(v.x, v.y);
   mag[i] = m;
@@ -864,11 +884,12 @@ ss_status launch_sample(const SftPlan& P, unsigned grid, size_t sm, const int64_
 struct Terms {
   DevBuf<int64_t> q, step, total;
   DevBuf<double2> coef;
+  DevBuf<int32_t> lead;   // index of the term each merged one is written in the orientation of (on request)
 };
 
 // Merge +-p terms (exact rewrite of the real sum) and compact them; no host
 // synchronisation (the merged count stays on the device).
-ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream_t st) {
+ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream_t st, bool want_lead = false) {
   ProfScope prof_("prep_terms", st);
   const int64_t n = g->n_terms;
   SS_TRY(T->total.alloc_tmp(1, st));
@@ -895,8 +916,9 @@ ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream
                                             flag.get(), merged.get(), imag.get());
   SS_LAUNCH_CHECK();
   SS_TRY(exclusive_scan_i32(flag.get(), pos.get(), n, T->total.get(), st));
+  if (want_lead) SS_TRY(T->lead.alloc_tmp(n, st));
   k_compact_terms<<<nblk(n * 32), 256, 0, st>>>(g->freq, n, L, flag.get(), pos.get(), merged.get(), T->q.get(),
-                                                T->step.get(), T->coef.get());
+                                                T->step.get(), T->coef.get(), want_lead ? T->lead.get() : nullptr);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
@@ -1131,31 +1153,36 @@ ss_status sample_into(const SftPlan& P, const LatticeDev& L, const ss_trig* g, v
   return launch_sample<float, 1>(P, grid, terms_sm, q.get(), step.get(), coef.get(), total.get(), out, st);
 }
 
-// Bins, threshold and compaction in candidate order; the reconstructing and
-// symmetry checks run on the device beside them and are read back with the
-// kept count in one synchronisation at the end.
-// FP64 plans with the double-float transform: the sums a and f (f may be
+// Value of one unit of the spectrum that fx_round_trip leaves.
+double fx_unit(const SftPlan& P) { return std::ldexp(1.0, P.fx.shift - kFxFrac); }
+
+// The samples of the spectrum in P.fxz, and their spectrum again.
+ss_status fx_round_trip(const SftPlan& P, cudaStream_t st) {
+  longlong2* Z = P.fxz.get();
+  SS_TRY(fx_fft(P.fx, P.fxtab.get(), Z, P.fxtmp.get(), Z, +1, st));
+  return fx_fft(P.fx, P.fxtab.get(), Z, P.fxtmp.get(), Z, -1, st);
+}
+
+// FP64 plans with the fixed-point transform: the sums a and f (f may be
 // null) are sampled by one inverse transform of Z = S_a + i S_f and the
-// samples s_a + i s_f transformed forward again; on return P.dfz holds that
+// samples s_a + i s_f transformed forward again; on return P.fxz holds that
 // spectrum (read by k_extract_pair).
-ss_status dff_round_trip(const SftPlan& P, const LatticeDev& L, const ss_trig* a, const ss_trig* f, cudaStream_t st) {
+ss_status fx_recover_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* a, const ss_trig* f, cudaStream_t st) {
   const ss_trig none{L.d, 0, nullptr, nullptr};
   if (!f) f = &none;
   Terms ta, tf;
   SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
-  float4* Z = P.dfz.get();
-  const float4* tab = reinterpret_cast<const float4*>(P.full.get());
-  SS_CUDA(cudaMemsetAsync(Z, 0, P.M * sizeof(float4), st));
-  double* scale = P.dfscale.get();
-  k_pair_scale<<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
+  longlong2* Z = P.fxz.get();
+  SS_CUDA(cudaMemsetAsync(Z, 0, P.M * sizeof(longlong2), st));
+  double* scale = P.fxscale.get();
+  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
   SS_LAUNCH_CHECK();
   if (a->n_terms + f->n_terms > 0) {
     k_bin_pair<<<nblk((a->n_terms + f->n_terms) * 32), 256, 0, st>>>(ta.q.get(), ta.coef.get(), ta.total.get(), tf.q.get(),
                                                               tf.coef.get(), tf.total.get(), scale, P.M, Z);
     SS_LAUNCH_CHECK();
   }
-  SS_TRY(df_fft(P.dff, tab, Z, P.dftmp.get(), Z, +1, st));
-  return df_fft(P.dff, tab, Z, P.dftmp.get(), Z, -1, st);
+  return fx_round_trip(P, st);
 }
 
 // Pruned path (a 7-smooth M above the full table): the two sums a and f (f
@@ -1168,7 +1195,7 @@ ss_status pr_sample_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* a
   Terms ta, tf;
   SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
   double* scale = P.prscale.get();
-  k_pair_scale<<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
+  k_pair_scale<false><<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
   SS_LAUNCH_CHECK();
   return pruned_eval_pair(P.prt, ta.q.get(), ta.coef.get(), ta.total.get(), a->n_terms, tf.q.get(), tf.coef.get(),
                           tf.total.get(), f->n_terms, scale, P.prz.get(),
@@ -1278,13 +1305,16 @@ ss_status pr_transform(const SftPlan& P, const void* s, bool real, const int64_t
   return pruned_forward(P.prt, s, fmt, bins.get(), 2 * n_cand, X, st);
 }
 
-// zh non-null: the bins come from the double-float spectrum zh (real part
-// sum, as left by dff_round_trip) instead of a transform of samples.
+// Bins, threshold and compaction in candidate order; the reconstructing and
+// symmetry checks run on the device beside them and are read back with the
+// kept count in one synchronisation at the end.
+// zh non-null: the bins come from the fixed-point spectrum zh (real part
+// sum, as left by fx_recover_pair) instead of a transform of samples.
 // pr != 0: the pruned forward transform of P.prz (pr = 1: complex samples of
 // one sum, scale P.prscale) or of the real FP64 samples (pr = 2).
 ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* samples, const int32_t* cand, int64_t n_cand,
                        int64_t s_max, double tau, int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st,
-                       const float4* zh = nullptr, int pr = 0) {
+                       const longlong2* zh = nullptr, int pr = 0) {
   DevBuf<int64_t> res, total;
   DevBuf<unsigned long long> table, maxbits;
   DevBuf<int32_t> flags, flag, pos;
@@ -1323,8 +1353,8 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
     k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), pr == 1 ? P.prscale.get() : nullptr,
                                                   val.get(), mag.get(), maxbits.get());
   else if (zh)
-    k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, P.dfscale.get(), val.get(), mag.get(),
-                                                    maxbits.get());
+    k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, fx_unit(P), P.fxscale.get(), val.get(),
+                                                    mag.get(), maxbits.get());
   else if (P.prec == SS_FP64)
     k_extract<double2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const double2*>(P.spectrum.get()),
                                                      val.get(), mag.get(), maxbits.get());
@@ -1397,19 +1427,64 @@ __global__ void k_rotate_coef(const int32_t* __restrict__ freq, const double2* _
   out[t] = make_double2(c.x * cs - c.y * sn, c.x * sn + c.y * cs);
 }
 
+// k_i from arg(X_i / X_0) = arg(v conj(a))
+__device__ __forceinline__ int32_t coord_of(const double2 v, const double2 a, int P) {
+  const double re = v.x * a.x + v.y * a.y, im = v.y * a.x - v.x * a.y;
+  long long k = llrint((double)P * atan2(im, re) / (2.0 * 3.141592653589793)) % P;
+  if (k < 0) k += P;
+  if (2 * k > P) k -= P;
+  return (int32_t)k;
+}
+
 template <typename T2>
 __global__ void k_identify_coord(const T2* __restrict__ spec, const int64_t* __restrict__ bins,
                                  const double2* __restrict__ x0, int64_t nb, int d, int i, int P, int32_t* kf) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nb) return;
   const T2 v = spec[bins[t]];
-  const double2 a = x0[t];
-  // arg(X_i / X_0) = arg(X_i conj(X_0))
-  const double re = (double)v.x * a.x + (double)v.y * a.y, im = (double)v.y * a.x - (double)v.x * a.y;
-  long long k = llrint((double)P * atan2(im, re) / (2.0 * 3.141592653589793)) % P;
-  if (k < 0) k += P;
-  if (2 * k > P) k -= P;
-  kf[t * d + i] = (int32_t)k;
+  kf[t * d + i] = coord_of(make_double2((double)v.x, (double)v.y), x0[t], P);
+}
+
+// The same from the transform Z of two rows s_i + i s_j (coordinates i and j;
+// below zero: that half is not wanted).  Only the argument counts, so the
+// units and the rows' common scale drop out.
+__global__ void k_identify_coord_pair(const longlong2* __restrict__ Z, int64_t M, const int64_t* __restrict__ bins,
+                                      const double2* __restrict__ x0, int64_t nb, int d, int i, int j, int P,
+                                      int32_t* kf) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nb) return;
+  const int64_t b = bins[t];
+  const longlong2 x = Z[b], y = Z[b ? M - b : 0];
+  if (i >= 0) kf[t * d + i] = coord_of(pair_bin<0>(x, y, 0.0), x0[t], P);
+  if (j >= 0) kf[t * d + j] = coord_of(pair_bin<1>(x, y, 0.0), x0[t], P);
+}
+
+// The half spectrum of the first row of Z, X_0[b] (unnormalised).
+__global__ void k_pair_spectrum(const longlong2* __restrict__ Z, int64_t M, int64_t nh, double unit,
+                                const double* __restrict__ scale, double2* __restrict__ spec) {
+  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= nh) return;
+  const double2 z = pair_bin<0>(Z[b], Z[b ? M - b : 0], scale[2]);
+  const double sc = 0.5 * unit * scale[0];
+  spec[b] = make_double2(z.x * sc, z.y * sc);
+}
+
+// Merged coefficients of the rows i0 and i1 (0: the lattice itself, i >= 1:
+// shifted by e_i / P, which turns the coefficient of p by exp(2 pi i p_i / P)).
+__global__ void k_rotate_pair(const int32_t* __restrict__ freq, const int32_t* __restrict__ lead,
+                              const double2* __restrict__ coef, const int64_t* __restrict__ n_dev, int d, int i0,
+                              int i1, int P, double2* __restrict__ out0, double2* __restrict__ out1) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= *n_dev) return;
+  const double2 c = coef[t];
+  const int32_t* p = freq + (int64_t)lead[t] * d;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = q ? i1 : i0;
+    double sn = 0.0, cs = 1.0;
+    if (i > 0) sincospi(2.0 * (double)p[i - 1] / (double)P, &sn, &cs);
+    (q ? out1 : out0)[t] = make_double2(c.x * cs - c.y * sn, c.x * sn + c.y * cs);
+  }
 }
 
 // valid[t]: the identified k reproduces its bin (k.z mod M == b); otherwise
@@ -1510,11 +1585,11 @@ ss_status exec_fft(const SftPlan& P, const void* samples, cudaStream_t st) {
   return SS_OK;
 }
 
-// Rows of the identification: row(i) leaves the samples of row i (0: the
-// lattice, i >= 1: the lattice shifted by e_i / P) in device memory and
-// returns them.
-template <typename T2, class Rows>
-ss_status identify_impl(const SftPlan& P, const LatticeDev& L, Rows row, int Pp, int64_t s_max, int64_t keep,
+// Identification from the rows' spectra (row 0: the lattice, row i >= 1: the
+// lattice shifted by e_i / P).  first() leaves row 0's half spectrum in
+// P.spectrum; coords(bins, x0, nb, kf) finds the d coordinates of every kept bin.
+template <typename T2, class First, class Coords>
+ss_status identify_impl(const SftPlan& P, const LatticeDev& L, First first, Coords coords, int64_t s_max, int64_t keep,
                         bool robust, double tau, int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st) {
   const int64_t nh = L.M / 2 + 1;
   const T2* spec = reinterpret_cast<const T2*>(P.spectrum.get());
@@ -1527,9 +1602,7 @@ ss_status identify_impl(const SftPlan& P, const LatticeDev& L, Rows row, int Pp,
   SS_TRY(pos.alloc(nh, st));
   SS_TRY(total.alloc(1, st));
   SS_TRY(err.alloc(1, st));
-  const void* r0 = nullptr;
-  SS_TRY(row(0, &r0));
-  SS_TRY(exec_fft(P, r0, st));
+  SS_TRY(first());
   SS_CUDA(cudaMemsetAsync(maxbits.get(), 0, sizeof(unsigned long long), st));
   SS_CUDA(cudaMemsetAsync(err.get(), 0, sizeof(int32_t), st));
   const unsigned gmax = (unsigned)std::min<int64_t>(nblk(nh), 4 * 152);
@@ -1576,13 +1649,7 @@ ss_status identify_impl(const SftPlan& P, const LatticeDev& L, Rows row, int Pp,
   SS_TRY(kf.alloc((size_t)nb * L.d, st));
   SS_TRY(valid.alloc(nb, st));
   SS_TRY(vpos.alloc(nb, st));
-  for (int i = 0; i < L.d; ++i) {
-    const void* ri = nullptr;
-    SS_TRY(row(i + 1, &ri));
-    SS_TRY(exec_fft(P, ri, st));
-    k_identify_coord<T2><<<nblk(nb), 256, 0, st>>>(spec, bins.get(), x0.get(), nb, L.d, i, Pp, kf.get());
-    SS_LAUNCH_CHECK();
-  }
+  SS_TRY(coords(bins.get(), x0.get(), nb, kf.get()));
   k_identify_check<<<nblk(nb), 256, 0, st>>>(kf.get(), bins.get(), nb, L, valid.get(), err.get());
   SS_LAUNCH_CHECK();
   SS_TRY(exclusive_scan_i32(valid.get(), vpos.get(), nb, total.get(), st));
@@ -1605,6 +1672,75 @@ ss_status identify_impl(const SftPlan& P, const LatticeDev& L, Rows row, int Pp,
   SS_CUDA(cudaStreamSynchronize(st));
   *n_out = n;
   return SS_OK;
+}
+
+// Row by row: row(i, &samples) leaves the samples of row i in device memory,
+// transformed by cuFFT.
+template <typename T2, class Rows>
+ss_status identify_rows(const SftPlan& P, const LatticeDev& L, Rows row, int Pp, int64_t s_max, int64_t keep,
+                        bool robust, double tau, int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st) {
+  auto first = [&]() -> ss_status {
+    const void* r0 = nullptr;
+    SS_TRY(row(0, &r0));
+    return exec_fft(P, r0, st);
+  };
+  auto coords = [&](const int64_t* bins, const double2* x0, int64_t nb, int32_t* kf) -> ss_status {
+    for (int i = 0; i < L.d; ++i) {
+      const void* ri = nullptr;
+      SS_TRY(row(i + 1, &ri));
+      SS_TRY(exec_fft(P, ri, st));
+      k_identify_coord<T2><<<nblk(nb), 256, 0, st>>>(reinterpret_cast<const T2*>(P.spectrum.get()), bins, x0, nb, L.d,
+                                                     i, Pp, kf);
+      SS_LAUNCH_CHECK();
+    }
+    return SS_OK;
+  };
+  return identify_impl<T2>(P, L, first, coords, s_max, keep, robust, tau, freq_out, val_out, n_out, st);
+}
+
+// FP64 plans with the fixed-point transform: the merged terms once for all
+// rows (a shift turns a merged coefficient like the coefficients it sums), and
+// two rows at a time as the real and imaginary part of one complex transform
+// each way.  d = 10, 840 terms, M = 10^6: 5.3 ms row by row through cuFFT's
+// FP64 transforms (205 us each way, 11 rows), 1.3 ms so.
+ss_status identify_pairs(const SftPlan& P, const LatticeDev& L, const ss_trig* g, int Pp, int64_t s_max, double tau,
+                         int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st) {
+  Terms T;
+  SS_TRY(prep_terms(L, g, &T, st, true));
+  DevBuf<double2> c0, c1;
+  SS_TRY(c0.alloc_tmp(g->n_terms, st));
+  SS_TRY(c1.alloc_tmp(g->n_terms, st));
+  double* scale = P.fxscale.get();
+  // every row has the same l1 norm: one scale for all
+  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(T.coef.get(), T.total.get(), T.coef.get(), T.total.get(), scale);
+  SS_LAUNCH_CHECK();
+  auto transform = [&](int i0, int i1) -> ss_status {   // i1 > d: the last row again, unused
+    k_rotate_pair<<<nblk(g->n_terms), 256, 0, st>>>(g->freq, T.lead.get(), T.coef.get(), T.total.get(), L.d, i0,
+                                                    std::min(i1, L.d), Pp, c0.get(), c1.get());
+    SS_CUDA(cudaMemsetAsync(P.fxz.get(), 0, P.M * sizeof(longlong2), st));
+    k_bin_pair<<<nblk(2 * g->n_terms * 32), 256, 0, st>>>(T.q.get(), c0.get(), T.total.get(), T.q.get(), c1.get(),
+                                                           T.total.get(), scale, P.M, P.fxz.get());
+    SS_LAUNCH_CHECK();
+    return fx_round_trip(P, st);
+  };
+  auto first = [&]() -> ss_status {
+    SS_TRY(transform(0, 1));
+    const int64_t nh = L.M / 2 + 1;
+    k_pair_spectrum<<<nblk(nh), 256, 0, st>>>(P.fxz.get(), L.M, nh, fx_unit(P), scale,
+                                              reinterpret_cast<double2*>(P.spectrum.get()));
+    SS_LAUNCH_CHECK();
+    return SS_OK;
+  };
+  auto coords = [&](const int64_t* bins, const double2* x0, int64_t nb, int32_t* kf) -> ss_status {
+    for (int i = 0; i <= L.d; i += 2) {   // rows i and i + 1 hold the coordinates i - 1 and i
+      if (i > 0) SS_TRY(transform(i, i + 1));
+      k_identify_coord_pair<<<nblk(nb), 256, 0, st>>>(P.fxz.get(), L.M, bins, x0, nb, L.d, i - 1, i < L.d ? i : -1, Pp,
+                                                      kf);
+      SS_LAUNCH_CHECK();
+    }
+    return SS_OK;
+  };
+  return identify_impl<double2>(P, L, first, coords, s_max, 0, false, tau, freq_out, val_out, n_out, st);
 }
 
 ss_status check_trig(const ss_trig* g, int d) {
@@ -1684,17 +1820,18 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
       SS_LAUNCH_CHECK();
     }
   }
-  if (P.has_dff) {
+  if (P.has_fx) {
     // FP64: both sums sampled by one inverse and recovered by one forward
-    // double-float transform of length M
-    SS_TRY(dff_round_trip(P, L, a, f, st));
-    const float4* Z = P.dfz.get();
+    // fixed-point transform of length M
+    SS_TRY(fx_recover_pair(P, L, a, f, st));
+    const longlong2* Z = P.fxz.get();
+    const double un = fx_unit(P);
     for (int k = 0; k < 2; ++k) {
       if (k == 0)
-        k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, P.dfscale.get(), val.get(), mag.get(),
+        k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, un, P.fxscale.get(), val.get(), mag.get(),
                                                         maxbits.get());
       else
-        k_extract_pair<1><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, P.dfscale.get(), val.get(), mag.get(),
+        k_extract_pair<1><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, un, P.fxscale.get(), val.get(), mag.get(),
                                                         maxbits.get() + 1);
       k_keep<<<nblk(n_cand), 256, 0, st>>>(mag.get(), n_cand, maxbits.get() + k, tau, flag.get());
       SS_LAUNCH_CHECK();
@@ -1704,7 +1841,7 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
       SS_LAUNCH_CHECK();
     }
   }
-  if (!P.has_dff && !P.has_pr && use_pair32(P)) {
+  if (!P.has_fx && !P.has_pr && use_pair32(P)) {
     SS_TRY(ensure_pair32(P, st));
     SS_TRY(sample_into(P, L, a, P.samples.get(), st));
     SS_TRY(sample_into(P, L, f, P.samples2.get(), st));
@@ -1734,7 +1871,7 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
       SS_LAUNCH_CHECK();
     }
   }
-  for (int k = 0; k < 2 && !P.has_dff && !P.has_pr && !use_pair32(P); ++k) {
+  for (int k = 0; k < 2 && !P.has_fx && !P.has_pr && !use_pair32(P); ++k) {
     // the plan's sample and spectrum buffers serve both sums in stream order
     SS_TRY(sample_into(P, L, g[k], P.samples.get(), st));
     if (P.prec == SS_FP64)
@@ -1814,9 +1951,9 @@ extern "C" ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_pre
   cudaStream_t st = as_stream(stream);
   std::shared_ptr<SftPlan> P;
   SS_TRY(get_plan(L.M, prec, st, &P));
-  if (P->has_dff) {
-    SS_TRY(dff_round_trip(*P, L, g, nullptr, st));
-    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, P->dfz.get());
+  if (P->has_fx) {
+    SS_TRY(fx_recover_pair(*P, L, g, nullptr, st));
+    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, P->fxz.get());
   }
   if (P->has_pr) {
     SS_TRY(pr_sample_pair(*P, L, g, nullptr, st));
@@ -1839,9 +1976,11 @@ extern "C" ss_status sft_identify(const ss_lattice* lat, const ss_trig* g, ss_pr
   cudaStream_t st = as_stream(stream);
   std::shared_ptr<SftPlan> Pl;
   SS_TRY(get_plan(L.M, prec, st, &Pl));
+  const SftPlan& PP = *Pl;
+  if (PP.has_fx && g->n_terms > 0)
+    return identify_pairs(PP, L, g, P, s_max, tau, freq_out, val_out, n_out, st);
   DevBuf<double2> rot;
   SS_TRY(rot.alloc(std::max<int64_t>(g->n_terms, 1), st));
-  const SftPlan& PP = *Pl;
   // row 0: g on the lattice; row i: the coefficients turned by exp(2 pi i p_i / P)
   auto rows = [&](int i, const void** out) -> ss_status {
     if (i == 0) {
@@ -1857,8 +1996,8 @@ extern "C" ss_status sft_identify(const ss_lattice* lat, const ss_trig* g, ss_pr
     return SS_OK;
   };
   if (prec == SS_FP64)
-    return identify_impl<double2>(PP, L, rows, P, s_max, 0, false, tau, freq_out, val_out, n_out, st);
-  return identify_impl<float2>(PP, L, rows, P, s_max, 0, false, tau, freq_out, val_out, n_out, st);
+    return identify_rows<double2>(PP, L, rows, P, s_max, 0, false, tau, freq_out, val_out, n_out, st);
+  return identify_rows<float2>(PP, L, rows, P, s_max, 0, false, tau, freq_out, val_out, n_out, st);
 }
 
 extern "C" ss_status sft_identify_samples(const ss_lattice* lat, int32_t P, const void* samples, ss_precision prec,
@@ -1884,6 +2023,6 @@ extern "C" ss_status sft_identify_samples(const ss_lattice* lat, int32_t P, cons
     return SS_OK;
   };
   if (prec == SS_FP64)
-    return identify_impl<double2>(*Pl, L, rows, P, s_max, keep, robust != 0, tau, freq_out, val_out, n_out, st);
-  return identify_impl<float2>(*Pl, L, rows, P, s_max, keep, robust != 0, tau, freq_out, val_out, n_out, st);
+    return identify_rows<double2>(*Pl, L, rows, P, s_max, keep, robust != 0, tau, freq_out, val_out, n_out, st);
+  return identify_rows<float2>(*Pl, L, rows, P, s_max, keep, robust != 0, tau, freq_out, val_out, n_out, st);
 }
