@@ -703,7 +703,7 @@ def next_prime_py(n):
 
 
 
-DF_OPS_PER_PAIR = 150   # ten double-float multiply-adds of 15 FP32 instructions per (term, point)
+DF_OPS_PER_PAIR = 18   # 36 FP32 instructions per evaluated (term, point); k and -k are evaluated as one
 
 
 def multiscale_section(B, gp, flush, reps=5):

@@ -341,7 +341,7 @@ ss_status proxy_residual(ss_stamp s, const double* u_prefix, int64_t n_u, const 
  * S = S^{N+1} and u solves on S^N, f^{s,N} = L[a_hat] u is exact (Proposition
  * LExpansion).  The estimate of ||f - f^{s,N}||_{L2} / ||f||_{L2} is
  * sqrt(sum r^2 / sum f^2).  Phases k.X mod 2^32 are exact integers; each
- * term is evaluated in double-float arithmetic (about 1e-13 of |coef| per
+ * term is evaluated in double-float arithmetic (about 2e-14 of |coef| per
  * term).  r_out, f_out: device FP64 [Q].  Deterministic; asynchronous on
  * `stream`; uses the stamp's operator scratch. */
 ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, const ss_trig* f, const uint32_t* X, int64_t Q,

@@ -2,153 +2,321 @@
 // testing overview"): r(x) = f(x) - f^{s,N}(x) at uniform random points of
 // T^d, with f^{s,N} = L[a_hat] u^{s,N} known through its coefficients on
 // S^{N+1} (Proposition LExpansion).  The work is a dense trigonometric sum of
-// |terms| x |points| exponentials.
+// |terms| x |points| cosines.
 //
 // Points lie on the grid (2^-32 Z)^d, so the phase k.x mod 1 of every term is
 // the exact integer (k.X mod 2^32) / 2^32, formed with wrapping 32-bit
-// multiply-adds.  exp(2 pi i ph / 2^32) is the product of three table entries
-// (bits 31..21, 20..10 and 9..0 of ph) held in shared memory as double-float
-// values, and every product and the running sum are double-float: the whole
-// inner loop stays on the FP32 pipe, which issues two orders of magnitude more
-// operations per clock than the FP64 pipe on this part.
+// multiply-adds.  A term is Re(c exp(2 pi i k.x)) = |c| cos(2 pi (k.x + phi)):
+// the argument phi of c joins the phase (32 bits as an integer, the rest as a
+// float), so that no complex product is left.  On a symmetric set the terms k
+// and -k are one, with c_k + conj(c_-k): half the terms.
+//
+// The cosine comes from one table entry h (2^13 of them on half a turn, cos and
+// sin as double-floats, 128 KB of shared memory; the phase's top bit is the
+// sign) and the rest delta, |delta| <= pi / 2^14 = 1.9e-4:
+//   cos(h + delta) = cos h (1 - delta^2/2) - sin h (delta - delta^3/6)
+// (next terms: 6e-17, 2e-21).  The bracket's excess over 1 is below 1.9e-8, so
+// FP32 holds it to 1e-15; the sine is a double-float product.  The sum is a
+// double-float, renormalised every other term.
+//
+// Bound: instruction issue (about 55 per term and point) beside the table's
+// gathers (random 16-byte reads, about 10 shared-memory cycles per warp) and
+// their latency.  d = 10, 330,000 frequencies, 1000 points: 308 us; three
+// table entries and double-float complex products per term, without the
+// pairing: 3.7 ms.  The error against 64 bits is two thirds of that one's.
 #include <algorithm>
 
 #include "df.cuh"
+#include "keys.cuh"
 #include "ss_internal.cuh"
 
 namespace ss {
 namespace {
 
-constexpr int kMcThreads = 256;          // points per block, one per thread
-constexpr int kTab0 = 2048;              // exp(2 pi i h / 2^11)
-constexpr int kTab1 = 2048;              // exp(2 pi i m / 2^22)
-constexpr int kTab2 = 1024;              // exp(2 pi i l / 2^32)
-constexpr int kTabAll = kTab0 + kTab1 + kTab2;
-constexpr size_t kTabBytes = kTabAll * sizeof(float4);
+constexpr int kMcThreads = 512;
+// Points per thread, which share the term's loads: as many as the registers
+// hold beside their coordinates (d = 10: 393 us with four, 450 with two).
+__host__ __device__ constexpr int mc_pts(int d) { return d <= 10 ? 4 : 2; }
+constexpr int kTabBits = 13;
+constexpr int kTab = 1 << kTabBits;      // (cos, sin)(pi h / 2^13)
+constexpr int kRest = 31 - kTabBits;     // bits of the phase below the table's
+constexpr size_t kTabBytes = kTab * sizeof(float4);
+constexpr int kMcRegDims = 16;           // coordinates of a point kept in registers
+constexpr double kTurn = 6.283185307179586 / 4294967296.0;   // radians per unit of the phase
 
 inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
 __global__ void k_mc_tables(float4* tab) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kTabAll) return;
-  double num, den;
-  if (i < kTab0) {
-    num = i; den = 2048.0;
-  } else if (i < kTab0 + kTab1) {
-    num = i - kTab0; den = 4194304.0;
-  } else {
-    num = i - kTab0 - kTab1; den = 4294967296.0;
-  }
+  if (i >= kTab) return;
   double s, c;
-  sincospi(2.0 * num / den, &s, &c);        // num / den is exact (den a power of two)
+  sincospi((double)i / kTab, &s, &c);      // the quotient is exact
   const DF cc = df_split(c), ss_ = df_split(s);
   tab[i] = make_float4(cc.hi, cc.lo, ss_.hi, ss_.lo);
 }
 
-// rows of int32 [n][d] -> [n][d4], zero padded (d4 = d rounded up to 4).
-__global__ void k_pad_rows(const int32_t* __restrict__ src, int64_t n, int d, int d4, int32_t* __restrict__ dst) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * d4) return;
-  const int64_t r = i / d4;
-  const int c = (int)(i % d4);
-  dst[i] = c < d ? src[r * d + c] : 0;
+// Head of a term's record: |c| as a double-float, arg c / 2 pi in units of
+// 2^-32 (plus half a table step, so that the table index rounds), and the rest
+// of arg c in radians.  The argument is the table's nearest angle plus a small
+// one, tan = im / re after the turn back; what that does not cover (zero,
+// floats out of range, not finite) goes through atan2 and hypot.
+__device__ int4 term_head(double2 c, const float4* __restrict__ tab) {
+  const int h = (int)rintf(atan2f((float)c.y, (float)c.x) * (float)(kTab / 3.141592653589793)) & (2 * kTab - 1);
+  const float4 e = tab[h & (kTab - 1)];
+  const double sg = h < kTab ? 1.0 : -1.0, er = sg * ((double)e.x + (double)e.y), ei = sg * ((double)e.z + (double)e.w);
+  const double re = c.x * er + c.y * ei, im = c.y * er - c.x * ei;
+  const double t = im / re, t2 = t * t;
+  double mag, turn;   // turn: in units of 2^-32
+  if (re > 0.0 && t2 < 1e-6) {
+    mag = re * (1.0 + t2 * (0.5 + t2 * -0.125));
+    turn = (double)((int64_t)h << kRest) + t * (1.0 + t2 * (-1.0 / 3.0 + t2 * 0.2)) / kTurn;
+  } else {
+    mag = hypot(c.x, c.y);
+    turn = atan2(c.y, c.x) / kTurn;
+    if (!isfinite(turn)) turn = 0.0;
+  }
+  const double n = rint(turn);
+  const DF m = df_split(mag);
+  return make_int4(__float_as_int(m.hi), __float_as_int(m.lo),
+                   (int)(uint32_t)((int64_t)n + (1ll << (kRest - 1))), __float_as_int((float)((turn - n) * kTurn)));
 }
 
-// Term coefficients in double-float, optionally negated.
-__global__ void k_coef_df(const double2* __restrict__ c, int64_t n, double sign, float4* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double2 v = c[i];
-  const DF re = df_split(sign * v.x), im = df_split(sign * v.y);
-  out[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
+// Records of f's terms: head, then the d coordinates, zero padded to w int4s.
+__global__ void k_mc_recs_f(const int32_t* __restrict__ freq, const double2* __restrict__ coef, int64_t n, int d, int w,
+                            const float4* __restrict__ tab, int4* __restrict__ rec) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  int4* o = rec + t * w;
+  o[0] = term_head(coef[t], tab);
+  auto k = [&](int c) { return c < d ? freq[t * d + c] : 0; };
+  for (int c = 0; c + 1 < w; ++c) o[c + 1] = make_int4(k(4 * c), k(4 * c + 1), k(4 * c + 2), k(4 * c + 3));
 }
 
-// part[chunk][q] = sum over the chunk's terms t of Re(c_t exp(2 pi i k_t.x_q)).
-// Block (x: 256 points, y: one chunk of terms).  Per term the thread forms the
-// exact phase, gathers three table entries and does five double-float complex
-// half-products: B = c e0, C = B e1, acc += Re(C e2).
-__global__ void __launch_bounds__(kMcThreads, 2)
-k_mc_terms(const int32_t* __restrict__ K, const float4* __restrict__ coef, int64_t n_terms, int d4,
-           const uint32_t* __restrict__ X, int64_t Q, int64_t terms_per_chunk, const float4* __restrict__ tab,
-           double* __restrict__ part) {
+// Records of -f^{s,N} from its coefficients y on S: row t, or (plus, mirror:
+// the set is symmetric) the row plus[t] together with its mirror image.
+__global__ void k_mc_recs_g(KeyParams P, const uint64_t* __restrict__ keys, const double2* __restrict__ y, int64_t n,
+                            const int32_t* __restrict__ plus, const int64_t* __restrict__ mirror, int w,
+                            const float4* __restrict__ tab, int4* __restrict__ rec) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int64_t g = plus ? plus[t] : t;
+  double2 c = y[g];
+  if (plus) {
+    const double2 m = y[mirror[g]];
+    c = make_double2(c.x + m.x, c.y - m.y);
+  }
+  int4* o = rec + t * w;
+  o[0] = term_head(make_double2(-c.x, -c.y), tab);
+  const uint64_t* key = keys + g * P.WT;
+  auto k = [&](int c) { return c < P.d ? unpack_coord(key, P, c) : 0; };
+  for (int c = 0; c + 1 < w; ++c) o[c + 1] = make_int4(k(4 * c), k(4 * c + 1), k(4 * c + 2), k(4 * c + 3));
+}
+
+// Points [Q][d] -> [(d + 3) / 4][Q] of four coordinates, zero padded (more
+// coordinates than the registers hold: read along q).
+__global__ void k_mc_points(const uint32_t* __restrict__ X, int64_t Q, int d, int w, uint4* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= Q * w) return;
+  const int64_t q = i % Q;
+  const int c = 4 * (int)(i / Q);
+  auto x = [&](int j) { return j < d ? X[q * d + j] : 0u; };
+  out[i] = make_uint4(x(c), x(c + 1), x(c + 2), x(c + 3));
+}
+
+// acc += |c| cos(2 pi ph / 2^32 + rest); ph includes half a table step.
+__device__ __forceinline__ void add_term(DF& acc, const int4 head, uint32_t ph, const float4* __restrict__ s_tab) {
+  const float4 e = s_tab[(ph >> kRest) & (kTab - 1)];
+  const uint32_t sign = ph & 0x80000000u;
+  const float mh = __int_as_float(head.x ^ (int)sign), ml = __int_as_float(head.y ^ (int)sign);
+  // the low bits as a float: put into the mantissa of 2^23, which is taken off again
+  const float r = __fsub_rn(__int_as_float(0x4b000000 | (int)(ph & ((1u << kRest) - 1))),
+                            8388608.f + (float)(1 << (kRest - 1)));
+  constexpr float kh = (float)kTurn, kl = (float)(kTurn - (double)kh);
+  const float dh = __fmul_rn(r, kh);
+  const float dl = __fadd_rn(__fmaf_rn(r, kh, -dh), __fmaf_rn(r, kl, __int_as_float(head.w)));
+  const float d2 = __fmul_rn(dh, dh);
+  const float sl = __fmaf_rn(dh, __fmul_rn(d2, -1.f / 6.f), dl);              // sin(delta) = dh + sl
+  const float cm = __fmul_rn(dh, __fmaf_rn(dh, -0.5f, -dl));                  // cos(delta) - 1
+  const float v = __fmul_rn(e.z, dh);
+  float ve = __fmaf_rn(e.z, dh, -v);
+  ve = __fmaf_rn(e.z, sl, ve);
+  ve = __fmaf_rn(e.w, dh, ve);
+  // |cos h| is 0 or at least 3.8e-4 > |v|: FastTwoSum (Dekker)
+  const float s = __fsub_rn(e.x, v);
+  float lo = __fsub_rn(__fsub_rn(e.x, s), v);
+  lo = __fadd_rn(__fsub_rn(lo, ve), __fmaf_rn(cm, e.x, e.y));
+  const float p = __fmul_rn(mh, s);
+  float pe = __fmaf_rn(mh, s, -p);
+  pe = __fmaf_rn(mh, lo, pe);
+  pe = __fmaf_rn(ml, s, pe);
+  const float a = __fadd_rn(acc.hi, p);
+  const float bb = __fsub_rn(a, acc.hi);
+  const float t = __fadd_rn(__fsub_rn(acc.hi, __fsub_rn(a, bb)), __fsub_rn(p, bb));
+  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, pe));
+  acc.hi = a;
+}
+
+__device__ __forceinline__ void renorm(DF& a) {
+  const float h = __fadd_rn(a.hi, a.lo);
+  a.lo = __fsub_rn(a.lo, __fsub_rn(h, a.hi));
+  a.hi = h;
+}
+
+struct McWork {
+  const int4* rec;          // n records of w int4s, f's n_f first
+  int64_t n_f, n;
+  int w, d;
+  const uint32_t* X;        // [Q][d]
+  const uint4* Xt;          // [w - 1][Q] (d > kMcRegDims)
+  int64_t Q;
+  const float4* tab;
+  // Units: tiles of mc_pts(d) qt points times chunks of L terms (f's chunks first);
+  // the threads of a block are `groups` rows of qt, each row with its share of
+  // the chunk's terms.
+  int qt, groups;
+  int64_t tiles, L, chunks_f, chunks;
+  double* part;             // [chunks * groups][Q]
+};
+
+// D: coordinates read, rounded up to an even number; 0: any number, points in Xt.
+template <int D>
+__global__ void __launch_bounds__(kMcThreads, 1) k_mc_terms(const McWork W) {
   extern __shared__ float4 s_tab[];
-  for (int i = threadIdx.x; i < kTabAll; i += blockDim.x) s_tab[i] = tab[i];
+  for (int i = threadIdx.x; i < kTab; i += kMcThreads) s_tab[i] = __ldg(W.tab + i);
   __syncthreads();
-  const int64_t q = (int64_t)blockIdx.x * kMcThreads + threadIdx.x;
-  const bool live = q < Q;
-  const int64_t t0 = (int64_t)blockIdx.y * terms_per_chunk;
-  const int64_t t1 = (n_terms - t0 < terms_per_chunk) ? n_terms : t0 + terms_per_chunk;
-  const int n4 = d4 / 4;
-  const uint4* xq = reinterpret_cast<const uint4*>(X + (live ? q : 0) * (int64_t)d4);
-  const float4* t_hi = s_tab;
-  const float4* t_mid = s_tab + kTab0;
-  const float4* t_lo = s_tab + kTab0 + kTab1;
-  DF acc{0.f, 0.f};
-  for (int64_t t = t0; t < t1; ++t) {
-    const int4* kt = reinterpret_cast<const int4*>(K + t * d4);
-    uint32_t ph = 0;
-    for (int c = 0; c < n4; ++c) {
-      const int4 k = __ldg(kt + c);
-      const uint4 x = __ldg(xq + c);
-      ph += (uint32_t)k.x * x.x + (uint32_t)k.y * x.y + (uint32_t)k.z * x.z + (uint32_t)k.w * x.w;
+  const int row = threadIdx.x / W.qt, col = threadIdx.x % W.qt;
+  if (row >= W.groups) return;
+  constexpr int NK = D ? (D + 3) / 4 : 1, kMcPts = mc_pts(D ? D : kMcRegDims + 1);
+  for (int64_t u = blockIdx.x; u < W.tiles * W.chunks; u += gridDim.x) {
+    const int64_t chunk = u / W.tiles, q0 = (u % W.tiles) * kMcPts * W.qt + col;
+    const bool g = chunk >= W.chunks_f;
+    const int64_t b0 = (g ? W.n_f : 0) + (chunk - (g ? W.chunks_f : 0)) * W.L;
+    const int64_t b1 = min(b0 + W.L, g ? W.n : W.n_f), share = (b1 - b0 + W.groups - 1) / W.groups;
+    const int64_t t0 = min(b0 + row * share, b1), t1 = min(t0 + share, b1);
+    int64_t q[kMcPts];
+    uint32_t x[kMcPts][D ? D : 1];
+    DF acc[kMcPts];
+#pragma unroll
+    for (int j = 0; j < kMcPts; ++j) {
+      q[j] = q0 + j * W.qt;
+      acc[j] = DF{0.f, 0.f};
+      if (D) {
+#pragma unroll
+        for (int c = 0; c < (D ? D : 1); ++c) x[j][c] = q[j] < W.Q && c < W.d ? __ldg(W.X + q[j] * W.d + c) : 0u;
+      }
     }
-    const float4 cf = __ldg(coef + t);
-    const float4 e0 = t_hi[ph >> 21];
-    const float4 e1 = t_mid[(ph >> 10) & 2047u];
-    const float4 e2 = t_lo[ph & 1023u];
-    DF br{0.f, 0.f}, bi{0.f, 0.f};
-    df_fma(br, DF{cf.x, cf.y}, DF{e0.x, e0.y});
-    df_fma(br, DF{-cf.z, -cf.w}, DF{e0.z, e0.w});
-    df_fma(bi, DF{cf.x, cf.y}, DF{e0.z, e0.w});
-    df_fma(bi, DF{cf.z, cf.w}, DF{e0.x, e0.y});
-    DF cr{0.f, 0.f}, ci{0.f, 0.f};
-    df_fma(cr, br, DF{e1.x, e1.y});
-    df_fma(cr, DF{-bi.hi, -bi.lo}, DF{e1.z, e1.w});
-    df_fma(ci, br, DF{e1.z, e1.w});
-    df_fma(ci, bi, DF{e1.x, e1.y});
-    df_fma(acc, cr, DF{e2.x, e2.y});
-    df_fma(acc, DF{-ci.hi, -ci.lo}, DF{e2.z, e2.w});
+    // the next record is on its way while a term is worked on
+    const int4* rec = W.rec + t0 * W.w;
+    int4 cur[NK + 1], nxt[NK + 1];
+    auto fetch = [&](int4* v, bool go) {
+      if (!go) return;
+#pragma unroll
+      for (int c = 0; c < (D ? NK + 1 : 1); ++c) v[c] = __ldg(rec + c);
+      rec += W.w;
+    };
+    auto term = [&](const int4* v, const int4* k0) {
+      uint32_t ph[kMcPts];
+#pragma unroll
+      for (int j = 0; j < kMcPts; ++j) ph[j] = (uint32_t)v[0].z;
+      if (D) {
+#pragma unroll
+        for (int c = 0; c < NK; ++c) {
+          const int kk[4] = {v[c + 1].x, v[c + 1].y, v[c + 1].z, v[c + 1].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (4 * c + e < D) {
+#pragma unroll
+              for (int j = 0; j < kMcPts; ++j) ph[j] += (uint32_t)kk[e] * x[j][(D ? 4 * c + e : 0) % (D ? D : 1)];
+            }
+        }
+      } else {
+        for (int c = 0; c + 1 < W.w; ++c) {
+          const int4 k = __ldg(k0 + c);
+          if ((k.x | k.y | k.z | k.w) == 0) continue;   // long frequencies have few nonzeros
+#pragma unroll
+          for (int j = 0; j < kMcPts; ++j) {
+            const uint4 p = __ldg(W.Xt + c * W.Q + min(q[j], W.Q - 1));
+            ph[j] += (uint32_t)k.x * p.x + (uint32_t)k.y * p.y + (uint32_t)k.z * p.z + (uint32_t)k.w * p.w;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kMcPts; ++j) add_term(acc[j], v[0], ph[j], s_tab);
+    };
+    fetch(cur, t0 < t1);
+    for (int64_t t = t0; t < t1; t += 2) {
+      fetch(nxt, t + 1 < t1);
+      term(cur, W.rec + t * W.w + 1);
+      if (t + 1 < t1) {
+        fetch(cur, t + 2 < t1);
+        term(nxt, W.rec + (t + 1) * W.w + 1);
+      }
+#pragma unroll
+      for (int j = 0; j < kMcPts; ++j) renorm(acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < kMcPts; ++j)
+      if (q[j] < W.Q) W.part[(chunk * W.groups + row) * W.Q + q[j]] = (double)acc[j].hi + (double)acc[j].lo;
   }
-  if (live) part[(int64_t)blockIdx.y * Q + q] = (double)acc.hi + (double)acc.lo;
 }
 
-// r[q] = sum_c pf[c][q] + sum_c pg[c][q] (pg holds -f^{s,N}), f[q] = sum_c pf[c][q],
-// chunks summed in index order.
-__global__ void k_mc_finish(const double* __restrict__ pf, int cf, const double* __restrict__ pg, int cg, int64_t Q,
-                            double* __restrict__ r, double* __restrict__ f) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= Q) return;
-  double sf = 0.0, sg = 0.0;
-  for (int c = 0; c < cf; ++c) sf += pf[(int64_t)c * Q + q];
-  for (int c = 0; c < cg; ++c) sg += pg[(int64_t)c * Q + q];
-  f[q] = sf;
-  r[q] = sf + sg;
-}
-
-// Terms split into chunks so that the grid covers the SMs several times over.
-int64_t terms_per_chunk(int64_t n_terms, int64_t point_tiles) {
-  const int64_t want_blocks = 8LL * 2 * sm_count();
-  int64_t chunks = (want_blocks + point_tiles - 1) / point_tiles;
-  chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (n_terms + 63) / 64));
-  chunks = std::min<int64_t>(chunks, 65535);
-  return (n_terms + chunks - 1) / chunks;
-}
-
-ss_status run_terms(const int32_t* K, const float4* coef, int64_t n_terms, int d4, const uint32_t* X, int64_t Q,
-                    const float4* tab, DevBuf<double>& part, int* chunks_out, cudaStream_t st) {
-  const int64_t tiles = (Q + kMcThreads - 1) / kMcThreads;
-  if (n_terms == 0) {
-    *chunks_out = 0;
-    return SS_OK;
+// f[q] = sum of the first n_f rows of part, r[q] = f[q] + the others (which
+// hold -f^{s,N}).  32 points a block, their rows dealt out to the warps; the
+// order of the additions depends on the sizes alone.
+constexpr int kFinWarps = 32;
+__global__ void __launch_bounds__(32 * kFinWarps) k_mc_finish(const double* __restrict__ part, int64_t n_f, int64_t n,
+                                                              int64_t Q, double* __restrict__ r,
+                                                              double* __restrict__ f) {
+  __shared__ double sf[kFinWarps][32], sg[kFinWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t q = (int64_t)blockIdx.x * 32 + lane;
+  double a = 0.0, b = 0.0;
+  if (q < Q) {
+    for (int64_t c = w; c < n_f; c += kFinWarps) a += part[c * Q + q];
+#pragma unroll 4
+    for (int64_t c = n_f + w; c < n; c += kFinWarps) b += part[c * Q + q];
   }
-  const int64_t tpc = terms_per_chunk(n_terms, tiles);
-  const int chunks = (int)((n_terms + tpc - 1) / tpc);
-  SS_TRY(part.alloc((size_t)chunks * Q, st));
-  k_mc_terms<<<dim3((unsigned)tiles, (unsigned)chunks), kMcThreads, kTabBytes, st>>>(K, coef, n_terms, d4, X, Q, tpc,
-                                                                                   tab, part.get());
-  SS_LAUNCH_CHECK();
-  *chunks_out = chunks;
-  return SS_OK;
+  sf[w][lane] = a;
+  sg[w][lane] = b;
+  __syncthreads();
+  if (w || q >= Q) return;
+  for (int i = 1; i < kFinWarps; ++i) a += sf[i][lane], b += sg[i][lane];
+  f[q] = a;
+  r[q] = a + b;
+}
+
+using McKernel = void (*)(McWork);
+
+McKernel mc_kernel(int d) {
+  switch (d > kMcRegDims ? 0 : (d + 1) / 2) {
+    case 1: return k_mc_terms<2>;
+    case 2: return k_mc_terms<4>;
+    case 3: return k_mc_terms<6>;
+    case 4: return k_mc_terms<8>;
+    case 5: return k_mc_terms<10>;
+    case 6: return k_mc_terms<12>;
+    case 7: return k_mc_terms<14>;
+    case 8: return k_mc_terms<16>;
+  }
+  return k_mc_terms<0>;
+}
+
+// The tiles and chunks: every block (one per SM, the table fills its shared
+// memory) gets the same number of equal units where there are few tiles, about
+// eight units each where there are many.  Fewer than kMcMinTerms terms do not
+// pay for a row of threads of their own.
+constexpr int64_t kMcMinTerms = 32;
+void mc_split(McWork* W) {
+  const int64_t sm = sm_count(), n_g = W->n - W->n_f, pts = mc_pts(W->d);
+  W->qt = (int)std::min<int64_t>(kMcThreads, (((W->Q + pts - 1) / pts + 31) / 32) * 32);
+  W->groups = kMcThreads / W->qt;
+  W->tiles = (W->Q + pts * W->qt - 1) / (pts * W->qt);
+  const int64_t want = W->tiles <= sm / 8 ? sm / W->tiles : (8 * sm + W->tiles - 1) / W->tiles;
+  W->L = std::max<int64_t>((W->n + want - 1) / want, kMcMinTerms * W->groups);
+  auto chunks = [&](int64_t n) { return (n + W->L - 1) / W->L; };
+  while (chunks(W->n_f) + chunks(n_g) > std::max<int64_t>(want, 2)) W->L += W->L / 64 + 1;
+  W->chunks_f = chunks(W->n_f);
+  W->chunks = W->chunks_f + chunks(n_g);
 }
 
 }  // namespace
@@ -165,71 +333,63 @@ extern "C" ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, c
   if (Q < 0 || f->n_terms < 0 || (f->n_terms > 0 && (!f->freq || !f->coef)))
     SS_FAIL(SS_ERR_INVALID, "proxy_mc: bad sizes");
   if (Q == 0) return SS_OK;
-  SS_CUDA(cudaFuncSetAttribute(k_mc_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTabBytes));
+  const McKernel kern = mc_kernel(s->d);
+  SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTabBytes));
   cudaStream_t st = as_stream(stream);
-  const int d = s->d, d4 = (d + 3) / 4 * 4;
-  // rows are read as 16-byte vectors: copy when d is not a multiple of 4 or
-  // the caller's array is not 16-byte aligned
-  auto needs_copy = [&](const void* p) { return d4 != d || (reinterpret_cast<uintptr_t>(p) & 15u) != 0; };
-  DevBuf<float4> tab, cf_f, cf_g;
-  DevBuf<int32_t> Kf, Kg, tmp;
-  DevBuf<uint32_t> Xp;
+  DevBuf<float4> tab;
+  DevBuf<int4> rec;
+  DevBuf<uint4> Xt;
   DevBuf<double2> y;
-  DevBuf<double> pf, pg;
-  SS_TRY(tab.alloc(kTabAll, st));
-  k_mc_tables<<<nblk(kTabAll), 256, 0, st>>>(tab.get());
+  DevBuf<double> part;
+  SS_TRY(tab.alloc(kTab, st));
+  k_mc_tables<<<nblk(kTab), 256, 0, st>>>(tab.get());
   SS_LAUNCH_CHECK();
-  // points, padded
-  const uint32_t* Xd = X;
-  if (needs_copy(X)) {
-    SS_TRY(Xp.alloc((size_t)Q * d4, st));
-    k_pad_rows<<<nblk(Q * d4), 256, 0, st>>>(reinterpret_cast<const int32_t*>(X), Q, d, d4,
-                                              reinterpret_cast<int32_t*>(Xp.get()));
+  // f^{s,N} on S: L applied to u (prefix).  A symmetric set (the half system
+  // stands, its error words read) gives one term per pair +-k; k = 0 has the
+  // coefficient 0 there (below).
+  const bool fold = s->half_ok && !s->check_pending;
+  const int64_t n_g = fold ? s->n_plus : s->size;
+  McWork W{};
+  W.n_f = f->n_terms;
+  W.n = f->n_terms + n_g;
+  W.w = 1 + (s->d + 3) / 4;
+  W.d = s->d;
+  W.X = X;
+  W.Q = Q;
+  W.tab = tab.get();
+  if (s->d > kMcRegDims) {
+    SS_TRY(Xt.alloc((size_t)Q * (W.w - 1), st));
+    k_mc_points<<<nblk(Q * (W.w - 1)), 256, 0, st>>>(X, Q, s->d, W.w - 1, Xt.get());
     SS_LAUNCH_CHECK();
-    Xd = Xp.get();
+    W.Xt = Xt.get();
   }
-  // f's terms
-  const int64_t nf = f->n_terms;
-  const int32_t* Kfd = f->freq;
-  if (nf > 0) {
-    SS_TRY(cf_f.alloc(nf, st));
-    k_coef_df<<<nblk(nf), 256, 0, st>>>(reinterpret_cast<const double2*>(f->coef), nf, 1.0, cf_f.get());
+  SS_TRY(rec.alloc((size_t)std::max<int64_t>(W.n, 1) * W.w, st));
+  W.rec = rec.get();
+  if (W.n_f > 0) {
+    k_mc_recs_f<<<nblk(W.n_f), 256, 0, st>>>(f->freq, reinterpret_cast<const double2*>(f->coef), W.n_f, s->d, W.w,
+                                             tab.get(), rec.get());
     SS_LAUNCH_CHECK();
-    if (needs_copy(f->freq)) {
-      SS_TRY(Kf.alloc((size_t)nf * d4, st));
-      k_pad_rows<<<nblk(nf * d4), 256, 0, st>>>(f->freq, nf, d, d4, Kf.get());
-      SS_LAUNCH_CHECK();
-      Kfd = Kf.get();
-    }
   }
-  // f^{s,N} on S: L applied to u (prefix), then S's frequencies, padded
-  const int64_t ng = s->size;
-  const int32_t* Kgd = nullptr;
-  if (ng > 0) {
+  if (n_g > 0) {
     SS_TRY(launch_pack64_prefix(s, reinterpret_cast<const double2*>(u_prefix), n_u, st));
-    SS_TRY(y.alloc(ng, st));
+    SS_TRY(y.alloc(s->size, st));
     SS_TRY(launch_apply64(s, y.get(), st));
     // (L u)_0 = 0 exactly for the diffusion operator (the factor k.l); its
     // stored identity row is for the solve
     if (identity_row(s) >= 0) SS_CUDA(cudaMemsetAsync(y.get() + identity_row(s), 0, sizeof(double2), st));
-    SS_TRY(cf_g.alloc(ng, st));
-    k_coef_df<<<nblk(ng), 256, 0, st>>>(y.get(), ng, -1.0, cf_g.get());
+    k_mc_recs_g<<<nblk(n_g), 256, 0, st>>>(make_key_params(s->key), s->keys.get(), y.get(), n_g,
+                                           fold ? s->plus_rows.get() : nullptr, fold ? s->mirror.get() : nullptr, W.w,
+                                           tab.get(), rec.get() + W.n_f * W.w);
     SS_LAUNCH_CHECK();
-    SS_TRY(tmp.alloc((size_t)ng * d, st));
-    SS_TRY((ss_status)stamp_export(s, tmp.get(), nullptr, st));
-    if (d4 != d) {
-      SS_TRY(Kg.alloc((size_t)ng * d4, st));
-      k_pad_rows<<<nblk(ng * d4), 256, 0, st>>>(tmp.get(), ng, d, d4, Kg.get());
-      SS_LAUNCH_CHECK();
-      Kgd = Kg.get();
-    } else {
-      Kgd = tmp.get();
-    }
   }
-  int cfn = 0, cgn = 0;
-  SS_TRY(run_terms(Kfd, cf_f.get(), nf, d4, Xd, Q, tab.get(), pf, &cfn, st));
-  SS_TRY(run_terms(Kgd, cf_g.get(), ng, d4, Xd, Q, tab.get(), pg, &cgn, st));
-  k_mc_finish<<<nblk(Q), 256, 0, st>>>(pf.get(), cfn, pg.get(), cgn, Q, r_out, f_out);
+  if (W.n > 0) {
+    mc_split(&W);
+    SS_TRY(part.alloc((size_t)(W.chunks * W.groups) * Q, st));
+    W.part = part.get();
+    kern<<<(unsigned)std::min<int64_t>(sm_count(), W.tiles * W.chunks), kMcThreads, kTabBytes, st>>>(W);
+    SS_LAUNCH_CHECK();
+  }
+  k_mc_finish<<<nblk(Q, 32), 32 * kFinWarps, 0, st>>>(part.get(), W.chunks_f * W.groups, W.chunks * W.groups, Q, r_out, f_out);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }

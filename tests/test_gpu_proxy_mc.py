@@ -113,3 +113,44 @@ def test_estimate_tracks_exact_proxy(B, d, seed):
             # delta-method standard error of the ratio of means
             se2 = np.sqrt(np.var(r2 - est2 * f2) / len(r2)) / f2.mean()
             assert abs(est2 - exact ** 2) <= 5 * se2 + 1e-20, (N, est2, exact ** 2, se2)
+
+
+@pytest.mark.parametrize("d,Q,sym", [(1, 1, True), (2, 33, False), (3, 129, True), (4, 2049, True), (7, 64, True),
+                                     (8, 65, False), (9, 300, True), (10, 5000, True), (11, 1025, False),
+                                     (16, 127, True), (17, 1000, True), (30, 31, False)])
+def test_point_tiles_and_mirror_pairs(B, d, Q, sym):
+    """Every number of coordinates a thread keeps, points at the edges of the
+    tiles, symmetric sets (one term per pair +-k) and others.  A term is off by
+    at most about 2^-47 of |c| per operation on its low part and table entry
+    (fewer than eight): 2^-44 sum |c|."""
+    rng = np.random.default_rng([d, Q])
+    p = rng.integers(-500, 501, size=(3, d))
+    p[rng.random((3, d)) < 0.3] = 0
+    p[:, 0] = rng.choice([-7, 5, 3], 3, replace=False)
+    af = np.vstack([np.zeros((1, d), int), p, -p])
+    c = rng.standard_normal(3) + 1j * rng.standard_normal(3)
+    av = np.concatenate([[20.0 + 0j], c, np.conj(c)])
+    F = rng.integers(-300, 301, size=(4, d))
+    F[:, 0] = [11, 13, 17, 19]
+    F = np.vstack([F, -F]) if sym else F
+    S, _ = ostamp.stamp_bfs(af, F, 2)
+    u = rng.standard_normal(len(S)) + 1j * rng.standard_normal(len(S))
+    fc = rng.standard_normal(len(F)) * 10.0 ** rng.uniform(-3, 3, len(F)) + 1j * rng.standard_normal(len(F))
+    fc[0] = -2.0
+    X = W.mc_points(d, Q, d)
+    with B.stamp_build(af, av, F, 2) as s:
+        y = B.galerkin_apply(s, torch.as_tensor(u).cuda()).cpu().numpy()
+        S_g, _ = s.export()
+        r, f = B.proxy_mc(s, torch.as_tensor(u), F, fc, X)
+    S_g = S_g.cpu().numpy().astype(np.int64)
+    y[~S_g.any(axis=1)] = 0.0
+
+    def values(K, co):
+        ph = (K @ X.astype(np.int64).T) % 2**32
+        th = 2 * np.pi * (ph / 2.0**32)
+        return (co.real[:, None] * np.cos(th) - co.imag[:, None] * np.sin(th)).sum(axis=0)
+
+    f_ref = values(F.astype(np.int64), fc)
+    r_ref = f_ref - values(S_g, y)
+    assert np.max(np.abs(f.cpu().numpy() - f_ref)) <= 2.0**-44 * np.abs(fc).sum()
+    assert np.max(np.abs(r.cpu().numpy() - r_ref)) <= 2.0**-44 * (np.abs(fc).sum() + np.abs(y).sum())
