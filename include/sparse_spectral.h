@@ -195,7 +195,9 @@ ss_status sft_recover_samples(const ss_lattice* lat, const void* samples, ss_pre
  * FFT buffers).  In FP64 on a 7-smooth M up to 2^22 both transforms (the
  * inverse one that samples g and the forward one that recovers it) run in the
  * library's fixed-point FFT instead of cuFFT.  Its rounding is about 2^-56 of
- * sum |coef| in every bin.  The thresholding and output are as in sft_recover_samples.
+ * sum |coef| in every bin.  On a shorter M with another prime factor (M up to
+ * 2^15, at most 4096 candidates, M times the candidates and M times the terms
+ * up to 2^22) samples and bins are direct FP64 sums.  The thresholding and output are as in sft_recover_samples.
  * Synchronises `stream`. */
 ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_precision prec, const int32_t* cand,
                       int64_t n_cand, int64_t s_max, double tau, int32_t* freq_out, double* val_out,

@@ -19,6 +19,7 @@
 // the nodes of a rank-1 lattice is a length-M inverse DFT.
 #include <cufft.h>
 
+#include <climits>
 #include <cstdlib>
 
 #include <list>
@@ -477,6 +478,11 @@ __global__ void k_compact(const int32_t* __restrict__ cand, const double2* __res
 inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
 // Per-(M, precision) FFT plan, sample and spectrum buffers and twiddle tables.
+// Direct sums (see direct_recover_pair): the largest M with a table of its
+// roots, and the bound on M times candidates or terms.
+constexpr int64_t kDirectMaxM = 1 << 15;
+constexpr int64_t kDirectMaxWork = 1 << 22;
+
 struct SftPlan {
   int64_t M = 0;
   ss_precision prec = SS_FP64;
@@ -493,6 +499,7 @@ struct SftPlan {
   FxFftPlan fx;
   DevBuf<longlong2> fxz, fxtmp;
   DevBuf<int4> fxtab;
+  DevBuf<double2> roots;    // exp(2 pi i r / M), r < M, of the direct sums (kDirectMaxM)
   DevBuf<double> fxscale;   // the two sums' scales and floors of the last round trip
   // pruned transforms (on a 7-smooth M above the full table's limit;
   // double-float arithmetic in FP64, FP32 in FP32): two-level twiddle table,
@@ -592,6 +599,10 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
       SS_TRY(p->fxscale.alloc(4, st));
       SS_TRY(fx_fft_table(p->fx, p->fxtab.get(), st));
       p->has_fx = true;
+    } else if (p->df && M <= kDirectMaxM) {
+      SS_TRY(p->roots.alloc(M, st));
+      k_twiddles_full<<<nblk(M), 256, 0, st>>>(M, p->roots.get());
+      SS_LAUNCH_CHECK();
     }
   }
   if (M > kFullTableMax && !(prec == SS_FP64 && native_fp64_sampling()) && pruned_supported(M)) {
@@ -607,7 +618,7 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
   // the plan is cached across calls and streams
   SS_CUDA(cudaStreamSynchronize(st));
   p->samples.settle(); p->spectrum.settle(); p->lo.settle(); p->hi.settle(); p->full.settle();
-  p->fxz.settle(); p->fxtmp.settle(); p->fxtab.settle(); p->fxscale.settle();
+  p->fxz.settle(); p->fxtmp.settle(); p->fxtab.settle(); p->fxscale.settle(); p->roots.settle();
   p->prt.t0.settle(); p->prt.t1.settle(); p->prz.settle(); p->prscale.settle();
   for (auto& t : p->t3) t.settle();
   g_plans.push_front(p);
@@ -715,13 +726,19 @@ __global__ void k_bin_terms(const int64_t* __restrict__ q, const double2* __rest
 // is zero, NaN where a coefficient of either sum is not finite or a scale has
 // no reciprocal (integers would hide it).
 constexpr int kScaleThreads = 512;
+// |c|: hypot, which costs thirty FP64 instructions more, only where squares leave the range
+__device__ __forceinline__ double magnitude(const double2 c) {
+  const double m = sqrt(fma(c.x, c.x, c.y * c.y));
+  return m > 1e-140 && m < 1e140 ? m : hypot(c.x, c.y);
+}
+
 template <bool UNITS = false>
 __device__ void pair_scale(const double2* const c[2], const int64_t n[2], double* scale) {
   double total[2];
   __shared__ double s_part[kScaleThreads];
   for (int w = 0; w < 2; ++w) {
     double acc = 0.0;
-    for (int64_t t = threadIdx.x; t < n[w]; t += kScaleThreads) acc += hypot(c[w][t].x, c[w][t].y);
+    for (int64_t t = threadIdx.x; t < n[w]; t += kScaleThreads) acc += magnitude(c[w][t]);
     s_part[threadIdx.x] = acc;
     __syncthreads();
     for (int o = kScaleThreads / 2; o > 0; o >>= 1) {
@@ -887,11 +904,222 @@ struct Terms {
   DevBuf<int32_t> lead;   // index of the term each merged one is written in the orientation of (on request)
 };
 
+// Sums with at most kPrepSmall terms: one launch, one block per sum doing every
+// step of prep_terms in shared memory.  A group of G lanes takes a term, as
+// many terms at once as the block holds.  Equal representatives meet in a hash
+// table, which keeps the smallest index of each and its number; a key that two
+// different representatives share (none is known) sends the block to the
+// comparison of all pairs.  Two blocks of 840 and 21 terms, d = 10: 155 us with
+// a warp per term and all pairs of hashes, 16 us so.
+constexpr int kPrepSmall = 1024;
+constexpr int kPrepSlots = 2 * kPrepSmall;
+
+struct PrepArgs {
+  const int32_t* freq;
+  const double2* coef;
+  int64_t n;
+  int64_t* q;
+  int64_t* step;
+  double2* coef_out;
+  int64_t* total;
+  int32_t* lead;   // nullable
+};
+
+__global__ void __launch_bounds__(1024) k_prep_terms_small(PrepArgs A0, PrepArgs A1, LatticeDev L) {
+  __shared__ int32_t s_sgn[kPrepSmall], s_first[kPrepSmall], s_pos[kPrepSmall];
+  __shared__ unsigned long long s_key[kPrepSlots];
+  __shared__ int32_t s_min[kPrepSlots];
+  __shared__ uint32_t s_cnt[kPrepSlots];   // members << 21 | sum of their indices
+  __shared__ int32_t s_wsum[32];
+  __shared__ int s_clash;
+  const PrepArgs& A = blockIdx.x == 0 ? A0 : A1;
+  const int n = (int)A.n, d = L.d;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int G = 1;
+  while (G < 32 && 2 * G * n <= (int)blockDim.x && G < d) G *= 2;
+  const int gl = threadIdx.x & (G - 1), g0 = threadIdx.x / G, ng = blockDim.x / G;
+  for (int i = threadIdx.x; i < kPrepSlots; i += blockDim.x) {
+    s_key[i] = 0;
+    s_min[i] = n;
+    s_cnt[i] = 0;
+  }
+  if (threadIdx.x == 0) s_clash = 0;
+  __syncthreads();
+  // sign of the first nonzero coordinate, and a hash of the representative sgn p
+  for (int t0 = 0; t0 < n; t0 += ng) {
+    const int t = t0 + g0;
+    uint64_t h = 0;
+    int lead = INT_MAX;   // 2 c + (p_c < 0) of the first nonzero c
+    if (t < n) {
+      const int32_t* p = A.freq + (int64_t)t * d;
+#pragma unroll 4
+      for (int c = gl; c < d; c += G) {
+        const int32_t v = p[c];
+        h += (uint64_t)(int64_t)v * mix64((uint64_t)c + 1);   // odd in p: -p has the hash -h
+        if (v && lead == INT_MAX) lead = 2 * c + (v < 0);
+      }
+    }
+    for (int o = G / 2; o > 0; o >>= 1) {
+      h += __shfl_xor_sync(0xffffffffu, h, o);
+      lead = min(lead, __shfl_xor_sync(0xffffffffu, lead, o));
+    }
+    if (t >= n || gl) continue;
+    const int sg = lead == INT_MAX ? 0 : (lead & 1 ? -1 : 1);
+    if (sg < 0) h = 0ull - h;
+    if (h == 0) h = 1;   // 0: free slot
+    s_sgn[t] = sg;
+    uint32_t at = (uint32_t)mix64(h) & (kPrepSlots - 1);
+    for (;;) {   // at most n < kPrepSlots keys
+      const unsigned long long old = atomicCAS(&s_key[at], 0ull, (unsigned long long)h);
+      if (old == 0 || old == h) break;
+      at = (at + 1) & (kPrepSlots - 1);
+    }
+    atomicMin(&s_min[at], t);
+    atomicAdd(&s_cnt[at], (1u << 21) + (uint32_t)t);
+    s_pos[t] = (int32_t)at;
+  }
+  __syncthreads();
+  auto differ = [&](int t, int u, int c) {
+    const int32_t x = A.freq[(int64_t)t * d + c], y = A.freq[(int64_t)u * d + c];
+    return (s_sgn[t] < 0 ? -x : x) != (s_sgn[u] < 0 ? -y : y);
+  };
+  // first occurrence of every representative (n: the term itself)
+  for (int t = g0; t < n; t += ng) {
+    const int u = s_min[s_pos[t]];
+    bool diff = false;
+    if (u != t)
+      for (int c = gl; c < d; c += G) diff |= differ(t, u, c);
+    if (diff) s_clash = 1;
+    if (gl == 0) s_first[t] = u == t ? n : u;
+  }
+  __syncthreads();
+  const bool clash = s_clash != 0;
+  if (clash) {
+    for (int t = w; t < n; t += nw) {
+      int fu = n;
+      for (int u = 0; u < t && fu == n; ++u) {
+        bool diff = false;
+        for (int c = lane; c < d; c += 32) diff |= differ(t, u, c);
+        if (!__any_sync(0xffffffffu, diff)) fu = u;
+      }
+      __syncwarp();
+      if (lane == 0) s_first[t] = fu;
+    }
+    __syncthreads();
+  }
+  // exclusive prefix sum of the leader flags (n <= blockDim)
+  const int t = threadIdx.x;
+  const int slot = t < n ? s_pos[t] : 0;
+  const int f = t < n && s_first[t] == n ? 1 : 0;
+  int x = f;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_wsum[w] = x;
+  __syncthreads();
+  int before = 0, total = 0;
+  for (int q = 0; q < nw; ++q) {
+    if (q < w) before += s_wsum[q];
+    total += s_wsum[q];
+  }
+  const int pos = f ? before + x - f : -1;
+  if (t < n) s_pos[t] = pos;
+  if (t == 0) *A.total = total;
+  // leaders of one or two terms sum their group here
+  const uint32_t cnt = t < n && !clash ? s_cnt[slot] : 0;
+  const bool few = f && (cnt >> 21) >= 1 && (cnt >> 21) <= 2;
+  if (few) {
+    double2 c = A.coef[t];
+    const int u = (int)(cnt & ((1u << 21) - 1)) - t;   // the other one
+    if ((cnt >> 21) == 2) {
+      const double2 e = A.coef[u];
+      c.x += e.x;
+      c.y += s_sgn[u] == s_sgn[t] ? e.y : -e.y;
+    }
+    if (s_sgn[t] == 0) c.y = 0.0;
+    A.coef_out[pos] = c;
+  }
+  const bool many = f && !few;
+  const int any_many = __syncthreads_or(many);   // (also: s_pos is written)
+  if (any_many) {
+    // larger groups: one warp each, lanes in a fixed stride, then a fixed butterfly
+    for (int v = w; v < n; v += nw) {
+      if (s_first[v] != n) continue;
+      const int st = s_sgn[v];
+      double re = 0.0, im = 0.0;
+      int members = 0;
+      for (int u = v + lane; u < n; u += 32) {
+        if (u != v && s_first[u] != v) continue;
+        const double2 c = A.coef[u];
+        re += c.x;
+        im += (s_sgn[u] == st) ? c.y : -c.y;
+        ++members;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+        members += __shfl_xor_sync(0xffffffffu, members, o);
+      }
+      if (lane == 0 && (clash || members > 2)) A.coef_out[s_pos[v]] = make_double2(re, st == 0 ? 0.0 : im);
+    }
+  }
+  // residues of the leaders
+  const uint64_t M = (uint64_t)L.M, inv = ~0ull / M;
+  for (int u0 = 0; u0 < n; u0 += ng) {
+    const int u = u0 + g0;
+    const int k = u < n ? s_pos[u] : -1;
+    uint64_t acc = 0;
+    if (k >= 0) {
+      const int32_t* p = A.freq + (int64_t)u * d;
+      for (int c = gl; c < d; c += G) {
+        int64_t kc = p[c];
+        if (kc < 0 || kc >= L.M) {
+          kc %= L.M;
+          if (kc < 0) kc += L.M;
+        }
+        acc += mulmod((uint64_t)kc, (uint64_t)L.z[c], M, inv);
+        if (acc >= M) acc -= M;
+      }
+    }
+    for (int o = G / 2; o > 0; o >>= 1) {
+      acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (acc >= M) acc -= M;
+    }
+    if (k < 0 || gl) continue;
+    A.q[k] = (int64_t)acc;
+    A.step[k] = (int64_t)((acc * (uint64_t)kSampThreads) % M);
+    if (A.lead) A.lead[k] = u;
+  }
+}
+
+ss_status small_args(const ss_trig* g, Terms* T, cudaStream_t st, PrepArgs* A) {
+  const int64_t n = g->n_terms;
+  SS_TRY(T->total.alloc_tmp(1, st));
+  SS_TRY(T->q.alloc_tmp(std::max<int64_t>(n, 1), st));
+  SS_TRY(T->step.alloc_tmp(std::max<int64_t>(n, 1), st));
+  SS_TRY(T->coef.alloc_tmp(std::max<int64_t>(n, 1), st));
+  *A = PrepArgs{g->freq, reinterpret_cast<const double2*>(g->coef), n, T->q.get(), T->step.get(), T->coef.get(),
+                T->total.get(), nullptr};
+  return SS_OK;
+}
+
 // Merge +-p terms (exact rewrite of the real sum) and compact them; no host
 // synchronisation (the merged count stays on the device).
 ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream_t st, bool want_lead = false) {
   ProfScope prof_("prep_terms", st);
   const int64_t n = g->n_terms;
+  if (want_lead) SS_TRY(T->lead.alloc_tmp(n, st));
+  if (n <= kPrepSmall) {
+    PrepArgs A;
+    SS_TRY(small_args(g, T, st, &A));
+    A.lead = want_lead ? T->lead.get() : nullptr;
+    k_prep_terms_small<<<1, 1024, 0, st>>>(A, A, L);
+    SS_LAUNCH_CHECK();
+    return SS_OK;
+  }
   SS_TRY(T->total.alloc_tmp(1, st));
   if (n == 0) {
     SS_CUDA(cudaMemsetAsync(T->total.get(), 0, sizeof(int64_t), st));
@@ -916,134 +1144,10 @@ ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream
                                             flag.get(), merged.get(), imag.get());
   SS_LAUNCH_CHECK();
   SS_TRY(exclusive_scan_i32(flag.get(), pos.get(), n, T->total.get(), st));
-  if (want_lead) SS_TRY(T->lead.alloc_tmp(n, st));
   k_compact_terms<<<nblk(n * 32), 256, 0, st>>>(g->freq, n, L, flag.get(), pos.get(), merged.get(), T->q.get(),
                                                 T->step.get(), T->coef.get(), want_lead ? T->lead.get() : nullptr);
   SS_LAUNCH_CHECK();
   return SS_OK;
-}
-
-// Both sums of a pair with at most kPrepSmall terms each: one launch, one
-// block per sum doing every step of prep_terms (signs, first occurrences,
-// leader sums in the same order, prefix sum, compaction) in shared memory.
-constexpr int kPrepSmall = 1024;
-
-struct PrepArgs {
-  const int32_t* freq;
-  const double2* coef;
-  int64_t n;
-  int64_t* q;
-  int64_t* step;
-  double2* coef_out;
-  int64_t* total;
-};
-
-__global__ void __launch_bounds__(1024) k_prep_terms_small(PrepArgs A0, PrepArgs A1, LatticeDev L) {
-  __shared__ int32_t s_sgn[kPrepSmall], s_first[kPrepSmall], s_pos[kPrepSmall];
-  __shared__ double2 s_merged[kPrepSmall];
-  __shared__ uint64_t s_hash[kPrepSmall];
-  __shared__ int32_t s_wsum[32];
-  const PrepArgs& A = blockIdx.x == 0 ? A0 : A1;
-  const int n = (int)A.n, d = L.d;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // signs of the first nonzero coordinates
-  for (int t = w; t < n; t += nw) {
-    int sg = 0;
-    for (int c0 = 0; c0 < d && sg == 0; c0 += 32) {
-      const int32_t v = c0 + lane < d ? A.freq[(int64_t)t * d + c0 + lane] : 0;
-      const unsigned m = __ballot_sync(0xffffffffu, v != 0);
-      if (m) sg = __shfl_sync(0xffffffffu, v, __ffs(m) - 1) > 0 ? 1 : -1;
-    }
-    // a hash of the representative sgn p: equal representatives, equal hashes
-    const int x = sg < 0 ? -1 : 1;
-    uint64_t h = 0;
-    for (int c = lane; c < d; c += 32)
-      h += (uint64_t)(int64_t)(x * A.freq[(int64_t)t * d + c]) * (0x9e3779b97f4a7c15ull ^ ((uint64_t)c << 32 | 1u));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
-    if (lane == 0) {
-      s_sgn[t] = sg;
-      s_hash[t] = h;
-    }
-  }
-  __syncthreads();
-  // first occurrence of every representative: hashes compared 32 at a time,
-  // the coordinates only where they agree
-  for (int t = w; t < n; t += nw) {
-    const int xt = s_sgn[t] < 0 ? -1 : 1;
-    const int32_t* pt = A.freq + (int64_t)t * d;
-    const uint64_t ht = s_hash[t];
-    int fu = n;
-    for (int u0 = 0; u0 < t && fu == n; u0 += 32) {
-      unsigned m = __ballot_sync(0xffffffffu, u0 + lane < t && s_hash[u0 + lane] == ht);
-      while (m) {
-        const int u = u0 + __ffs(m) - 1;
-        m &= m - 1;
-        const int xu = s_sgn[u] < 0 ? -1 : 1;
-        const int32_t* pu = A.freq + (int64_t)u * d;
-        bool diff = false;
-        for (int c = lane; c < d; c += 32) diff |= xu * pu[c] != xt * pt[c];
-        if (!__any_sync(0xffffffffu, diff)) {
-          fu = u;
-          break;
-        }
-      }
-    }
-    if (lane == 0) s_first[t] = fu;
-  }
-  __syncthreads();
-  // leaders sum their groups (lanes in a fixed stride, then a fixed butterfly)
-  for (int t = w; t < n; t += nw) {
-    const bool leader = s_first[t] == n;
-    if (lane == 0) s_pos[t] = leader ? 1 : 0;
-    if (!leader) continue;
-    const int st = s_sgn[t];
-    double re = 0.0, im = 0.0;
-    for (int u = t + lane; u < n; u += 32) {
-      if (u != t && s_first[u] != t) continue;
-      const double2 c = A.coef[u];
-      re += c.x;
-      im += (s_sgn[u] == st) ? c.y : -c.y;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      re += __shfl_xor_sync(0xffffffffu, re, o);
-      im += __shfl_xor_sync(0xffffffffu, im, o);
-    }
-    if (lane == 0) s_merged[t] = make_double2(re, st == 0 ? 0.0 : im);
-  }
-  __syncthreads();
-  // exclusive prefix sum of the leader flags (n <= blockDim)
-  const int t = threadIdx.x;
-  const int f = t < n ? s_pos[t] : 0;
-  int x = f;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_wsum[w] = x;
-  __syncthreads();
-  int before = 0, total = 0;
-  for (int q = 0; q < nw; ++q) {
-    if (q < w) before += s_wsum[q];
-    total += s_wsum[q];
-  }
-  __syncthreads();
-  if (t < n) s_pos[t] = f ? before + x - f : -1;
-  if (t == 0) *A.total = total;
-  __syncthreads();
-  // compaction: the residue of every leader by its warp
-  for (int u = w; u < n; u += nw) {
-    const int k = s_pos[u];
-    if (k < 0) continue;
-    const int64_t r = residue_warp(A.freq + (int64_t)u * d, d, L);
-    if (lane == 0) {
-      A.q[k] = r;
-      A.step[k] = (int64_t)(((uint64_t)r * (uint64_t)kSampThreads) % (uint64_t)L.M);
-      A.coef_out[k] = s_merged[u];
-    }
-  }
 }
 
 // prep_terms of the two sums of a pair (f may have no terms).
@@ -1055,17 +1159,8 @@ ss_status prep_terms_pair(const LatticeDev& L, const ss_trig* a, const ss_trig* 
   }
   ProfScope prof_("prep_terms", st);
   PrepArgs A[2];
-  Terms* T[2] = {Ta, Tf};
-  const ss_trig* g[2] = {a, f};
-  for (int i = 0; i < 2; ++i) {
-    const int64_t n = g[i]->n_terms;
-    SS_TRY(T[i]->total.alloc_tmp(1, st));
-    SS_TRY(T[i]->q.alloc_tmp(std::max<int64_t>(n, 1), st));
-    SS_TRY(T[i]->step.alloc_tmp(std::max<int64_t>(n, 1), st));
-    SS_TRY(T[i]->coef.alloc_tmp(std::max<int64_t>(n, 1), st));
-    A[i] = PrepArgs{g[i]->freq, reinterpret_cast<const double2*>(g[i]->coef), n, T[i]->q.get(), T[i]->step.get(),
-                    T[i]->coef.get(), T[i]->total.get()};
-  }
+  SS_TRY(small_args(a, Ta, st, &A[0]));
+  SS_TRY(small_args(f, Tf, st, &A[1]));
   k_prep_terms_small<<<2, 1024, 0, st>>>(A[0], A[1], L);
   SS_LAUNCH_CHECK();
   return SS_OK;
@@ -1231,65 +1326,268 @@ __global__ void k_extract_pr(const int64_t* __restrict__ res, int64_t n, int64_t
   atomicMax(maxbits, (unsigned long long)__double_as_longlong(m));
 }
 
-// Extraction, threshold and compaction of both sums in one launch (block k:
-// sum k) for at most kExtractSmall candidates: the same values, the same
-// threshold tau max|c| and the same candidate order as k_extract_pr, k_keep,
-// the prefix sum and k_compact.
-constexpr int kExtractSmall = 1024;
+// Extraction, threshold and compaction in two launches for at most
+// kExtractSmall candidates: the values bin(i, k) and their moduli (FP64, so
+// spread over the chip), then the threshold tau max|c| and the compaction in
+// candidate order by one block per sum: the same results as k_extract_*,
+// k_keep, the prefix sum and k_compact (ten launches for two sums).
+constexpr int kExtractRounds = 4;
+constexpr int kExtractSmall = 1024 * kExtractRounds;
 
-__global__ void __launch_bounds__(1024) k_extract_keep_pr(const int64_t* __restrict__ res, int64_t n, int64_t M,
-                                                          const float4* __restrict__ X,
-                                                          const double* __restrict__ scale, double tau,
-                                                          const int32_t* __restrict__ cand, int d, int32_t* fo0,
-                                                          double2* vo0, int32_t* fo1, double2* vo1, int64_t* total) {
-  __shared__ double s_max[32];
-  __shared__ int32_t s_wsum[32];
-  __shared__ int32_t s_pos[kExtractSmall];
-  const int k = blockIdx.x;
-  const int i = threadIdx.x, lane = i & 31, w = i >> 5, nw = blockDim.x >> 5;
-  double2 v = make_double2(0.0, 0.0);
-  double m = 0.0;
-  if (i < n) {
+struct BinPr {       // k_extract_pr
+  const float4* X;
+  const double* scale;
+  int64_t M;
+  __device__ double2 operator()(int64_t i, int k) const {
     const float4 xs = X[2 * i], ys = X[2 * i + 1];
     const double xr = (double)xs.x + (double)xs.y, xi = (double)xs.z + (double)xs.w;
     const double yr = (double)ys.x + (double)ys.y, yi = (double)ys.z + (double)ys.w;
-    const double sc = 0.5 / (double)M * scale[k];
-    v = k == 0 ? make_double2((xr + yr) * sc, (xi - yi) * sc) : make_double2((xi + yi) * sc, (yr - xr) * sc);
-    m = hypot(v.x, v.y);
+    const double sc = 0.5 / (double)M * (scale ? scale[k] : 1.0);
+    return k == 0 ? make_double2((xr + yr) * sc, (xi - yi) * sc) : make_double2((xi + yi) * sc, (yr - xr) * sc);
   }
-  double mx = m;
+};
+struct BinFx {       // k_extract_pair
+  const longlong2* Z;
+  const int64_t* res;
+  const double* scale;
+  double unit;
+  int64_t M;
+  __device__ double2 operator()(int64_t i, int k) const {
+    const int64_t b = res[i];
+    const longlong2 x = Z[b], y = Z[b ? M - b : 0];
+    const double2 z = k == 0 ? pair_bin<0>(x, y, scale[2]) : pair_bin<1>(x, y, scale[3]);
+    const double sc = 0.5 / (double)M * unit * scale[k];
+    return make_double2(z.x * sc, z.y * sc);
+  }
+};
+struct BinDirect {   // the parts of k_direct_bins
+  const double2* part;
+  const int64_t* res;
+  int parts;
+  int64_t nb, M;
+  bool by_bin;
+  __device__ double2 operator()(int64_t i, int k) const {
+    const int64_t b = res[i], bb = min(b, M - b);
+    const double2* v = part + (int64_t)k * parts * nb + (by_bin ? bb : i);
+    double re = v->x, im = v->y;
+    for (int p = 1; p < parts; ++p) {
+      re += v[p * nb].x;
+      im += v[p * nb].y;
+    }
+    const double sc = 1.0 / (double)M;
+    if (bb == 0 || 2 * bb == M) im = 0.0;
+    return make_double2(re * sc, (b != bb ? -im : im) * sc);
+  }
+};
+
+template <class Bin>
+__global__ void k_extract_bins(Bin bin, int64_t n, double2* __restrict__ val, double* __restrict__ mag) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = blockIdx.y;
+  if (i >= n) return;
+  const double2 v = bin(i, k);
+  val[k * n + i] = v;
+  mag[k * n + i] = hypot(v.x, v.y);
+}
+
+__global__ void __launch_bounds__(1024) k_keep_compact(const double2* __restrict__ val, const double* __restrict__ mag,
+                                                       int64_t n, double tau, const int32_t* __restrict__ cand, int d,
+                                                       int32_t* fo0, double2* vo0, int32_t* fo1, double2* vo1,
+                                                       int64_t* total) {
+  __shared__ unsigned long long s_max[32];
+  __shared__ int32_t s_wsum[kExtractRounds][32];
+  __shared__ int32_t s_pos[kExtractSmall];
+  const int k = blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const double2* v = val + k * n;
+  double m[kExtractRounds];
+  unsigned long long mx = 0;   // moduli order like their bits, a NaN above all
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int r = 0; r < kExtractRounds; ++r) {
+    const int64_t i = r * 1024 + threadIdx.x;
+    m[r] = i < n ? mag[k * n + i] : 0.0;
+    mx = max(mx, (unsigned long long)__double_as_longlong(m[r]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) s_max[w] = mx;
   __syncthreads();
-  mx = 0.0;
-  for (int q = 0; q < nw; ++q) mx = fmax(mx, s_max[q]);
-  const int keep = (i < n && m > tau * mx) ? 1 : 0;
-  int x = keep;
+  for (int q = 0; q < nw; ++q) mx = max(mx, s_max[q]);
+  const double thr = tau * __longlong_as_double((long long)mx);
+  int x[kExtractRounds];
+  bool keep[kExtractRounds];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+  for (int r = 0; r < kExtractRounds; ++r) {
+    keep[r] = r * 1024 + threadIdx.x < n && m[r] > thr;
+    const unsigned b = __ballot_sync(0xffffffffu, keep[r]);
+    x[r] = __popc(b & ((1u << lane) - 1u));
+    if (lane == 0) s_wsum[r][w] = __popc(b);
   }
-  if (lane == 31) s_wsum[w] = x;
   __syncthreads();
-  int before = 0, tot = 0;
-  for (int q = 0; q < nw; ++q) {
-    if (q < w) before += s_wsum[q];
-    tot += s_wsum[q];
-  }
-  if (i == 0) total[k] = tot;
   int32_t* fo = k == 0 ? fo0 : fo1;
   double2* vo = k == 0 ? vo0 : vo1;
-  if (i < n) s_pos[i] = keep ? before + x - 1 : -1;
-  if (keep) vo[before + x - 1] = v;
+  int tot = 0;
+#pragma unroll
+  for (int r = 0; r < kExtractRounds; ++r) {
+    if (r * 1024 >= n) break;
+    int before = tot;
+    for (int q = 0; q < nw; ++q) {
+      if (q < w) before += s_wsum[r][q];
+      tot += s_wsum[r][q];
+    }
+    const int i = r * 1024 + threadIdx.x;
+    if (i < n) s_pos[i] = keep[r] ? before + x[r] : -1;
+    if (keep[r]) vo[before + x[r]] = v[i];
+  }
+  if (threadIdx.x == 0) total[k] = tot;
   __syncthreads();
-  // the kept frequencies, one warp per row (coalesced coordinates)
-  for (int u = w; u < n; u += nw) {
+  // the kept frequencies: a group of G lanes per row
+  int G = 1;
+  while (G < 32 && G < d) G *= 2;
+  for (int u = threadIdx.x / G; u < n; u += 1024 / G) {
     const int p = s_pos[u];
     if (p < 0) continue;
-    for (int c = lane; c < d; c += 32) fo[(int64_t)p * d + c] = cand[(int64_t)u * d + c];
+    for (int c = threadIdx.x & (G - 1); c < d; c += G) fo[(int64_t)p * d + c] = cand[(int64_t)u * d + c];
   }
+}
+
+template <class Bin>
+ss_status extract_keep(const Bin& bin, int sums, int64_t n, double tau, const int32_t* cand, int d, int32_t* const fo[2],
+                       double* const vo[2], int64_t* total, cudaStream_t st) {
+  ProfScope prof_("extract", st);
+  DevBuf<double2> val;
+  DevBuf<double> mag;
+  SS_TRY(val.alloc_tmp(sums * n, st));
+  SS_TRY(mag.alloc_tmp(sums * n, st));
+  k_extract_bins<Bin><<<dim3(nblk(n, 64), sums), 64, 0, st>>>(bin, n, val.get(), mag.get());
+  k_keep_compact<<<sums, 1024, 0, st>>>(val.get(), mag.get(), n, tau, cand, d, fo[0],
+                                        reinterpret_cast<double2*>(vo[0]), fo[sums - 1],
+                                        reinterpret_cast<double2*>(vo[sums - 1]), total);
+  SS_LAUNCH_CHECK();
+  return SS_OK;
+}
+
+// ----------------------------------------------------- small lattices, direct
+//
+// A short M that is not 7-smooth: the samples of both sums straight from their
+// merged terms and the bins straight from the samples, in FP64 with a table of
+// the M roots.  M = 24,500, 35 candidates: 22 us for both sums; M = 1089 with as
+// many candidates: 15 us.  cuFFT's transforms (Bluestein; M = 1089: radix 11)
+// take 140 us and 68 us for each sum, the double-float sampling before them 20
+// to 35 us.  FP64 issue bounds the bins
+// (4 multiply-adds per node and candidate, 304 a clock): kDirectMaxWork is
+// 30 us of them, below one such transform.
+// Both split their sums over warps or threads and add the parts in a fixed order.
+
+// x mod M for x < 2^30, M < 2^15 (inv = floor((2^32 - 1) / M))
+__device__ __forceinline__ uint32_t small_mod(uint32_t x, uint32_t M, uint32_t inv) {
+  uint32_t r = x - __umulhi(x, inv) * M;
+  r = r >= M ? r - M : r;
+  return r >= M ? r - M : r;
+}
+
+constexpr int kDirectWarps = 16;
+
+// out[y][j] = sum_t Re(c_t exp(2 pi i j q_t / M)) of sum y = blockIdx.y; a lane
+// per node, the terms dealt out to the warps.
+__global__ void __launch_bounds__(32 * kDirectWarps) k_direct_sample(
+    const int64_t* __restrict__ qa, const double2* __restrict__ ca, const int64_t* __restrict__ na_dev,
+    const int64_t* __restrict__ qf, const double2* __restrict__ cf, const int64_t* __restrict__ nf_dev, int M,
+    const double2* __restrict__ roots, double* __restrict__ out) {
+  __shared__ double s_part[kDirectWarps][32];
+  const bool f = blockIdx.y != 0;
+  const int64_t* q = f ? qf : qa;
+  const double2* c = f ? cf : ca;
+  const int n = (int)*(f ? nf_dev : na_dev);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t j = blockIdx.x * 32 + lane, inv = 0xffffffffu / (uint32_t)M;
+  double acc = 0.0;
+  if (j < (uint32_t)M) {
+#pragma unroll 4
+    for (int t = w; t < n; t += kDirectWarps) {
+      const double2 e = __ldg(roots + small_mod(j * (uint32_t)__ldg(q + t), (uint32_t)M, inv)), k = __ldg(c + t);
+      acc = fma(k.x, e.x, fma(-k.y, e.y, acc));
+    }
+  }
+  s_part[w][lane] = acc;
+  __syncthreads();
+  if (w || j >= (uint32_t)M) return;
+#pragma unroll
+  for (int i = 1; i < kDirectWarps; ++i) acc += s_part[i][lane];
+  out[(int64_t)blockIdx.y * M + j] = acc;
+}
+
+// part[y][p][i] = sum_j s_y[j] exp(-2 pi i j b / M) over the p-th of gridDim.y
+// ranges of nodes, for both sums y (sums: 1 or 2); b = min(r, M - r) with r the
+// residue of candidate i, or the bin i itself (res null).
+constexpr int kDirectThreads = 128;
+__global__ void __launch_bounds__(kDirectThreads) k_direct_bins(const double* __restrict__ s, int sums, int M,
+                                                                const int64_t* __restrict__ res, int64_t nb,
+                                                                const double2* __restrict__ roots,
+                                                                double2* __restrict__ part) {
+  __shared__ double s_part[kDirectThreads / 32][4];
+  const int64_t i = blockIdx.x;
+  const uint32_t r = res ? (uint32_t)res[i] : (uint32_t)i, b = min(r, (uint32_t)M - r), inv = 0xffffffffu / (uint32_t)M;
+  const uint32_t len = ((uint32_t)M + gridDim.y - 1) / gridDim.y, j0 = blockIdx.y * len, j1 = min(j0 + len, (uint32_t)M);
+  const double* s1 = s + (sums > 1 ? M : 0);
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (uint32_t j = j0 + threadIdx.x; j < j1; j += kDirectThreads) {
+    const double2 e = __ldg(roots + small_mod(j * b, (uint32_t)M, inv));
+    const double x = __ldg(s + j), y = __ldg(s1 + j);
+    v[0] = fma(x, e.x, v[0]);
+    v[1] = fma(-x, e.y, v[1]);
+    v[2] = fma(y, e.x, v[2]);
+    v[3] = fma(-y, e.y, v[3]);
+  }
+  // butterfly in which half of the values leave at each of the first two steps
+  const int lane = threadIdx.x & 31;
+  const double k0 = lane & 16 ? v[2] : v[0], k1 = lane & 16 ? v[3] : v[1];
+  double a0 = k0 + __shfl_xor_sync(0xffffffffu, lane & 16 ? v[0] : v[2], 16);
+  double a1 = k1 + __shfl_xor_sync(0xffffffffu, lane & 16 ? v[1] : v[3], 16);
+  double a = (lane & 8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, lane & 8 ? a0 : a1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if ((lane & 7) == 0) s_part[threadIdx.x >> 5][lane >> 3] = a;   // re, im of sum 0, then of sum 1
+  __syncthreads();
+  if (threadIdx.x >= (unsigned)sums) return;
+  const int y = threadIdx.x;
+  double re = 0.0, im = 0.0;
+#pragma unroll
+  for (int w = 0; w < kDirectThreads / 32; ++w) {
+    re += s_part[w][2 * y];
+    im += s_part[w][2 * y + 1];
+  }
+  part[((int64_t)y * gridDim.y + blockIdx.y) * nb + i] = make_double2(re, im);
+}
+
+bool use_direct(const SftPlan& P, int64_t n_terms, int64_t n_cand) {
+  return P.roots.get() && P.M * std::max(n_terms, n_cand) <= kDirectMaxWork && n_cand <= kExtractSmall;
+}
+
+// Both sums (f null: one) through extract_keep.  More candidates than bins up
+// to M/2: every bin once, else every candidate's; the nodes are split over
+// blocks where the bins alone leave SMs idle.
+ss_status direct_recover_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* a, const ss_trig* f,
+                              const int64_t* res, const int32_t* cand, int64_t n_cand, double tau,
+                              int32_t* const fo[2], double* const vo[2], int64_t* total, cudaStream_t st) {
+  const int sums = f ? 2 : 1, M = (int)P.M;
+  Terms ta, tf;
+  if (f) SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
+  else SS_TRY(prep_terms(L, a, &ta, st));
+  const bool by_bin = n_cand > M / 2 + 1;
+  const int64_t nb = by_bin ? M / 2 + 1 : n_cand;
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(4LL * sm_count() / nb, M / (4 * kDirectThreads)));
+  DevBuf<double> s;
+  DevBuf<double2> part;
+  SS_TRY(s.alloc_tmp((size_t)sums * M, st));
+  SS_TRY(part.alloc_tmp((size_t)sums * parts * nb, st));
+  k_direct_sample<<<dim3((M + 31) / 32, sums), 32 * kDirectWarps, 0, st>>>(
+      ta.q.get(), ta.coef.get(), ta.total.get(), tf.q.get(), tf.coef.get(), tf.total.get(), M, P.roots.get(), s.get());
+  k_direct_bins<<<dim3((unsigned)nb, parts), kDirectThreads, 0, st>>>(s.get(), sums, M, by_bin ? nullptr : res, nb,
+                                                                      P.roots.get(), part.get());
+  SS_LAUNCH_CHECK();
+  return extract_keep(BinDirect{part.get(), res, parts, nb, M, by_bin}, sums, n_cand, tau, cand, L.d, fo, vo, total, st);
 }
 
 // Pruned forward transform of s (P.prz, or the caller's real samples) at
@@ -1312,9 +1610,10 @@ ss_status pr_transform(const SftPlan& P, const void* s, bool real, const int64_t
 // sum, as left by fx_recover_pair) instead of a transform of samples.
 // pr != 0: the pruned forward transform of P.prz (pr = 1: complex samples of
 // one sum, scale P.prscale) or of the real FP64 samples (pr = 2).
+// direct non-null: that sum by direct_recover_pair.
 ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* samples, const int32_t* cand, int64_t n_cand,
                        int64_t s_max, double tau, int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st,
-                       const longlong2* zh = nullptr, int pr = 0) {
+                       const longlong2* zh = nullptr, int pr = 0, const ss_trig* direct = nullptr) {
   DevBuf<int64_t> res, total;
   DevBuf<unsigned long long> table, maxbits;
   DevBuf<int32_t> flags, flag, pos;
@@ -1337,7 +1636,7 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
   if (pr) {
     SS_TRY(X.alloc_tmp(2 * n_cand, st));
     SS_TRY(pr_transform(P, pr == 1 ? (const void*)P.prz.get() : samples, pr == 2, res.get(), n_cand, X.get(), st));
-  } else if (!zh) {
+  } else if (!zh && !direct) {
     cufftResult r = cufftSetStream(P.fft, st);
     if (r != CUFFT_SUCCESS) SS_FAIL(SS_ERR_CUDA, "cufftSetStream failed: %d", (int)r);
     if (P.prec == SS_FP64)
@@ -1348,25 +1647,37 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
                        reinterpret_cast<cufftComplex*>(P.spectrum.get()));
     if (r != CUFFT_SUCCESS) SS_FAIL(SS_ERR_CUDA, "cuFFT exec failed: %d", (int)r);
   }
-  SS_CUDA(cudaMemsetAsync(maxbits.get(), 0, sizeof(unsigned long long), st));
-  if (pr)
-    k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), pr == 1 ? P.prscale.get() : nullptr,
-                                                  val.get(), mag.get(), maxbits.get());
-  else if (zh)
-    k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, fx_unit(P), P.fxscale.get(), val.get(),
-                                                    mag.get(), maxbits.get());
-  else if (P.prec == SS_FP64)
-    k_extract<double2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const double2*>(P.spectrum.get()),
-                                                     val.get(), mag.get(), maxbits.get());
-  else
-    k_extract<float2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const float2*>(P.spectrum.get()),
+  int32_t* const fo[2] = {freq_out, freq_out};
+  double* const vo[2] = {val_out, val_out};
+  if (direct) {
+    SS_TRY(direct_recover_pair(P, L, direct, nullptr, res.get(), cand, n_cand, tau, fo, vo, total.get(), st));
+  } else if (pr && n_cand <= kExtractSmall) {
+    SS_TRY(extract_keep(BinPr{X.get(), pr == 1 ? P.prscale.get() : nullptr, L.M}, 1, n_cand, tau, cand, L.d, fo, vo,
+                        total.get(), st));
+  } else if (zh && n_cand <= kExtractSmall) {
+    SS_TRY(extract_keep(BinFx{zh, res.get(), P.fxscale.get(), fx_unit(P), L.M}, 1, n_cand, tau, cand, L.d, fo, vo,
+                        total.get(), st));
+  } else {
+    SS_CUDA(cudaMemsetAsync(maxbits.get(), 0, sizeof(unsigned long long), st));
+    if (pr)
+      k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), pr == 1 ? P.prscale.get() : nullptr,
                                                     val.get(), mag.get(), maxbits.get());
-  k_keep<<<nblk(n_cand), 256, 0, st>>>(mag.get(), n_cand, maxbits.get(), tau, flag.get());
-  SS_LAUNCH_CHECK();
-  SS_TRY(exclusive_scan_i32(flag.get(), pos.get(), n_cand, total.get(), st));
-  k_compact<<<nblk(n_cand), 256, 0, st>>>(cand, val.get(), n_cand, L.d, flag.get(), pos.get(), freq_out,
-                                          reinterpret_cast<double2*>(val_out));
-  SS_LAUNCH_CHECK();
+    else if (zh)
+      k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, fx_unit(P), P.fxscale.get(), val.get(),
+                                                      mag.get(), maxbits.get());
+    else if (P.prec == SS_FP64)
+      k_extract<double2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const double2*>(P.spectrum.get()),
+                                                       val.get(), mag.get(), maxbits.get());
+    else
+      k_extract<float2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const float2*>(P.spectrum.get()),
+                                                      val.get(), mag.get(), maxbits.get());
+    k_keep<<<nblk(n_cand), 256, 0, st>>>(mag.get(), n_cand, maxbits.get(), tau, flag.get());
+    SS_LAUNCH_CHECK();
+    SS_TRY(exclusive_scan_i32(flag.get(), pos.get(), n_cand, total.get(), st));
+    k_compact<<<nblk(n_cand), 256, 0, st>>>(cand, val.get(), n_cand, L.d, flag.get(), pos.get(), freq_out,
+                                            reinterpret_cast<double2*>(val_out));
+    SS_LAUNCH_CHECK();
+  }
   int64_t kept = 0;
   int32_t hf[4];
   SS_TRY(read_back(st, {{&kept, total.get(), sizeof(int64_t)}, {hf, flags.get(), sizeof(hf)}}));
@@ -1798,13 +2109,8 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
     DevBuf<float4> X;
     SS_TRY(X.alloc_tmp(2 * n_cand, st));
     SS_TRY(pr_transform(P, P.prz.get(), false, res.get(), n_cand, X.get(), st));
-    if (n_cand <= kExtractSmall) {
-      ProfScope prof_("extract", st);
-      k_extract_keep_pr<<<2, 1024, 0, st>>>(res.get(), n_cand, L.M, X.get(), P.prscale.get(), tau, cand, L.d,
-                                           fo[0], reinterpret_cast<double2*>(vo[0]), fo[1],
-                                           reinterpret_cast<double2*>(vo[1]), total.get());
-      SS_LAUNCH_CHECK();
-    }
+    if (n_cand <= kExtractSmall)
+      SS_TRY(extract_keep(BinPr{X.get(), P.prscale.get(), L.M}, 2, n_cand, tau, cand, L.d, fo, vo, total.get(), st));
     for (int k = 0; k < 2 && n_cand > kExtractSmall; ++k) {
       if (k == 0)
         k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), P.prscale.get(), val.get(),
@@ -1826,7 +2132,10 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
     SS_TRY(fx_recover_pair(P, L, a, f, st));
     const longlong2* Z = P.fxz.get();
     const double un = fx_unit(P);
-    for (int k = 0; k < 2; ++k) {
+    if (n_cand <= kExtractSmall)
+      SS_TRY(extract_keep(BinFx{Z, res.get(), P.fxscale.get(), un, L.M}, 2, n_cand, tau, cand, L.d, fo, vo, total.get(),
+                          st));
+    for (int k = 0; k < 2 && n_cand > kExtractSmall; ++k) {
       if (k == 0)
         k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, un, P.fxscale.get(), val.get(), mag.get(),
                                                         maxbits.get());
@@ -1841,6 +2150,8 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
       SS_LAUNCH_CHECK();
     }
   }
+  const bool direct = use_direct(P, a->n_terms + f->n_terms, n_cand);
+  if (direct) SS_TRY(direct_recover_pair(P, L, a, f, res.get(), cand, n_cand, tau, fo, vo, total.get(), st));
   if (!P.has_fx && !P.has_pr && use_pair32(P)) {
     SS_TRY(ensure_pair32(P, st));
     SS_TRY(sample_into(P, L, a, P.samples.get(), st));
@@ -1871,7 +2182,7 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
       SS_LAUNCH_CHECK();
     }
   }
-  for (int k = 0; k < 2 && !P.has_fx && !P.has_pr && !use_pair32(P); ++k) {
+  for (int k = 0; k < 2 && !direct && !P.has_fx && !P.has_pr && !use_pair32(P); ++k) {
     // the plan's sample and spectrum buffers serve both sums in stream order
     SS_TRY(sample_into(P, L, g[k], P.samples.get(), st));
     if (P.prec == SS_FP64)
@@ -1955,6 +2266,8 @@ extern "C" ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_pre
     SS_TRY(fx_recover_pair(*P, L, g, nullptr, st));
     return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, P->fxz.get());
   }
+  if (use_direct(*P, g->n_terms, n_cand))
+    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, nullptr, 0, g);
   if (P->has_pr) {
     SS_TRY(pr_sample_pair(*P, L, g, nullptr, st));
     return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, nullptr, 1);
