@@ -124,6 +124,46 @@ __device__ __forceinline__ double2 row_apply64(const OpView& op, int64_t s, int 
                   : row_apply64_t<CG, false, SKIP>(op, s, lane, rec, self);
 }
 
+// The same on an array u of n values, taken as zero from n on (padding entries
+// name column rows_pad, one past any row of u; a prefix of the rows may be
+// given alone): nothing is packed first.  U entries are in flight per thread;
+// the products are added in the order of row_apply64_t.
+template <bool REAL, int U>
+__device__ __forceinline__ double2 row_apply64_direct(const OpView& op, int64_t s, int lane, int64_t n,
+                                                      const double2* __restrict__ u) {
+  const int32_t w0 = __ldg(op.woff + s), w1 = __ldg(op.woff + s + 1);
+  const int64_t base = (int64_t)w0 * kSlice + lane;
+  const uint32_t* e = op.ent + base;
+  const double2* cf = op.ecoef + base;
+  const double* cfr = reinterpret_cast<const double*>(op.ecoef) + base;
+  double ar = 0.0, ai = 0.0;
+  const int w = w1 - w0;
+  for (int t = 0; t < w; t += U) {
+    uint32_t col[U];
+    double2 c[U], v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const bool in = t + q < w;
+      col[q] = in ? __ldg(e + (int64_t)(t + q) * kSlice) & op.colmask : 0xffffffffu;
+      if constexpr (REAL) c[q] = make_double2(in ? __ldg(cfr + (int64_t)(t + q) * kSlice) : 0.0, 0.0);
+      else c[q] = in ? __ldg(cf + (int64_t)(t + q) * kSlice) : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) v[q] = (int64_t)col[q] < n ? __ldg(u + col[q]) : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      if (t + q >= w) break;
+      ar = fma(c[q].x, v[q].x, ar);
+      ai = fma(c[q].x, v[q].y, ai);
+      if constexpr (!REAL) {
+        ar = fma(-c[q].y, v[q].y, ar);
+        ai = fma(c[q].y, v[q].x, ai);
+      }
+    }
+  }
+  return make_double2(ar, ai);
+}
+
 // Same in FP32 (FP32 values, FP32 accumulation).  nk, the records' third
 // word and pn are FP32 norm words (norm_word): int32 norms, or FP32 values
 // when WIDE.

@@ -371,9 +371,8 @@ extern "C" ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, c
     SS_LAUNCH_CHECK();
   }
   if (n_g > 0) {
-    SS_TRY(launch_pack64_prefix(s, reinterpret_cast<const double2*>(u_prefix), n_u, st));
     SS_TRY(y.alloc(s->size, st));
-    SS_TRY(launch_apply64(s, y.get(), st));
+    SS_TRY(launch_apply64(s, reinterpret_cast<const double2*>(u_prefix), n_u, y.get(), st));
     // (L u)_0 = 0 exactly for the diffusion operator (the factor k.l); its
     // stored identity row is for the solve
     if (identity_row(s) >= 0) SS_CUDA(cudaMemsetAsync(y.get() + identity_row(s), 0, sizeof(double2), st));

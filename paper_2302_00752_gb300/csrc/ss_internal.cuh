@@ -254,7 +254,7 @@ struct ss_stamp_s {
   ss::DevBuf<float4> ecoefdf;         // [n_ent + 1] the same as double-float, built on first DF64 solve
   ss::DevBuf<int32_t> nw32;           // [rows_pad + 1] FP32 norm words of |k|^2 (norm_word; 0 on padding)
   // scratch for galerkin_apply (FP64)
-  ss::DevBuf<double2> rec64;          // [rows_pad + 1] FP64 values gathered by the FP64 operator
+  ss::DevBuf<double2> rec64;          // [rows_pad + 1] scratch of the FP64 operator in place
   // build state kept for stamp_extend
   int maxabs_f = 0, maxabs_a = 0;     // largest |coordinate| of F and of supp a_hat
   // operator of Remark ADR (advection b.grad u and reaction c u added; not
@@ -311,11 +311,9 @@ __host__ __device__ inline uint32_t colmask_of(int jbits) { return (jbits >= 32)
 __host__ __device__ inline int colbits_of(int jbits) { return 32 - jbits; }
 
 // Apply launchers used by galerkin_apply and the solver (apply.cu).
-ss_status launch_pack64(const ss_stamp_s* s, const double2* u, cudaStream_t st);
-ss_status launch_apply64(const ss_stamp_s* s, double2* y, cudaStream_t st);
-// u on the first n_u rows of S (a vector on S^N is the prefix of one on
-// S^{N+L}), zero on the rest, into the FP64 record array.
-ss_status launch_pack64_prefix(const ss_stamp_s* s, const double2* u, int64_t n_u, cudaStream_t st);
+// y = L u, u on the first n_u rows of S (a vector on S^N is the prefix of one on
+// S^{N+L}), zero on the rest.  u and y may be the same array.
+ss_status launch_apply64(const ss_stamp_s* s, const double2* u, int64_t n_u, double2* y, cudaStream_t st);
 // FP32 operator straight from the caller's u (no packing step).
 ss_status launch_apply32(const ss_stamp_s* s, const float2* u, float2* y, cudaStream_t st);
 // Double-float copy of the FP64 entry coefficients (built once per operator).

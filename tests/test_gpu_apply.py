@@ -85,3 +85,19 @@ def test_full_size_sampled_rows(B, name, rows):
     assert rel_l2(y32[pick], ref) <= TOL32
     lhs, rhs = np.vdot(v, y64), np.vdot(Lv, u)
     assert abs(lhs - rhs) <= 1e-12 * abs(lhs)
+
+
+@pytest.mark.parametrize("d,N", [(2, 1), (3, 3), (6, 2)])
+def test_in_place(B, d, N):
+    # y = u, and y overlapping u by half: the values are those of separate arrays
+    inst = W.make_tiny(d, d=d, n_cos=3, n_u=3, N=N)
+    _, af, av, ff, _ = stamp_inputs(inst)
+    with B.stamp_build(af, av, ff, N) as s:
+        n = s.size
+        u = torch.as_tensor(rand_u(n, d)).cuda()
+        want = B.galerkin_apply(s, u)
+        for shift in (0, n // 2):
+            buf = torch.zeros(n + shift, dtype=torch.complex128, device="cuda")
+            buf[shift:] = u
+            B._check(B.lib.galerkin_apply(s.handle, B._ptr(buf[shift:]), B._ptr(buf), B.SS_FP64, B._stream()))
+            assert torch.equal(buf[:n], want)
