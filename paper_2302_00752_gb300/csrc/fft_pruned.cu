@@ -486,6 +486,103 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
   }
 }
 
+// FP32 evaluation with P = 16 or 32: a thread holds a whole column in registers,
+// so the length-P transform (radix 8, then P / 8) needs neither shared memory
+// nor index arithmetic, and writes its P samples (a warp: 32 neighbours of each
+// p).  The tiles of W columns, their entries and every operation are
+// k_pr_eval's, in its order: the same samples bit for bit.  256 / W tiles per
+// block at once, the base values of kPrColRounds rounds of them together (their
+// table reads overlap).
+// M = 2^26, 42 entries, P = 32: 370 us by k_pr_eval (integer and shared-memory
+// issue: 130 instructions a sample), 216 us so (latency of the entry loops at 16
+// warps an SM; 24 warps spill); the 537 MB of samples take 79.
+constexpr int kPrColEntries = 128;   // step powers in shared memory (64 KB at W = 64)
+constexpr int kPrColRounds = 4;
+
+__host__ __device__ constexpr bool pr_col_supported(int P) { return P == 16 || P == 32; }
+
+template <int P, bool OUT_REAL>
+__global__ void __launch_bounds__(kPrThreads, 2) k_pr_eval_col(int64_t M, int64_t Q, const float4* __restrict__ t0,
+                                                               const float4* __restrict__ t1, int b,
+                                                               const int64_t* __restrict__ er,
+                                                               const float4* __restrict__ ev,
+                                                               const int32_t* __restrict__ boff_g,
+                                                               const float4* __restrict__ estep, int n_stage,
+                                                               int64_t n_tiles, void* __restrict__ out) {
+  using A = ArF32;
+  constexpr int W = kPrEvalTile / P, SUB = kPrThreads / W, R2 = P / 8;
+  static_assert(W <= kPrThreads, "a tile within a block");
+  extern __shared__ __align__(16) float4 sm4[];
+  float2* tw = reinterpret_cast<float2*>(sm4);
+  float2* es = tw + P;                              // [ne][W]
+  float2* base = es + n_stage;                      // [kPrColRounds][SUB][ne]
+  __shared__ int32_t boff[P + 1];
+  const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
+  for (int m = threadIdx.x; m < P; m += blockDim.x) tw[m] = A::root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q);
+  for (int k = threadIdx.x; k <= P; k += blockDim.x) boff[k] = boff_g[k];
+  __syncthreads();
+  const int ne = boff[P];
+  for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::from_df(__ldg(estep + x));
+  const float2 cs[1] = {tw[P / 8]};
+  const int sub = threadIdx.x / W, i = threadIdx.x % W;
+  // the block's tiles: SUB neighbours a round, the rounds gridDim.x SUB tiles apart
+  const int64_t stride = (int64_t)gridDim.x * SUB;
+  for (int64_t first = (int64_t)blockIdx.x * SUB; first < n_tiles; first += kPrColRounds * stride) {
+    __syncthreads();   // the last rounds' values are read
+#pragma unroll 4
+    for (int x = threadIdx.x; x < kPrColRounds * SUB * ne; x += blockDim.x) {
+      const int t = x / ne, e = x - t * ne;   // tile t % SUB of round t / SUB
+      const uint64_t q0 = (uint64_t)min(first + (t / SUB) * stride + t % SUB, n_tiles - 1) * W;
+      base[x] = A::mul(A::from_df(__ldg(ev + e)), A::root<1>(t0, t1, b, mulmod(q0, (uint64_t)er[e], Mu, inv)));
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int rnd = 0; rnd < kPrColRounds && first + rnd * stride < n_tiles; ++rnd) {
+      const int64_t tile0 = first + rnd * stride;
+      const float2* bs = base + (rnd * SUB + sub) * ne;
+      const float2* ei = es + i;
+      // every bucket's first entry without a branch (its reads overlap), the others after it
+      float2 c[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        const int lo = boff[k], e = max(0, min(lo, ne - 1));
+        const float2 x = A::add(A::zero(), A::mul(bs[e], ei[e * W]));
+        c[k] = lo < boff[k + 1] ? x : A::zero();
+      }
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        const int hi = boff[k + 1];
+        for (int e = boff[k] + 1; e < hi; ++e) c[k] = A::add(c[k], A::mul(bs[e], ei[e * W]));
+      }
+      // radix 8: butterfly j takes j + r P / 8, output r goes to 8 j + r
+#pragma unroll
+      for (int j = 0; j < R2; ++j) {
+        float2 v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = c[j + r * R2];
+        A::dft<8, 1>(v, cs);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) c[j + r * R2] = v[r];   // position 8 j + r
+      }
+      // radix P / 8: butterfly k takes k + 8 r (butterfly r's output k), output r is the sample k + 8 r
+      const int64_t q = (tile0 + sub) * W + i;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        float2 v[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) v[r] = r && k ? A::mul(c[r + k * R2], tw[k * r]) : c[r + k * R2];
+        A::dft<R2, 1>(v, nullptr);
+        if (q >= Q) continue;
+#pragma unroll
+        for (int r = 0; r < R2; ++r) {
+          if (OUT_REAL) static_cast<float*>(out)[q + Q * (k + 8 * r)] = A::real_out(v[r]);
+          else static_cast<float2*>(out)[q + Q * (k + 8 * r)] = v[r];
+        }
+      }
+    }
+  }
+}
+
 // Pruned forward transform: per tile the length-P transforms of the W
 // columns, then every output o accumulates
 //   w^{-q0 b_o} sum_i Y[b_o mod P][q0 + i] z_o^i,   z_o = w^{-b_o},
@@ -833,6 +930,20 @@ ss_status launch_eval16_p(const TwoLevelTable& T, const PrunedSplit& S, const in
   return launch_eval16<A, 128, OUT_REAL>(T, S, er, ev, boff, estep, n_stage, out, st);
 }
 
+template <int P, bool OUT_REAL>
+ss_status launch_eval_col(const TwoLevelTable& T, const PrunedSplit& S, int64_t ne_max, const int64_t* er,
+                          const float4* ev, const int32_t* boff, const float4* estep, void* out, cudaStream_t st) {
+  constexpr int W = kPrEvalTile / P, SUB = kPrThreads / W;
+  const int64_t n_tiles = (S.Q + W - 1) / W;
+  const size_t smem = (size_t)(P + ne_max * W + kPrColRounds * SUB * ne_max) * sizeof(float2);
+  int grid = 0;
+  SS_TRY(grid_for(k_pr_eval_col<P, OUT_REAL>, smem, (n_tiles + SUB - 1) / SUB, &grid));
+  k_pr_eval_col<P, OUT_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.Q, T.t0.get(), T.t1.get(), T.b, er, ev, boff, estep,
+                                                            (int)(ne_max * W), n_tiles, out);
+  SS_LAUNCH_CHECK();
+  return SS_OK;
+}
+
 template <class A, int P, bool IN_REAL>
 ss_status launch_fwd16(const TwoLevelTable& T, const PrunedSplit& S, const void* in, const int64_t* ob,
                        const int32_t* kout, int nc, const float4* oz, float4* X, cudaStream_t st) {
@@ -978,6 +1089,15 @@ ss_status pruned_eval_pair(const TwoLevelTable& T, const int64_t* qa, const doub
       default:
         return launch_eval16_p<ArF32, true>(T, S, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
     }
+  }
+  // FP32, P = 16 or 32, the step powers within shared memory: a column per
+  // thread.  (FP64: a column of double-floats does not fit the registers.)
+  const bool f32 = fmt == PrunedFormat::kF32Complex || fmt == PrunedFormat::kF32Real;
+  if (f32 && pr_col_supported(S.P) && ne_max <= kPrColEntries && S.W == kPrEvalTile / S.P) {
+    const bool real = fmt == PrunedFormat::kF32Real;
+    auto go = [&](auto launch) { return launch(T, S, ne_max, er.get(), ev.get(), boff.get(), estep.get(), out, st); };
+    if (S.P == 16) return real ? go(launch_eval_col<16, true>) : go(launch_eval_col<16, false>);
+    return real ? go(launch_eval_col<32, true>) : go(launch_eval_col<32, false>);
   }
   switch (fmt) {
     case PrunedFormat::kDfComplex:

@@ -200,3 +200,21 @@ def test_cfg5_fp32_pair_recovery(B):
     assert rel_l2(r.u.cpu().numpy(), staged.u.cpu().numpy()) <= 1e-5
     r.stamp.destroy()
     staged.stamp.destroy()
+
+
+@pytest.mark.parametrize("M", [2**23, 2**17 * 3**4, 2**5 * 7**7])
+@pytest.mark.parametrize("n_terms", [1, 10, 24, 60])
+def test_fp32_samples_by_columns(B, M, n_terms):
+    # FP32 samples (P = 16 or 32: a column per thread; other P beside them) against the FP64
+    # ones, at the ends, the tile edges and random nodes.  A sample sums 2 n products of two
+    # roots (each an FP32 product of two) and passes two radix stages with one more root:
+    # about 2^-24 sum |c| (log2 M + 12)
+    freq, coef, _, z = _instance(M, max(n_terms, 3), 7)
+    freq, coef = freq[:n_terms], coef[:n_terms]
+    s32 = B.lattice_sample(z, M, freq, coef, "fp32").cpu().numpy()
+    s64 = B.lattice_sample(z, M, freq, coef, "fp64").cpu().numpy()
+    rel = np.abs(s32 - s64).max() / np.abs(coef).sum()
+    assert rel <= 2.0**-24 * (np.log2(M) + 12)
+    if n_terms == 1:   # no terms at all: an empty spectrum
+        f, _ = B.sft_recover(z, M, freq[:0], coef[:0], np.array([[0, 0, 0], [1, 2, 3], [-1, -2, -3]]), precision="fp32")
+        assert len(f) == 0
