@@ -1,19 +1,28 @@
 // Pruned DFTs of a 7-smooth length M (the split, the index maps and the cost
-// are stated in fft_pruned.cuh), in double-float arithmetic (the FP64
-// recovery) or in FP32 (the FP32 recovery).
+// are stated in fft_pruned.cuh): in 64-bit fixed point (the FP64 recovery of
+// two sums), in double-float (FP64 real samples) or in FP32 (the FP32 recovery).
 //
 // Inside a block a tile holds W columns of length P in shared memory, column c
 // at c (P + 1) (one element of padding: threads that share a row offset and
 // differ in the column hit distinct banks).  The length-P transforms run as
 // self-sorting (Stockham) radix passes over all W columns at once, thread u
 // taking column u mod W, butterfly u / W, with the P-th roots staged in
-// shared memory.  The arithmetic is a policy (ArDF: complex double-float
-// values as float4 and the butterflies of dfc.cuh; ArF32: float2).  All sums
-// run in a fixed order, so results are bit-reproducible.
+// shared memory.  The arithmetic is a policy (ArFX: fixed point, longlong2, the
+// butterflies of fxc.cuh; ArDF: complex double-float values as float4, those of
+// dfc.cuh; ArF32: float2).  All sums run in a fixed order, so results are
+// bit-reproducible.
+//
+// Fixed point against double-float, M = 2^26, d = 100 (142 entries, 282 bins):
+// evaluation 654 us, 757; forward 621 us, 774.  An addition takes 2
+// instructions against 8 to 20, a product 14 to 26 against 50, and the rounding
+// of a sample is 2^-55 of the l1 norm instead of 2^-47 of the values.  Bound:
+// issue and latency at 16 warps an SM, the most that the registers of a radix-16
+// butterfly leave (24 warps spill: 665, 684).
 #include <algorithm>
 #include <cmath>
 
 #include "dfc.cuh"
+#include "fxc.cuh"
 #include "fft_pruned.cuh"
 
 namespace ss {
@@ -178,28 +187,42 @@ __device__ __forceinline__ void dft16(C4 (&v)[16], const C4 w1, const C4 w2, con
 struct ArDF {
   using V = float4;
   using C = C4;
+  using TV = float4;   // roots, stored and as operands
+  using T = C4;
+  using AccV = float4; // the outputs' sums over the tiles
+  using Acc = C4;
+  static constexpr bool kFixed = false;
   static constexpr int kMinBlocks16 = 2;   // resident blocks per SM of the 4096-value-tile kernels
   static __device__ __forceinline__ C ld(const V v) { return dfc::ld(v); }
   static __device__ __forceinline__ V st(const C c) { return st4(c); }
   static __device__ __forceinline__ C add(const C a, const C b) { return cadd(a, b); }
   static __device__ __forceinline__ C mul(const C a, const C b) { return cmul(a, b); }
-  static __device__ __forceinline__ C conj(const C a) { return conj4(a); }
   static __device__ __forceinline__ C zero() { return zero4(); }
-  // a double-float table or entry value
-  static __device__ __forceinline__ C from_df(const float4 v) { return dfc::ld(v); }
+  static __device__ __forceinline__ C down(const C a, int) { return a; }
+  static __device__ __forceinline__ C mulq(const C a, const T w) { return mul(a, w); }
+  static __device__ __forceinline__ C bias(const C a, int) { return a; }
+  static __device__ __forceinline__ C shr(const C a, int) { return a; }
+  static __device__ __forceinline__ T ldt(const TV v) { return dfc::ld(v); }
+  static __device__ __forceinline__ TV stt(const T c) { return st4(c); }
+  static __device__ __forceinline__ T conjt(const T a) { return conj4(a); }
+  // an entry's value, a step's root (16 bytes each, written by k_pr_entries and k_pr_steps)
+  static __device__ __forceinline__ C entry(const float4 v) { return dfc::ld(v); }
+  static __device__ __forceinline__ T step(const float4 v) { return dfc::ld(v); }
+  static __device__ __forceinline__ AccV acc_zero() { return st4(zero4()); }
+  static __device__ __forceinline__ AccV acc_add(const AccV a, const C b) { return st4(cadd(dfc::ld(a), b)); }
   template <int SIGN>
-  static __device__ __forceinline__ C root(const float4* t0, const float4* t1, int b, uint64_t r) {
+  static __device__ __forceinline__ T root(const float4* t0, const float4* t1, int b, uint64_t r) {
     return tw2<SIGN>(t0, t1, b, r);
   }
   template <int R, int SIGN>
-  static __device__ __forceinline__ void dft(C (&v)[R], const C* cs) {
+  static __device__ __forceinline__ void dft(C (&v)[R], const T* cs) {
     dfc::dft<R, SIGN>(v, cs);
   }
   template <int SIGN>
-  static __device__ __forceinline__ void dft16(C (&v)[16], const C w1, const C w2, const C w3) {
+  static __device__ __forceinline__ void dft16(C (&v)[16], const T w1, const T w2, const T w3) {
     ss::dft16<SIGN>(v, w1, w2, w3);
   }
-  static __device__ __forceinline__ double2 to_double2(const V v) {
+  static __device__ __forceinline__ double2 to_double2(const AccV v) {
     return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
   }
   using Real = double;   // real samples: FP64
@@ -211,16 +234,29 @@ struct ArDF {
 struct ArF32 {
   using V = float2;
   using C = float2;
+  using TV = float2;
+  using T = float2;
+  using AccV = float2;
+  static constexpr bool kFixed = false;
   static constexpr int kMinBlocks16 = 3;
   static __device__ __forceinline__ C ld(const V v) { return v; }
   static __device__ __forceinline__ V st(const C c) { return c; }
   static __device__ __forceinline__ C add(const C a, const C b) { return fadd(a, b); }
   static __device__ __forceinline__ C mul(const C a, const C b) { return fmul(a, b); }
-  static __device__ __forceinline__ C conj(const C a) { return fconj(a); }
   static __device__ __forceinline__ C zero() { return make_float2(0.f, 0.f); }
-  static __device__ __forceinline__ C from_df(const float4 v) { return make_float2(v.x, v.z); }
+  static __device__ __forceinline__ C down(const C a, int) { return a; }
+  static __device__ __forceinline__ C mulq(const C a, const T w) { return mul(a, w); }
+  static __device__ __forceinline__ C bias(const C a, int) { return a; }
+  static __device__ __forceinline__ C shr(const C a, int) { return a; }
+  static __device__ __forceinline__ T ldt(const TV v) { return v; }
+  static __device__ __forceinline__ TV stt(const T c) { return c; }
+  static __device__ __forceinline__ T conjt(const T a) { return fconj(a); }
+  static __device__ __forceinline__ C entry(const float4 v) { return make_float2(v.x, v.z); }
+  static __device__ __forceinline__ T step(const float4 v) { return make_float2(v.x, v.z); }
+  static __device__ __forceinline__ AccV acc_zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ AccV acc_add(const AccV a, const C b) { return fadd(a, b); }
   template <int SIGN>
-  static __device__ __forceinline__ C root(const float4* t0, const float4* t1, int b, uint64_t r) {
+  static __device__ __forceinline__ T root(const float4* t0, const float4* t1, int b, uint64_t r) {
     const float4 u = __ldg(t1 + (r >> b)), l = __ldg(t0 + (r & ((1ull << b) - 1)));
     const float2 w = fmul(make_float2(u.x, u.z), make_float2(l.x, l.z));
     return SIGN > 0 ? w : fconj(w);
@@ -238,6 +274,144 @@ struct ArF32 {
   static __device__ __forceinline__ C from_real(const float x) { return make_float2(x, 0.f); }
   static __device__ __forceinline__ float real_out(const V v) { return v.x; }
 };
+
+// Fixed-point complex values.  An entry (below 1 in modulus, all of them below
+// 4) counts units of 2^-61; its products with the tile's and the column's root
+// divide by four each (mulq), and so does the evaluation's second pass (or its
+// end): samples count units of 2^-55 and stay below 2^56.5.  A sample's rounding
+// (a few units) is averaged over the M samples of a bin.  Forward, 4096-value
+// tiles: 2^60.5 after the first pass, divided by four by the second's roots,
+// 2^62.5 (P = 256) or 2^61.5 after it, divided by 2^6: Horner's sums over the
+// 16 or 32 columns stay below 2^60.5.  Forward, other tiles: fwd_shifts.  (A
+// column transform may be the same for every column, where its rounding does
+// not average: it stays at 2^-52 of the scale or below.)  The sums over tiles
+// and blocks run in FP64.  Roots: two-level table of Q62 limbs.
+constexpr int kPrEntryFrac = 61, kPrSampleFrac = 55, kPrStoreShift = 6;
+struct ArFX {
+  using V = longlong2;
+  using C = fxc::CX;
+  using TV = int4;
+  using T = fxc::TW;
+  using AccV = double2;
+  static constexpr bool kFixed = true;
+  static constexpr int kMinBlocks16 = 2;
+  static __device__ __forceinline__ C ld(const V v) { return fxc::ld(v); }
+  static __device__ __forceinline__ V st(const C c) { return fxc::st(c); }
+  static __device__ __forceinline__ C add(const C a, const C b) { return fxc::add(a, b); }
+  static __device__ __forceinline__ C mul(const C a, const T w) { return fxc::mul(a, w); }
+  static __device__ __forceinline__ C zero() { return C{0, 0}; }
+  static __device__ __forceinline__ C mulq(const C a, const T w) { return fxc::mulq(a, w); }   // a w / 4
+  // a / 2^s rounded; the same for all outputs of a transform: bias its input 0
+  // (an impulse adds to every output), then shift
+  static __device__ __forceinline__ C down(const C a, int s) { return fxc::scale_down(a, s); }
+  static __device__ __forceinline__ C bias(const C a, int s) {
+    const long long h = 1ll << (s - 1);
+    return C{a.re + h, a.im + h};
+  }
+  static __device__ __forceinline__ C shr(const C a, int s) { return C{a.re >> s, a.im >> s}; }
+  static __device__ __forceinline__ T ldt(const TV v) { return fxc::ld_tw(v); }
+  static __device__ __forceinline__ TV stt(const T w) { return fxc::st_tw(w); }
+  static __device__ __forceinline__ T conjt(const T w) { return fxc::conj(w); }
+  static __device__ __forceinline__ int4 bits(const float4 v) {
+    return make_int4(__float_as_int(v.x), __float_as_int(v.y), __float_as_int(v.z), __float_as_int(v.w));
+  }
+  static __device__ __forceinline__ float4 unbits(const int4 v) {
+    return make_float4(__int_as_float(v.x), __int_as_float(v.y), __int_as_float(v.z), __int_as_float(v.w));
+  }
+  static __device__ __forceinline__ C entry(const float4 v) {
+    const int4 i = bits(v);
+    return C{(long long)(((unsigned long long)(unsigned)i.y << 32) | (unsigned)i.x),
+             (long long)(((unsigned long long)(unsigned)i.w << 32) | (unsigned)i.z)};
+  }
+  static __device__ __forceinline__ float4 entry_bits(long long x, long long y) {
+    return unbits(make_int4((int)x, (int)(x >> 32), (int)y, (int)(y >> 32)));
+  }
+  static __device__ __forceinline__ T step(const float4 v) { return fxc::ld_tw(bits(v)); }
+  static __device__ __forceinline__ AccV acc_zero() { return make_double2(0.0, 0.0); }
+  static __device__ __forceinline__ AccV acc_add(const AccV a, const C b) {
+    return make_double2(a.x + (double)b.re, a.y + (double)b.im);
+  }
+  template <int SIGN>
+  static __device__ __forceinline__ T root(const float4* t0, const float4* t1, int b, uint64_t r) {
+    const T u = step(__ldg(t1 + (r >> b))), l = step(__ldg(t0 + (r & ((1ull << b) - 1))));
+    // the value of balanced limbs is h 2^32 + l
+    const C w = fxc::mul(C{((long long)u.rh << 32) + u.rl, ((long long)u.ih << 32) + u.il}, l);
+    const T t = fxc::to_tw(w.re, w.im);
+    return SIGN > 0 ? t : fxc::conj(t);
+  }
+  template <int R, int SIGN>
+  static __device__ __forceinline__ void dft(C (&v)[R], const T* cs) {
+    fxc::dft<R, SIGN>(v, cs);
+  }
+  template <int SIGN>
+  static __device__ __forceinline__ void dft16(C (&v)[16], const T w1, const T w2, const T w3) {
+    fxc::dft16<SIGN>(v, w1, w2, w3);
+  }
+  static __device__ __forceinline__ double2 to_double2(const AccV v) { return v; }
+  using Real = double;   // no real format
+  static __device__ __forceinline__ C from_real(const double) { return zero(); }
+  static __device__ __forceinline__ double real_out(const V) { return 0.0; }
+};
+
+// Shifts of the general forward transform: after pass p, and of a column's value
+// where Horner's sums take it up.
+struct PrShifts {
+  int pass[kDfFftMaxPasses] = {}, col = 0;
+};
+
+// exp(2 pi i r / M) in units of 2^-62, to about one unit (Horner's sums raise an
+// output's root to the W-th power, so FP64's 2^-54 would show): the angle
+// reduced to [0, pi/4] by integers, the series in pairs of doubles.
+struct D2 {
+  double h, l;
+};
+__device__ __forceinline__ D2 d2_norm(double h, double l) {
+  const double s = h + l;
+  return D2{s, l - (s - h)};
+}
+__device__ __forceinline__ D2 d2_mul(const D2 a, const D2 b) {
+  const double p = a.h * b.h;
+  return d2_norm(p, fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+__device__ __forceinline__ D2 d2_div(const D2 a, double n) {
+  const double q = a.h / n;
+  return d2_norm(q, (fma(-q, n, a.h) + a.l) / n);
+}
+__device__ __forceinline__ D2 d2_one_minus(const D2 a) {
+  const double s = 1.0 - a.h;   // |a| < 1
+  return d2_norm(s, (1.0 - s) - a.h - a.l);
+}
+__device__ long long d2_q62(const D2 a) {
+  const double x = a.h * 0x1p62, y = rint(x);
+  return (long long)y + __double2ll_rn((x - y) + a.l * 0x1p62);
+}
+__device__ fxc::TW exact_root(int64_t r, int64_t M) {
+  const int64_t q = 8 * r / M, rem = 8 * r - q * M, y = q & 1 ? M - rem : rem;
+  const double t = (double)y / (double)M, m = (double)M;
+  const D2 x = d2_mul(D2{0.78539816339744830962, 3.0616169978683830e-17}, D2{t, fma(-t, m, (double)y) / m});
+  const D2 x2 = d2_mul(x, x);
+  D2 c{1.0, 0.0}, sn{1.0, 0.0};
+  for (int k = 12; k > 0; --k) {   // x^26 / 26! < 2^-95
+    c = d2_one_minus(d2_div(d2_mul(x2, c), (double)((2 * k - 1) * (2 * k))));
+    sn = d2_one_minus(d2_div(d2_mul(x2, sn), (double)((2 * k) * (2 * k + 1))));
+  }
+  sn = d2_mul(x, sn);
+  long long a = d2_q62(c), b = d2_q62(sn);   // octant 0
+  if ((q + 1) & 2) {                         // octants 1, 2, 5, 6: nearer to the imaginary axis
+    const long long v = a;
+    a = b;
+    b = v;
+  }
+  if (q >= 2 && q <= 5) a = -a;
+  if (q >= 4) b = -b;
+  return fxc::to_tw(a, b);
+}
+
+__global__ void k_tl_table_fx(int64_t M, int b, int64_t n1, float4* t0, float4* t1) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < (1ll << b)) t0[i] = ArFX::unbits(fxc::st_tw(exact_root(i, M)));
+  if (i < n1) t1[i] = ArFX::unbits(fxc::st_tw(exact_root(i << b, M)));
+}
 
 __global__ void k_tl_table(int64_t M, int b, int64_t n1, float4* t0, float4* t1) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -259,12 +433,13 @@ __global__ void k_tl_table(int64_t M, int b, int64_t n1, float4* t0, float4* t1)
 // j, Ns < 2^16.
 template <class A, int R, int SIGN>
 __device__ __forceinline__ void mpass(const typename A::V* __restrict__ a, typename A::V* __restrict__ b, int P,
-                                      int wsh, int CS, int Ns, const typename A::V* __restrict__ tw) {
+                                      int wsh, int CS, int Ns, const typename A::TV* __restrict__ tw, int sh) {
   using C = typename A::C;
   constexpr int NC = R == 8 ? 1 : (R - 1) / 2;
-  C cs[NC > 0 ? NC : 1];
+  using T = typename A::T;
+  T cs[NC > 0 ? NC : 1];
 #pragma unroll
-  for (int m = 0; m < NC; ++m) cs[m] = A::ld(tw[(P / R) * (m + 1)]);
+  for (int m = 0; m < NC; ++m) cs[m] = A::ldt(tw[(P / R) * (m + 1)]);
   const int nb = P / R;
   const int tstride = P / (Ns * R);
   const int total = nb << wsh;
@@ -282,14 +457,14 @@ __device__ __forceinline__ void mpass(const typename A::V* __restrict__ a, typen
     if (Ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const C w = A::ld(tw[tstride * (k * r)]);
-        v[r] = A::mul(v[r], SIGN > 0 ? w : A::conj(w));
+        const T w = A::ldt(tw[tstride * (k * r)]);
+        v[r] = A::mul(v[r], SIGN > 0 ? w : A::conjt(w));
       }
     }
     A::template dft<R, SIGN>(v, cs);
     const int base = jq * Ns * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) bc[base + r * Ns] = A::st(v[r]);
+    for (int r = 0; r < R; ++r) bc[base + r * Ns] = A::st(SIGN < 0 && sh ? A::down(v[r], sh) : v[r]);
   }
 }
 
@@ -297,17 +472,18 @@ __device__ __forceinline__ void mpass(const typename A::V* __restrict__ a, typen
 // the buffer that holds the result.  Ends with a block barrier.
 template <class A, int SIGN>
 __device__ typename A::V* columns_dft(typename A::V* a, typename A::V* b, int P, int wsh, int CS,
-                                      const DfRadices& rad, const typename A::V* __restrict__ tw) {
+                                      const DfRadices& rad, const PrShifts& shifts,
+                                      const typename A::TV* __restrict__ tw) {
   int Ns = 1;
   for (int p = 0; p < rad.n; ++p) {
-    const int R = rad.r[p];
+    const int R = rad.r[p], sh = shifts.pass[p];
     switch (R) {
-      case 8: mpass<A, 8, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
-      case 4: mpass<A, 4, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
-      case 2: mpass<A, 2, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
-      case 5: mpass<A, 5, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
-      case 3: mpass<A, 3, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
-      default: mpass<A, 7, SIGN>(a, b, P, wsh, CS, Ns, tw); break;
+      case 8: mpass<A, 8, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
+      case 4: mpass<A, 4, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
+      case 2: mpass<A, 2, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
+      case 5: mpass<A, 5, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
+      case 3: mpass<A, 3, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
+      default: mpass<A, 7, SIGN>(a, b, P, wsh, CS, Ns, tw, sh); break;
     }
     __syncthreads();
     typename A::V* t = a;
@@ -324,6 +500,7 @@ __device__ typename A::V* columns_dft(typename A::V* a, typename A::V* b, int P,
 // r mod P in term order (a's terms, then f's; r before M - r).  One block;
 // boff[k] = first entry of bucket k, boff[P] = the number of entries.
 // kq: scratch of 2 (na + nf) int32 (the two buckets of every term).
+template <bool FX>
 __global__ void k_pr_entries(const int64_t* __restrict__ qa, const double2* __restrict__ ca,
                              const int64_t* __restrict__ na_dev, const int64_t* __restrict__ qf,
                              const double2* __restrict__ cf, const int64_t* __restrict__ nf_dev,
@@ -387,15 +564,20 @@ __global__ void k_pr_entries(const int64_t* __restrict__ qa, const double2* __re
         y = 0.5 * c.x * jf;
       }
     }
-    const DF dx = df_split(x), dy = df_split(y);
     er[pos] = neg ? M - r : r;
-    ev[pos] = make_float4(dx.hi, dx.lo, dy.hi, dy.lo);
+    if (FX) {
+      const double un = ldexp(1.0, kPrEntryFrac);
+      ev[pos] = ArFX::entry_bits(__double2ll_rn(x * un), __double2ll_rn(y * un));
+    } else {
+      const DF dx = df_split(x), dy = df_split(y);
+      ev[pos] = make_float4(dx.hi, dx.lo, dy.hi, dy.lo);
+    }
   }
 }
 
 // tab[e][i] = exp(sign 2 pi i (i r_e mod M) / M) for e < n (device count n_dev
 // when given, else n_host), i < W.
-template <int SIGN>
+template <int SIGN, bool FX>
 __global__ void k_pr_steps(const int64_t* __restrict__ r, const int32_t* __restrict__ n_dev, int64_t n_host, int W,
                            int64_t M, const float4* __restrict__ t0, const float4* __restrict__ t1, int b,
                            float4* tab) {
@@ -405,7 +587,8 @@ __global__ void k_pr_steps(const int64_t* __restrict__ r, const int32_t* __restr
   const int i = (int)(id % W);
   if (e >= n) return;
   const uint64_t idx = ((uint64_t)i * (uint64_t)r[e]) % (uint64_t)M;
-  tab[id] = st4(tw2<SIGN>(t0, t1, b, idx));
+  if (FX) tab[id] = ArFX::unbits(fxc::st_tw(ArFX::root<SIGN>(t0, t1, b, idx)));
+  else tab[id] = st4(tw2<SIGN>(t0, t1, b, idx));
 }
 
 // Output bins: bucket b mod P of every output.
@@ -425,24 +608,26 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
                                                         int64_t n_tiles, void* __restrict__ out) {
   using V = typename A::V;
   using C = typename A::C;
+  using TV = typename A::TV;
+  using T = typename A::T;
   extern __shared__ __align__(16) float4 sm4[];
   const int CS = P + 1, W = 1 << wsh;
   const unsigned wmask = (unsigned)W - 1u;
   V* Av = reinterpret_cast<V*>(sm4);
   V* Bf = Av + W * CS;
-  V* tw = Bf + W * CS;
-  V* base = tw + P;
-  V* es = base + kPrChunk;                          // staged step powers (n_stage > 0)
+  TV* tw = reinterpret_cast<TV*>(Bf + W * CS);
+  V* base = reinterpret_cast<V*>(tw + P);
+  TV* es = reinterpret_cast<TV*>(base + kPrChunk);   // staged step powers (n_stage > 0)
   int32_t* boff = reinterpret_cast<int32_t*>(es + n_stage);
   const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
   for (int m = threadIdx.x; m < P; m += blockDim.x)
-    tw[m] = A::st(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
+    tw[m] = A::stt(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
   for (int k = threadIdx.x; k <= P; k += blockDim.x) boff[k] = boff_g[k];
   __syncthreads();
   const int ne = boff[P];
   // the step powers exp(2 pi i i r_e / M) are the same for every tile
   if (n_stage > 0) {
-    for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::st(A::from_df(__ldg(estep + x)));
+    for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::stt(A::step(__ldg(estep + x)));
     __syncthreads();
   }
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -452,7 +637,7 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
     do {
       const int e1 = min(ne, e0 + kPrChunk);
       for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x)
-        base[e - e0] = A::st(A::mul(A::from_df(__ldg(ev + e)),
+        base[e - e0] = A::st(A::mulq(A::entry(__ldg(ev + e)),
                                     A::template root<1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)er[e], Mu, inv))));
       __syncthreads();
 #pragma unroll 4
@@ -461,10 +646,10 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
         const int lo = max(boff[k], e0), hi = min(boff[k + 1], e1);
         C s = e0 == 0 ? A::zero() : A::ld(Av[i * CS + k]);
         if (n_stage > 0) {
-          for (int e = lo; e < hi; ++e) s = A::add(s, A::mul(A::ld(base[e - e0]), A::ld(es[e * W + i])));
+          for (int e = lo; e < hi; ++e) s = A::add(s, A::mulq(A::ld(base[e - e0]), A::ldt(es[e * W + i])));
         } else {
           for (int e = lo; e < hi; ++e)
-            s = A::add(s, A::mul(A::ld(base[e - e0]), A::from_df(__ldg(estep + (int64_t)e * W + i))));
+            s = A::add(s, A::mulq(A::ld(base[e - e0]), A::step(__ldg(estep + (int64_t)e * W + i))));
         }
         Av[i * CS + k] = A::st(s);
       }
@@ -472,7 +657,7 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
       e0 += kPrChunk;
     } while (e0 < ne);
     // s[q0 + i + Q p] = sum_k w_P^{p k} C[k][i]
-    const V* res = columns_dft<A, 1>(Av, Bf, P, wsh, CS, rad, tw);
+    const V* res = columns_dft<A, 1>(Av, Bf, P, wsh, CS, rad, PrShifts{}, tw);
     for (int u = threadIdx.x; u < P * W; u += blockDim.x) {
       const int i = (int)((unsigned)u & wmask), p = u >> wsh;
       const int64_t q = q0 + i;
@@ -480,7 +665,7 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_
       if (OUT_REAL)
         static_cast<typename A::Real*>(out)[q + Q * p] = A::real_out(res[i * CS + p]);
       else
-        static_cast<V*>(out)[q + Q * p] = res[i * CS + p];
+        static_cast<V*>(out)[q + Q * p] = A::st(A::down(A::ld(res[i * CS + p]), 2));
     }
     __syncthreads();
   }
@@ -522,7 +707,7 @@ __global__ void __launch_bounds__(kPrThreads, 2) k_pr_eval_col(int64_t M, int64_
   for (int k = threadIdx.x; k <= P; k += blockDim.x) boff[k] = boff_g[k];
   __syncthreads();
   const int ne = boff[P];
-  for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::from_df(__ldg(estep + x));
+  for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::step(__ldg(estep + x));
   const float2 cs[1] = {tw[P / 8]};
   const int sub = threadIdx.x / W, i = threadIdx.x % W;
   // the block's tiles: SUB neighbours a round, the rounds gridDim.x SUB tiles apart
@@ -533,7 +718,7 @@ __global__ void __launch_bounds__(kPrThreads, 2) k_pr_eval_col(int64_t M, int64_
     for (int x = threadIdx.x; x < kPrColRounds * SUB * ne; x += blockDim.x) {
       const int t = x / ne, e = x - t * ne;   // tile t % SUB of round t / SUB
       const uint64_t q0 = (uint64_t)min(first + (t / SUB) * stride + t % SUB, n_tiles - 1) * W;
-      base[x] = A::mul(A::from_df(__ldg(ev + e)), A::root<1>(t0, t1, b, mulmod(q0, (uint64_t)er[e], Mu, inv)));
+      base[x] = A::mul(A::entry(__ldg(ev + e)), A::root<1>(t0, t1, b, mulmod(q0, (uint64_t)er[e], Mu, inv)));
     }
     __syncthreads();
 #pragma unroll 1
@@ -590,25 +775,29 @@ __global__ void __launch_bounds__(kPrThreads, 2) k_pr_eval_col(int64_t M, int64_
 // owns output o for the whole launch).
 template <class A, bool IN_REAL>
 __global__ void __launch_bounds__(kPrThreads) k_pr_fwd(int64_t M, int P, int64_t Q, int wsh, DfRadices rad,
+                                                       PrShifts shifts,
                                                        const float4* __restrict__ t0, const float4* __restrict__ t1,
                                                        int b, const void* __restrict__ in,
                                                        const int64_t* __restrict__ ob,
                                                        const int32_t* __restrict__ kout, int n_out,
                                                        const float4* __restrict__ oz, int64_t n_tiles,
-                                                       typename A::V* __restrict__ partial) {
+                                                       typename A::AccV* __restrict__ partial) {
   using V = typename A::V;
   using C = typename A::C;
+  using TV = typename A::TV;
+  using T = typename A::T;
+  using AccV = typename A::AccV;
   extern __shared__ __align__(16) float4 sm4[];
   const int CS = P + 1, W = 1 << wsh;
   const unsigned wmask = (unsigned)W - 1u;
   V* Av = reinterpret_cast<V*>(sm4);
   V* Bf = Av + W * CS;
-  V* tw = Bf + W * CS;
-  V* acc = tw + P;
+  TV* tw = reinterpret_cast<TV*>(Bf + W * CS);
+  AccV* acc = reinterpret_cast<AccV*>(tw + P);
   const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
   for (int m = threadIdx.x; m < P; m += blockDim.x)
-    tw[m] = A::st(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
-  for (int o = threadIdx.x; o < n_out; o += blockDim.x) acc[o] = A::st(A::zero());
+    tw[m] = A::stt(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
+  for (int o = threadIdx.x; o < n_out; o += blockDim.x) acc[o] = A::acc_zero();
   __syncthreads();
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int64_t q0 = tile * W;
@@ -623,15 +812,15 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_fwd(int64_t M, int P, int64_t
       Av[i * CS + p] = A::st(v);
     }
     __syncthreads();
-    const V* res = columns_dft<A, -1>(Av, Bf, P, wsh, CS, rad, tw);
+    const V* res = columns_dft<A, -1>(Av, Bf, P, wsh, CS, rad, shifts, tw);
     const int wl = Q - q0 < (int64_t)W ? (int)(Q - q0) : W;
     for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
       const int k = kout[o];
-      const C w = A::template root<-1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)ob[o], Mu, inv));
-      const C z = A::from_df(__ldg(oz + 2 * o));   // oz: stride 2 (the step table of width 2, entry 1)
-      C s = A::ld(res[(wl - 1) * CS + k]);
-      for (int i = wl - 2; i >= 0; --i) s = A::add(A::mul(s, z), A::ld(res[i * CS + k]));
-      acc[o] = A::st(A::add(A::ld(acc[o]), A::mul(s, w)));
+      const T w = A::template root<-1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)ob[o], Mu, inv));
+      const T z = A::step(__ldg(oz + 2 * o));   // oz: stride 2 (the step table of width 2, entry 1)
+      C s = A::down(A::ld(res[(wl - 1) * CS + k]), shifts.col);
+      for (int i = wl - 2; i >= 0; --i) s = A::add(A::mul(s, z), A::down(A::ld(res[i * CS + k]), shifts.col));
+      acc[o] = A::acc_add(acc[o], A::mul(s, w));
     }
     __syncthreads();
   }
@@ -657,10 +846,11 @@ __host__ __device__ constexpr bool pr16_supported(int P) { return P == 128 || P 
 // output r at k + 16 r.  out(p, value) receives the outputs (position p in the
 // column); with IN_PLACE the block synchronises between reads and writes.
 template <class A, int P, int SIGN, bool IN_PLACE, class Out>
-__device__ __forceinline__ void pr16_pass2(const typename A::V* col, int k, const typename A::V* tw,
-                                           const typename A::C w1, const typename A::C w2, const typename A::C w3,
+__device__ __forceinline__ void pr16_pass2(const typename A::V* col, int k, const typename A::TV* tw,
+                                           const typename A::T w1, const typename A::T w2, const typename A::T w3,
                                            Out out) {
   using C = typename A::C;
+  using T = typename A::T;
   if constexpr (P == 256) {
     C v[16];
 #pragma unroll
@@ -668,9 +858,11 @@ __device__ __forceinline__ void pr16_pass2(const typename A::V* col, int k, cons
     if (IN_PLACE) __syncthreads();
 #pragma unroll
     for (int r = 1; r < 16; ++r) {
-      const C w = A::ld(tw[k * r]);
-      v[r] = A::mul(v[r], SIGN > 0 ? w : A::conj(w));
+      const T w = A::ldt(tw[k * r]);
+      v[r] = A::mulq(v[r], SIGN > 0 ? w : A::conjt(w));
     }
+    v[0] = A::down(v[0], 2);
+    if (SIGN < 0) v[0] = A::bias(v[0], kPrStoreShift);
     A::template dft16<SIGN>(v, w1, w2, w3);
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1)
@@ -683,15 +875,17 @@ __device__ __forceinline__ void pr16_pass2(const typename A::V* col, int k, cons
 #pragma unroll
       for (int r = 0; r < 8; ++r) v[h][r] = A::ld(col[k + 8 * h + 16 * r]);
     if (IN_PLACE) __syncthreads();
-    const C cs[1] = {w2};   // exp(2 pi i / 8)
+    const T cs[1] = {w2};   // exp(2 pi i / 8)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int kk = k + 8 * h;
 #pragma unroll
       for (int r = 1; r < 8; ++r) {
-        const C w = A::ld(tw[kk * r]);
-        v[h][r] = A::mul(v[h][r], SIGN > 0 ? w : A::conj(w));
+        const T w = A::ldt(tw[kk * r]);
+        v[h][r] = A::mulq(v[h][r], SIGN > 0 ? w : A::conjt(w));
       }
+      v[h][0] = A::down(v[h][0], 2);
+      if (SIGN < 0) v[h][0] = A::bias(v[h][0], kPrStoreShift);
       A::template dft<8, SIGN>(v[h], cs);
 #pragma unroll
       for (int r = 0; r < 8; ++r) out(kk + 16 * r, v[h][r]);
@@ -710,24 +904,26 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_eval16(int
                                                                int64_t n_tiles, void* __restrict__ out) {
   using V = typename A::V;
   using C = typename A::C;
+  using TV = typename A::TV;
+  using T = typename A::T;
   constexpr int W = kPr16Tile / P, CS = P + 1, R2 = P / 16;
   extern __shared__ __align__(16) float4 sm4[];
   V* tl = reinterpret_cast<V*>(sm4);
-  V* tw = tl + W * CS;
-  V* base = tw + P;
-  V* es = base + kPrChunk;
+  TV* tw = reinterpret_cast<TV*>(tl + W * CS);
+  V* base = reinterpret_cast<V*>(tw + P);
+  TV* es = reinterpret_cast<TV*>(base + kPrChunk);
   int32_t* boff = reinterpret_cast<int32_t*>(es + n_stage);
   const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
   for (int m = threadIdx.x; m < P; m += blockDim.x)
-    tw[m] = A::st(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
+    tw[m] = A::stt(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
   for (int k = threadIdx.x; k <= P; k += blockDim.x) boff[k] = boff_g[k];
   __syncthreads();
   const int ne = boff[P];
   if (n_stage > 0) {
-    for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::st(A::from_df(__ldg(estep + x)));
+    for (int x = threadIdx.x; x < ne * W; x += blockDim.x) es[x] = A::stt(A::step(__ldg(estep + x)));
     __syncthreads();
   }
-  const C w1 = A::ld(tw[P / 16]), w2 = A::ld(tw[2 * P / 16]), w3 = A::ld(tw[3 * P / 16]);
+  const T w1 = A::ldt(tw[P / 16]), w2 = A::ldt(tw[2 * P / 16]), w3 = A::ldt(tw[3 * P / 16]);
   const int u = threadIdx.x;
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int64_t q0 = tile * W;
@@ -736,7 +932,7 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_eval16(int
     do {
       const int e1 = min(ne, e0 + kPrChunk);
       for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x)
-        base[e - e0] = A::st(A::mul(A::from_df(__ldg(ev + e)),
+        base[e - e0] = A::st(A::mulq(A::entry(__ldg(ev + e)),
                                     A::template root<1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)er[e], Mu, inv))));
       __syncthreads();
       for (int x = threadIdx.x; x < P * W; x += blockDim.x) {
@@ -744,8 +940,8 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_eval16(int
         const int lo = max(boff[k], e0), hi = min(boff[k + 1], e1);
         C sum = e0 == 0 ? A::zero() : A::ld(tl[i * CS + k]);
         for (int e = lo; e < hi; ++e) {
-          const C st = n_stage > 0 ? A::ld(es[e * W + i]) : A::from_df(__ldg(estep + (int64_t)e * W + i));
-          sum = A::add(sum, A::mul(A::ld(base[e - e0]), st));
+          const T st = n_stage > 0 ? A::ldt(es[e * W + i]) : A::step(__ldg(estep + (int64_t)e * W + i));
+          sum = A::add(sum, A::mulq(A::ld(base[e - e0]), st));
         }
         tl[i * CS + k] = A::st(sum);
       }
@@ -792,20 +988,23 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_fwd16(int6
                                                               const int64_t* __restrict__ ob,
                                                               const int32_t* __restrict__ kout, int n_out,
                                                               const float4* __restrict__ oz, int64_t n_tiles,
-                                                              typename A::V* __restrict__ partial) {
+                                                              typename A::AccV* __restrict__ partial) {
   using V = typename A::V;
   using C = typename A::C;
+  using TV = typename A::TV;
+  using T = typename A::T;
+  using AccV = typename A::AccV;
   constexpr int W = kPr16Tile / P, CS = P + 1, R2 = P / 16;
   extern __shared__ __align__(16) float4 sm4[];
   V* tl = reinterpret_cast<V*>(sm4);
-  V* tw = tl + W * CS;
-  V* acc = tw + P;
+  TV* tw = reinterpret_cast<TV*>(tl + W * CS);
+  AccV* acc = reinterpret_cast<AccV*>(tw + P);
   const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
   for (int m = threadIdx.x; m < P; m += blockDim.x)
-    tw[m] = A::st(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
-  for (int o = threadIdx.x; o < n_out; o += blockDim.x) acc[o] = A::st(A::zero());
+    tw[m] = A::stt(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
+  for (int o = threadIdx.x; o < n_out; o += blockDim.x) acc[o] = A::acc_zero();
   __syncthreads();
-  const C w1 = A::ld(tw[P / 16]), w2 = A::ld(tw[2 * P / 16]), w3 = A::ld(tw[3 * P / 16]);
+  const T w1 = A::ldt(tw[P / 16]), w2 = A::ldt(tw[2 * P / 16]), w3 = A::ldt(tw[3 * P / 16]);
   const int u = threadIdx.x;
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int64_t q0 = tile * W;
@@ -833,17 +1032,19 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_fwd16(int6
     {
       const int c = u % W, k = u / W;
       V* col = tl + c * CS;
-      pr16_pass2<A, P, -1, true>(col, k, tw, w1, w2, w3, [&](int p, const C val) { col[p] = A::st(val); });
+      pr16_pass2<A, P, -1, true>(col, k, tw, w1, w2, w3, [&](int p, const C val) {
+        col[p] = A::st(A::shr(val, kPrStoreShift));
+      });
     }
     __syncthreads();
     const int wl = Q - q0 < (int64_t)W ? (int)(Q - q0) : W;
     for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
       const int k = kout[o];
-      const C w = A::template root<-1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)ob[o], Mu, inv));
-      const C z = A::from_df(__ldg(oz + 2 * o));
+      const T w = A::template root<-1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)ob[o], Mu, inv));
+      const T z = A::step(__ldg(oz + 2 * o));
       C sum = A::ld(tl[(wl - 1) * CS + k]);
       for (int i = wl - 2; i >= 0; --i) sum = A::add(A::mul(sum, z), A::ld(tl[i * CS + k]));
-      acc[o] = A::st(A::add(A::ld(acc[o]), A::mul(sum, w)));
+      acc[o] = A::acc_add(acc[o], A::mul(sum, w));
     }
     __syncthreads();
   }
@@ -851,9 +1052,10 @@ __global__ void __launch_bounds__(kPr16Threads, A::kMinBlocks16) k_pr_fwd16(int6
 }
 
 // X[o] = sum over blocks of partial[blk][o] in FP64: one warp per output,
-// lanes in a fixed stride, then a fixed butterfly; written as double-float.
+// lanes in a fixed stride, then a fixed butterfly; times unit.
 template <class A>
-__global__ void k_pr_reduce(const typename A::V* __restrict__ partial, int nb, int n_out, float4* __restrict__ X) {
+__global__ void k_pr_reduce(const typename A::AccV* __restrict__ partial, int nb, int n_out, double unit,
+                            double2* __restrict__ X) {
   const int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (o >= n_out) return;   // warp-uniform
@@ -868,11 +1070,13 @@ __global__ void k_pr_reduce(const typename A::V* __restrict__ partial, int nb, i
     sr += __shfl_xor_sync(0xffffffffu, sr, m);
     si += __shfl_xor_sync(0xffffffffu, si, m);
   }
-  if (lane == 0) {
-    const DF r = df_split(sr), i = df_split(si);
-    X[o] = make_float4(r.hi, r.lo, i.hi, i.lo);
-  }
+  if (lane == 0) X[o] = make_double2(sr * unit, si * unit);
 }
+
+template <class A>
+const float4* table0(const TwoLevelTable& T) { return A::kFixed ? T.x0.get() : T.t0.get(); }
+template <class A>
+const float4* table1(const TwoLevelTable& T) { return A::kFixed ? T.x1.get() : T.t1.get(); }
 
 template <class A>
 size_t eval_smem(const PrunedSplit& S, int64_t n_stage) {
@@ -902,7 +1106,7 @@ ss_status launch_eval(const TwoLevelTable& T, const PrunedSplit& S, int wsh, con
   const size_t smem = eval_smem<A>(S, n_stage);
   int grid = 0;
   SS_TRY(grid_for(k_pr_eval<A, OUT_REAL>, smem, n_tiles, &grid));
-  k_pr_eval<A, OUT_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, T.t0.get(), T.t1.get(), T.b, er,
+  k_pr_eval<A, OUT_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, table0<A>(T), table1<A>(T), T.b, er,
                                                          ev, boff, estep, (int)n_stage, n_tiles, out);
   SS_LAUNCH_CHECK();
   return SS_OK;
@@ -917,7 +1121,7 @@ ss_status launch_eval16(const TwoLevelTable& T, const PrunedSplit& S, const int6
       (size_t)(W * (P + 1) + P + kPrChunk + n_stage) * sizeof(typename A::V) + (P + 1) * sizeof(int32_t);
   int grid = 0;
   SS_TRY(grid_for(k_pr_eval16<A, P, OUT_REAL>, smem, n_tiles, &grid));
-  k_pr_eval16<A, P, OUT_REAL><<<grid, kPr16Threads, smem, st>>>(T.M, S.Q, T.t0.get(), T.t1.get(), T.b, er, ev, boff,
+  k_pr_eval16<A, P, OUT_REAL><<<grid, kPr16Threads, smem, st>>>(T.M, S.Q, table0<A>(T), table1<A>(T), T.b, er, ev, boff,
                                                                  estep, (int)n_stage, n_tiles, out);
   SS_LAUNCH_CHECK();
   return SS_OK;
@@ -946,55 +1150,73 @@ ss_status launch_eval_col(const TwoLevelTable& T, const PrunedSplit& S, int64_t 
 
 template <class A, int P, bool IN_REAL>
 ss_status launch_fwd16(const TwoLevelTable& T, const PrunedSplit& S, const void* in, const int64_t* ob,
-                       const int32_t* kout, int nc, const float4* oz, float4* X, cudaStream_t st) {
+                       const int32_t* kout, int nc, const float4* oz, double unit, double2* X, cudaStream_t st) {
   constexpr int W = kPr16Tile / P;
   const int64_t n_tiles = (S.Q + W - 1) / W;
   const size_t smem = (size_t)(W * (P + 1) + P + nc) * sizeof(typename A::V);
   int grid = 0;
   SS_TRY(grid_for(k_pr_fwd16<A, P, IN_REAL>, smem, n_tiles, &grid));
-  DevBuf<typename A::V> partial;
+  DevBuf<typename A::AccV> partial;
   SS_TRY(partial.alloc_tmp((size_t)grid * nc, st));
   {
     ProfScope prof_("k_pr_fwd", st, true);
-    k_pr_fwd16<A, P, IN_REAL><<<grid, kPr16Threads, smem, st>>>(T.M, S.Q, T.t0.get(), T.t1.get(), T.b, in, ob, kout,
+    k_pr_fwd16<A, P, IN_REAL><<<grid, kPr16Threads, smem, st>>>(T.M, S.Q, table0<A>(T), table1<A>(T), T.b, in, ob, kout,
                                                                  nc, oz, n_tiles, partial.get());
     SS_LAUNCH_CHECK();
   }
-  k_pr_reduce<A><<<nblk((int64_t)nc * 32), 256, 0, st>>>(partial.get(), grid, nc, X);
+  k_pr_reduce<A><<<nblk((int64_t)nc * 32), 256, 0, st>>>(partial.get(), grid, nc, unit, X);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
 
 template <class A, bool IN_REAL>
 ss_status launch_fwd16_p(const TwoLevelTable& T, const PrunedSplit& S, const void* in, const int64_t* ob,
-                         const int32_t* kout, int nc, const float4* oz, float4* X, cudaStream_t st) {
-  if (S.P == 256) return launch_fwd16<A, 256, IN_REAL>(T, S, in, ob, kout, nc, oz, X, st);
-  return launch_fwd16<A, 128, IN_REAL>(T, S, in, ob, kout, nc, oz, X, st);
+                         const int32_t* kout, int nc, const float4* oz, double unit, double2* X, cudaStream_t st) {
+  if (S.P == 256) return launch_fwd16<A, 256, IN_REAL>(T, S, in, ob, kout, nc, oz, unit, X, st);
+  return launch_fwd16<A, 128, IN_REAL>(T, S, in, ob, kout, nc, oz, unit, X, st);
 }
 
 template <class A, bool IN_REAL>
-ss_status launch_fwd(const TwoLevelTable& T, const PrunedSplit& S, int wsh, const void* in, const int64_t* ob,
-                     const int32_t* kout, int nc, const float4* oz, float4* X, cudaStream_t st) {
+ss_status launch_fwd(const TwoLevelTable& T, const PrunedSplit& S, int wsh, const PrShifts& shifts, const void* in,
+                     const int64_t* ob,
+                     const int32_t* kout, int nc, const float4* oz, double unit, double2* X, cudaStream_t st) {
   const int64_t n_tiles = (S.Q + S.W - 1) / S.W;
   const size_t smem = fwd_smem<A>(S, nc);
   int grid = 0;
   SS_TRY(grid_for(k_pr_fwd<A, IN_REAL>, smem, n_tiles, &grid));
-  DevBuf<typename A::V> partial;
+  DevBuf<typename A::AccV> partial;
   SS_TRY(partial.alloc_tmp((size_t)grid * nc, st));
   {
     ProfScope prof_("k_pr_fwd", st, true);
-    k_pr_fwd<A, IN_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, T.t0.get(), T.t1.get(), T.b, in,
+    k_pr_fwd<A, IN_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, shifts, table0<A>(T), table1<A>(T), T.b, in,
                                                          ob, kout, nc, oz, n_tiles, partial.get());
     SS_LAUNCH_CHECK();
   }
-  k_pr_reduce<A><<<nblk((int64_t)nc * 32), 256, 0, st>>>(partial.get(), grid, nc, X);
+  k_pr_reduce<A><<<nblk((int64_t)nc * 32), 256, 0, st>>>(partial.get(), grid, nc, unit, X);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
 
+// Samples stay below 2^56.5; a value enters a pass below 2^59.5 (a radix-8 sum
+// then stays below 2^62.5), and 2^wsh columns add up to less than 2^60.5.
+// Returns the sum of the shifts.
+int fwd_shifts(const PrunedSplit& S, int wsh, PrShifts* out) {
+  double g = -3.0;   // log2 of a value, less 59.5
+  int sum = 0;
+  for (int p = 0; p < S.rad.n; ++p) {
+    g += std::log2((double)S.rad.r[p]);
+    const int sh = p + 1 < S.rad.n && g > 0.0 ? (int)std::ceil(g) : 0;
+    out->pass[p] = sh;
+    sum += sh;
+    g -= sh;
+  }
+  out->col = std::max(0, (int)std::ceil(g + wsh - 1.0));
+  return sum + out->col;
+}
+
 }  // namespace
 
-ss_status two_level_table(int64_t M, TwoLevelTable* T, cudaStream_t st) {
+ss_status two_level_table(int64_t M, bool fx, TwoLevelTable* T, cudaStream_t st) {
   int bits = 0;
   while ((1ll << bits) < M) ++bits;
   T->M = M;
@@ -1003,6 +1225,11 @@ ss_status two_level_table(int64_t M, TwoLevelTable* T, cudaStream_t st) {
   SS_TRY(T->t0.alloc(n0, st));
   SS_TRY(T->t1.alloc(n1, st));
   k_tl_table<<<nblk(std::max(n0, n1)), 256, 0, st>>>(M, T->b, n1, T->t0.get(), T->t1.get());
+  if (fx) {
+    SS_TRY(T->x0.alloc(n0, st));
+    SS_TRY(T->x1.alloc(n1, st));
+    k_tl_table_fx<<<nblk(std::max(n0, n1)), 256, 0, st>>>(M, T->b, n1, T->x0.get(), T->x1.get());
+  }
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
@@ -1064,13 +1291,15 @@ ss_status pruned_eval_pair(const TwoLevelTable& T, const int64_t* qa, const doub
     const int eb = std::min(1024, (S.P + 31) / 32 * 32);
     // the entries' buckets in shared memory when they fit (48 KB with the counts)
     const int kq_smem = (int)std::min<int64_t>(ne_max, 12288 - (S.P + 1));
-    k_pr_entries<<<1, eb, (S.P + 1 + kq_smem) * sizeof(int32_t), st>>>(qa, ca, na_dev, qf, cf, qf ? nf_dev : nullptr,
-                                                                        scale, M,
-                                                                        S.P, kq.get(), er.get(), ev.get(),
-                                                                        boff.get(), kq_smem);
+    const bool fx = fmt == PrunedFormat::kFxComplex;
+    const auto entries = fx ? k_pr_entries<true> : k_pr_entries<false>;
+    entries<<<1, eb, (S.P + 1 + kq_smem) * sizeof(int32_t), st>>>(qa, ca, na_dev, qf, cf, qf ? nf_dev : nullptr, scale,
+                                                                  M, S.P, kq.get(), er.get(), ev.get(), boff.get(),
+                                                                  kq_smem);
     SS_LAUNCH_CHECK();
-    k_pr_steps<1><<<nblk(ne_max * Wt), 256, 0, st>>>(er.get(), boff.get() + S.P, 0, Wt, M, T.t0.get(), T.t1.get(),
-                                                     T.b, estep.get());
+    const auto steps = fx ? k_pr_steps<1, true> : k_pr_steps<1, false>;
+    steps<<<nblk(ne_max * Wt), 256, 0, st>>>(er.get(), boff.get() + S.P, 0, Wt, M, fx ? T.x0.get() : T.t0.get(),
+                                             fx ? T.x1.get() : T.t1.get(), T.b, estep.get());
     SS_LAUNCH_CHECK();
   }
   int wsh = 0;
@@ -1080,8 +1309,8 @@ ss_status pruned_eval_pair(const TwoLevelTable& T, const int64_t* qa, const doub
   ProfScope prof_("k_pr_eval", st, true);
   if (t16) {
     switch (fmt) {
-      case PrunedFormat::kDfComplex:
-        return launch_eval16_p<ArDF, false>(T, S, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
+      case PrunedFormat::kFxComplex:
+        return launch_eval16_p<ArFX, false>(T, S, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
       case PrunedFormat::kF64Real:
         return launch_eval16_p<ArDF, true>(T, S, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
       case PrunedFormat::kF32Complex:
@@ -1100,8 +1329,8 @@ ss_status pruned_eval_pair(const TwoLevelTable& T, const int64_t* qa, const doub
     return real ? go(launch_eval_col<32, true>) : go(launch_eval_col<32, false>);
   }
   switch (fmt) {
-    case PrunedFormat::kDfComplex:
-      return launch_eval<ArDF, false>(T, S, wsh, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
+    case PrunedFormat::kFxComplex:
+      return launch_eval<ArFX, false>(T, S, wsh, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
     case PrunedFormat::kF64Real:
       return launch_eval<ArDF, true>(T, S, wsh, er.get(), ev.get(), boff.get(), estep.get(), n_stage, out, st);
     case PrunedFormat::kF32Complex:
@@ -1112,13 +1341,20 @@ ss_status pruned_eval_pair(const TwoLevelTable& T, const int64_t* qa, const doub
 }
 
 ss_status pruned_forward(const TwoLevelTable& T, const void* s, PrunedFormat fmt, const int64_t* bins, int64_t n_out,
-                         float4* X, cudaStream_t st) {
+                         double2* X, cudaStream_t st) {
   const int64_t M = T.M;
   if (n_out < 1) return SS_OK;
   PrunedSplit S;
   if (!pruned_split(M, n_out, &S)) SS_FAIL(SS_ERR_INVALID, "pruned transform: M = %lld has no split", (long long)M);
   int wsh = 0;
   while ((1 << wsh) < S.W) ++wsh;
+  const bool fx = fmt == PrunedFormat::kFxComplex, t16 = pr16_supported(S.P);   // 4096-value tiles
+  double unit = 1.0;
+  PrShifts shifts;
+  if (fx) {   // what the passes and Horner's sums divide out
+    const int sh = t16 ? 2 + kPrStoreShift : fwd_shifts(S, wsh, &shifts);
+    unit = std::ldexp(1.0, sh - kPrSampleFrac);
+  }
   for (int64_t o0 = 0; o0 < n_out; o0 += kPrMaxOut) {
     const int nc = (int)std::min<int64_t>(kPrMaxOut, n_out - o0);
     DevBuf<int32_t> kout;
@@ -1127,27 +1363,27 @@ ss_status pruned_forward(const TwoLevelTable& T, const void* s, PrunedFormat fmt
     SS_TRY(oz.alloc_tmp((size_t)nc * 2, st));
     k_pr_kout<<<nblk(nc), 256, 0, st>>>(bins + o0, nc, S.P, kout.get());
     // oz[2 o + 1] = exp(-2 pi i b_o / M): the Horner root of output o
-    k_pr_steps<-1><<<nblk((int64_t)nc * 2), 256, 0, st>>>(bins + o0, nullptr, nc, 2, M, T.t0.get(), T.t1.get(), T.b,
-                                                          oz.get());
+    const auto steps = fx ? k_pr_steps<-1, true> : k_pr_steps<-1, false>;
+    steps<<<nblk((int64_t)nc * 2), 256, 0, st>>>(bins + o0, nullptr, nc, 2, M, fx ? T.x0.get() : T.t0.get(),
+                                                 fx ? T.x1.get() : T.t1.get(), T.b, oz.get());
     SS_LAUNCH_CHECK();
     const float4* z = oz.get() + 1;
-    const bool t16 = pr16_supported(S.P);   // 4096-value tiles
     switch (fmt) {
-      case PrunedFormat::kDfComplex:
-        if (t16) SS_TRY((launch_fwd16_p<ArDF, false>(T, S, s, bins + o0, kout.get(), nc, z, X + o0, st)));
-        else SS_TRY((launch_fwd<ArDF, false>(T, S, wsh, s, bins + o0, kout.get(), nc, z, X + o0, st)));
+      case PrunedFormat::kFxComplex:
+        if (t16) SS_TRY((launch_fwd16_p<ArFX, false>(T, S, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
+        else SS_TRY((launch_fwd<ArFX, false>(T, S, wsh, shifts, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
         break;
       case PrunedFormat::kF64Real:
-        if (t16) SS_TRY((launch_fwd16_p<ArDF, true>(T, S, s, bins + o0, kout.get(), nc, z, X + o0, st)));
-        else SS_TRY((launch_fwd<ArDF, true>(T, S, wsh, s, bins + o0, kout.get(), nc, z, X + o0, st)));
+        if (t16) SS_TRY((launch_fwd16_p<ArDF, true>(T, S, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
+        else SS_TRY((launch_fwd<ArDF, true>(T, S, wsh, shifts, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
         break;
       case PrunedFormat::kF32Complex:
-        if (t16) SS_TRY((launch_fwd16_p<ArF32, false>(T, S, s, bins + o0, kout.get(), nc, z, X + o0, st)));
-        else SS_TRY((launch_fwd<ArF32, false>(T, S, wsh, s, bins + o0, kout.get(), nc, z, X + o0, st)));
+        if (t16) SS_TRY((launch_fwd16_p<ArF32, false>(T, S, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
+        else SS_TRY((launch_fwd<ArF32, false>(T, S, wsh, shifts, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
         break;
       default:
-        if (t16) SS_TRY((launch_fwd16_p<ArF32, true>(T, S, s, bins + o0, kout.get(), nc, z, X + o0, st)));
-        else SS_TRY((launch_fwd<ArF32, true>(T, S, wsh, s, bins + o0, kout.get(), nc, z, X + o0, st)));
+        if (t16) SS_TRY((launch_fwd16_p<ArF32, true>(T, S, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
+        else SS_TRY((launch_fwd<ArF32, true>(T, S, wsh, shifts, s, bins + o0, kout.get(), nc, z, unit, X + o0, st)));
         break;
     }
   }

@@ -93,6 +93,20 @@ __device__ __forceinline__ CX mul(const CX a, const TW w) {
   return CX{(hr << 2) + (mr >> 30), (hi << 2) + (mi >> 30)};
 }
 
+// a w / 4, where the caller has the range to spare: the middle products' high
+// words are added as they are (14 integer instructions less per product).
+__device__ __forceinline__ CX mulq(const CX a, const TW w) {
+  constexpr i64 half = 1ll << 31;
+  int ah, al, bh, bl;
+  split(a.re, ah, al);
+  split(a.im, bh, bl);
+  const int nh = -w.ih, nl = -w.il;
+  const i64 hr = mad(bh, nh, mulw(ah, w.rh)), hi = mad(bh, w.rh, mulw(ah, w.ih));
+  const i64 mr = mad(bl, nh, mad(bh, nl, mad(al, w.rh, mad(ah, w.rl, half))));
+  const i64 mi = mad(bl, w.rh, mad(bh, w.rl, mad(al, w.ih, mad(ah, w.il, half))));
+  return CX{mad((int)(mr >> 32), 1, hr), mad((int)(mi >> 32), 1, hi)};
+}
+
 template <int SIGN>
 __device__ __forceinline__ CX mul_t(const CX a, const TW w) {   // a w or a conj(w)
   return mul(a, SIGN > 0 ? w : conj(w));

@@ -606,9 +606,9 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
     }
   }
   if (M > kFullTableMax && !(prec == SS_FP64 && native_fp64_sampling()) && pruned_supported(M)) {
-    SS_TRY(two_level_table(M, &p->prt, st));
+    SS_TRY(two_level_table(M, prec == SS_FP64, &p->prt, st));
     SS_TRY(p->prz.alloc(prec == SS_FP64 ? M : (M + 1) / 2, st));   // float4 or float2 per node
-    SS_TRY(p->prscale.alloc(2, st));
+    SS_TRY(p->prscale.alloc(4, st));
     p->has_pr = true;
   }
   note_alloc();   // the plan allocates its work area
@@ -619,7 +619,7 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
   SS_CUDA(cudaStreamSynchronize(st));
   p->samples.settle(); p->spectrum.settle(); p->lo.settle(); p->hi.settle(); p->full.settle();
   p->fxz.settle(); p->fxtmp.settle(); p->fxtab.settle(); p->fxscale.settle(); p->roots.settle();
-  p->prt.t0.settle(); p->prt.t1.settle(); p->prz.settle(); p->prscale.settle();
+  p->prt.t0.settle(); p->prt.t1.settle(); p->prt.x0.settle(); p->prt.x1.settle(); p->prz.settle(); p->prscale.settle();
   for (auto& t : p->t3) t.settle();
   g_plans.push_front(p);
   while (g_plans.size() > kMaxPlans) g_plans.pop_back();
@@ -1290,11 +1290,12 @@ ss_status pr_sample_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* a
   Terms ta, tf;
   SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
   double* scale = P.prscale.get();
-  k_pair_scale<false><<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
+  const auto pair_scale_of = P.prec == SS_FP64 ? k_pair_scale<true> : k_pair_scale<false>;
+  pair_scale_of<<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
   SS_LAUNCH_CHECK();
   return pruned_eval_pair(P.prt, ta.q.get(), ta.coef.get(), ta.total.get(), a->n_terms, tf.q.get(), tf.coef.get(),
                           tf.total.get(), f->n_terms, scale, P.prz.get(),
-                          P.prec == SS_FP64 ? PrunedFormat::kDfComplex : PrunedFormat::kF32Complex, st);
+                          P.prec == SS_FP64 ? PrunedFormat::kFxComplex : PrunedFormat::kF32Complex, st);
 }
 
 // Output bins of the pruned forward transform: for candidate i, its residue
@@ -1306,20 +1307,29 @@ __global__ void k_pr_bins(const int64_t* __restrict__ res, int64_t n, int64_t M,
   bins[2 * i + 1] = (M - res[i]) % M;
 }
 
-// k_extract_pair on the pruned transform's outputs (x = X[2 i], y = X[2 i + 1]);
-// scale null: one real sum given as samples (scale 1).
+// The bin of sum k from the pruned transform's outputs x (bin b) and y (M - b),
+// as in k_extract_pair; scale null: one real sum given as samples (scale 1);
+// fx: fixed-point samples (scale[2 + k] as there).
+struct BinPr {
+  const double2* X;
+  const double* scale;
+  int64_t M;
+  bool fx;
+  __device__ double2 operator()(int64_t i, int k) const {
+    const double2 x = X[2 * i], y = X[2 * i + 1];
+    const double sc = 0.5 / (double)M * (scale ? scale[k] : 1.0);
+    double2 v = k == 0 ? make_double2((x.x + y.x) * sc, (x.y - y.y) * sc)
+                       : make_double2((x.y + y.y) * sc, (y.x - x.x) * sc);
+    if (fx) v.x += 0.0 * scale[2 + k];   // not a number where a coefficient is not
+    return v;
+  }
+};
+
 template <int WHICH>
-__global__ void k_extract_pr(const int64_t* __restrict__ res, int64_t n, int64_t M, const float4* __restrict__ X,
-                             const double* __restrict__ scale, double2* val, double* mag,
-                             unsigned long long* maxbits) {
+__global__ void k_extract_pr(BinPr bin, int64_t n, double2* val, double* mag, unsigned long long* maxbits) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 xs = X[2 * i], ys = X[2 * i + 1];
-  const double xr = (double)xs.x + (double)xs.y, xi = (double)xs.z + (double)xs.w;
-  const double yr = (double)ys.x + (double)ys.y, yi = (double)ys.z + (double)ys.w;
-  const double sc = 0.5 / (double)M * (scale ? scale[WHICH] : 1.0);
-  const double2 v = WHICH == 0 ? make_double2((xr + yr) * sc, (xi - yi) * sc)
-                               : make_double2((xi + yi) * sc, (yr - xr) * sc);
+  const double2 v = bin(i, WHICH);
   val[i] = v;
   const double m = hypot(v.x, v.y);
   mag[i] = m;
@@ -1334,18 +1344,6 @@ __global__ void k_extract_pr(const int64_t* __restrict__ res, int64_t n, int64_t
 constexpr int kExtractRounds = 4;
 constexpr int kExtractSmall = 1024 * kExtractRounds;
 
-struct BinPr {       // k_extract_pr
-  const float4* X;
-  const double* scale;
-  int64_t M;
-  __device__ double2 operator()(int64_t i, int k) const {
-    const float4 xs = X[2 * i], ys = X[2 * i + 1];
-    const double xr = (double)xs.x + (double)xs.y, xi = (double)xs.z + (double)xs.w;
-    const double yr = (double)ys.x + (double)ys.y, yi = (double)ys.z + (double)ys.w;
-    const double sc = 0.5 / (double)M * (scale ? scale[k] : 1.0);
-    return k == 0 ? make_double2((xr + yr) * sc, (xi - yi) * sc) : make_double2((xi + yi) * sc, (yr - xr) * sc);
-  }
-};
 struct BinFx {       // k_extract_pair
   const longlong2* Z;
   const int64_t* res;
@@ -1592,13 +1590,13 @@ ss_status direct_recover_pair(const SftPlan& P, const LatticeDev& L, const ss_tr
 
 // Pruned forward transform of s (P.prz, or the caller's real samples) at
 // the 2 n_cand bins of the candidates' residues; X: device [2 n_cand].
-ss_status pr_transform(const SftPlan& P, const void* s, bool real, const int64_t* res, int64_t n_cand, float4* X,
+ss_status pr_transform(const SftPlan& P, const void* s, bool real, const int64_t* res, int64_t n_cand, double2* X,
                        cudaStream_t st) {
   DevBuf<int64_t> bins;
   SS_TRY(bins.alloc_tmp(2 * n_cand, st));
   k_pr_bins<<<nblk(n_cand), 256, 0, st>>>(res, n_cand, P.M, bins.get());
   SS_LAUNCH_CHECK();
-  const PrunedFormat fmt = P.prec == SS_FP64 ? (real ? PrunedFormat::kF64Real : PrunedFormat::kDfComplex)
+  const PrunedFormat fmt = P.prec == SS_FP64 ? (real ? PrunedFormat::kF64Real : PrunedFormat::kFxComplex)
                                              : (real ? PrunedFormat::kF32Real : PrunedFormat::kF32Complex);
   return pruned_forward(P.prt, s, fmt, bins.get(), 2 * n_cand, X, st);
 }
@@ -1632,10 +1630,12 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
   SS_TRY(total.alloc_tmp(1, st));
   SS_TRY(residues(cand, n_cand, L, res.get(), st));
   SS_TRY(check_reconstructing_async(cand, n_cand, L, res.get(), true, table.get(), cap, flags.get(), st));
-  DevBuf<float4> X;
+  DevBuf<double2> X;
+  BinPr bin_pr{};
   if (pr) {
     SS_TRY(X.alloc_tmp(2 * n_cand, st));
     SS_TRY(pr_transform(P, pr == 1 ? (const void*)P.prz.get() : samples, pr == 2, res.get(), n_cand, X.get(), st));
+    bin_pr = BinPr{X.get(), pr == 1 ? P.prscale.get() : nullptr, L.M, pr == 1 && P.prec == SS_FP64};
   } else if (!zh && !direct) {
     cufftResult r = cufftSetStream(P.fft, st);
     if (r != CUFFT_SUCCESS) SS_FAIL(SS_ERR_CUDA, "cufftSetStream failed: %d", (int)r);
@@ -1652,7 +1652,7 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
   if (direct) {
     SS_TRY(direct_recover_pair(P, L, direct, nullptr, res.get(), cand, n_cand, tau, fo, vo, total.get(), st));
   } else if (pr && n_cand <= kExtractSmall) {
-    SS_TRY(extract_keep(BinPr{X.get(), pr == 1 ? P.prscale.get() : nullptr, L.M}, 1, n_cand, tau, cand, L.d, fo, vo,
+    SS_TRY(extract_keep(bin_pr, 1, n_cand, tau, cand, L.d, fo, vo,
                         total.get(), st));
   } else if (zh && n_cand <= kExtractSmall) {
     SS_TRY(extract_keep(BinFx{zh, res.get(), P.fxscale.get(), fx_unit(P), L.M}, 1, n_cand, tau, cand, L.d, fo, vo,
@@ -1660,8 +1660,7 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
   } else {
     SS_CUDA(cudaMemsetAsync(maxbits.get(), 0, sizeof(unsigned long long), st));
     if (pr)
-      k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), pr == 1 ? P.prscale.get() : nullptr,
-                                                    val.get(), mag.get(), maxbits.get());
+      k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(bin_pr, n_cand, val.get(), mag.get(), maxbits.get());
     else if (zh)
       k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, fx_unit(P), P.fxscale.get(), val.get(),
                                                       mag.get(), maxbits.get());
@@ -2106,18 +2105,17 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
     // a long 7-smooth lattice: both sums sampled by one sparse evaluation
     // and recovered by one pruned forward transform
     SS_TRY(pr_sample_pair(P, L, a, f, st));
-    DevBuf<float4> X;
+    DevBuf<double2> X;
     SS_TRY(X.alloc_tmp(2 * n_cand, st));
     SS_TRY(pr_transform(P, P.prz.get(), false, res.get(), n_cand, X.get(), st));
+    const BinPr bin_pr{X.get(), P.prscale.get(), L.M, P.prec == SS_FP64};
     if (n_cand <= kExtractSmall)
-      SS_TRY(extract_keep(BinPr{X.get(), P.prscale.get(), L.M}, 2, n_cand, tau, cand, L.d, fo, vo, total.get(), st));
+      SS_TRY(extract_keep(bin_pr, 2, n_cand, tau, cand, L.d, fo, vo, total.get(), st));
     for (int k = 0; k < 2 && n_cand > kExtractSmall; ++k) {
       if (k == 0)
-        k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), P.prscale.get(), val.get(),
-                                                      mag.get(), maxbits.get());
+        k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(bin_pr, n_cand, val.get(), mag.get(), maxbits.get());
       else
-        k_extract_pr<1><<<nblk(n_cand), 256, 0, st>>>(res.get(), n_cand, L.M, X.get(), P.prscale.get(), val.get(),
-                                                      mag.get(), maxbits.get() + 1);
+        k_extract_pr<1><<<nblk(n_cand), 256, 0, st>>>(bin_pr, n_cand, val.get(), mag.get(), maxbits.get() + 1);
       k_keep<<<nblk(n_cand), 256, 0, st>>>(mag.get(), n_cand, maxbits.get() + k, tau, flag.get());
       SS_LAUNCH_CHECK();
       SS_TRY(exclusive_scan_i32(flag.get(), pos.get(), n_cand, total.get() + k, st));

@@ -218,3 +218,25 @@ def test_fp32_samples_by_columns(B, M, n_terms):
     if n_terms == 1:   # no terms at all: an empty spectrum
         f, _ = B.sft_recover(z, M, freq[:0], coef[:0], np.array([[0, 0, 0], [1, 2, 3], [-1, -2, -3]]), precision="fp32")
         assert len(f) == 0
+
+
+@pytest.mark.parametrize("M,n_terms", [(M, n) for M in SIZES + [2**26] for n in (3, 80)] + [(2**24, 600), (2**23, 1100)])
+def test_recover_fixed_point(B, M, n_terms):
+    # the closed form's coefficients: a sample's rounding (2^-55 of sum |c|, times the square root
+    # of a column) averages over M samples; the roots (two factors, each rounded at 2^-54) and the
+    # FP64 sums leave less than 2^-50 of sum |c|
+    freq, coef, I, z = _instance(M, n_terms, 11)
+    gf, gv = B.sft_recover(z, M, freq, coef, I, tau=1e-9)
+    want = osft.true_coefficients(freq, coef)
+    got = gv.cpu().numpy()
+    err = [abs(v - want.get(tuple(k), 0.0)) for k, v in zip(gf.cpu().numpy().tolist(), got)]
+    assert max(err) <= 2.0**-50 * np.abs(coef).sum()
+    big = 1e-8 * max(abs(v) for v in want.values())
+    assert set(map(tuple, gf.cpu().numpy().tolist())) >= {k for k, v in want.items() if abs(v) > big}
+
+
+def test_nonfinite_pair(B):
+    # a coefficient that is not finite leaves no bin
+    freq, coef, I, z = _instance(2**23, 10, 12)
+    coef[4] = np.nan
+    assert len(B.sft_recover(z, 2**23, freq, coef, I, tau=0.0)[0]) == 0
