@@ -2611,6 +2611,7 @@ extern "C" ss_status solve_set_config(ss_stamp s, int32_t block, int32_t blocks_
   C->blocks_per_sm = blocks_per_sm;
   C->chunks_per_block = chunks_per_block;
   C->planned_mode = -1;
+  C->work.rows_total = 0;   // the records anew: the two solver kernels lay them out differently
   return SS_OK;
 }
 
@@ -2673,6 +2674,7 @@ extern "C" ss_status solve(ss_stamp s, const double* f_on_S, double* u_on_S, dou
       H->blocks_per_sm = C->blocks_per_sm;
       H->chunks_per_block = C->chunks_per_block;
       H->planned_mode = -1;
+      H->work.rows_total = 0;
     }
     SS_TRY(stamp_plan_half(s, *H, mode, st));
     SS_TRY(C->fh.ensure(s->rows_pad_h, st));
