@@ -8,7 +8,7 @@ f = 50 sine/cosine pairs of the same form (|supp f| = 100), N = 3
 
 One step = one sparse_spectral_solve call, the whole path at FP64 grade:
 lattice choice and its reconstructing check, recovery of a and f (sampling by
-the double-float sparse evaluation, one pruned double-float transform),
+the fixed-point sparse evaluation, one pruned fixed-point transform),
 stamping set S^3 with its neighbour table, right-hand side on S, FP64 CG to
 relative residual 1e-12 (error against the oracle below 1e-10).
 
@@ -54,7 +54,7 @@ ORACLE_ROWS = 2000           # random rows of the oracle's residual check (plus 
 CPU_SAMPLE_ROWS = 20000      # rows of the CPU baseline's timed operator sample
 WORKLOAD = ("cfg5: d=100, a = 1 + 20 cosines with 3 nonzeros in [-4,4] (s_a=41), f = 50 pairs of the same form "
             "(|supp f|=100), N=3, |S|=1152100, random rank-1 lattice M=2^26 (7-smooth); FP64 recovery "
-            "(double-float sparse evaluation + pruned transform), FP64 CG to relative residual 1e-12")
+            "(fixed-point sparse evaluation + pruned transform), FP64 CG to relative residual 1e-12")
 
 
 def parse():
@@ -167,14 +167,13 @@ def measure_rates():
 
 # ------------------------------------------------------- roofline models
 #
-# The recovery kernels are double-float arithmetic on the FP32 pipes: their
-# algorithmic work is the FP32 instruction count of the double-float
-# operations the transform performs (df.cuh, dfc.cuh): add/subtract 11,
-# product 7, dot product of two pairs 19, multiply-add 15; complex add 22,
-# complex product 38.  Loads, stores and index arithmetic are not counted.
+# The recovery kernels are 64-bit fixed-point arithmetic: their algorithmic work
+# is the instruction count of the operations the transform performs (fxc.cuh):
+# complex add/subtract 4, complex product 26 (8 multiply-adds, the limbs and
+# shifts), product without its final shift 16, product by a power of exp(i pi / 4)
+# 24.  Loads, stores and index arithmetic are not counted.
 
-DF_ADD, DF_MUL, DF_DOT2, DF_FMA = 11, 7, 19, 15
-C_ADD, C_MUL = 2 * DF_ADD, 2 * DF_DOT2
+C_ADD, C_MUL, C_MULQ, C_W8 = 4, 26, 16, 24
 
 
 def radices_py(L):
@@ -186,19 +185,19 @@ def radices_py(L):
     return out if L == 1 else None
 
 
-def butterfly_instr(R, twiddled):
+def butterfly_instr(R, twiddle):
     if R == 2:
         d = 2 * C_ADD
     elif R == 4:
         d = 8 * C_ADD
     elif R == 8:
-        d = 2 * 8 * C_ADD + 2 * (2 * DF_MUL + 2 * DF_ADD) + 8 * C_ADD
+        d = 3 * 8 * C_ADD + 2 * C_W8
     elif R == 16:   # 4 x 4: eight 4-point transforms, eight products by w16 powers (w16^4 = i is free)
-        d = 8 * 8 * C_ADD + 8 * C_MUL
-    else:
+        d = 8 * 8 * C_ADD + 4 * C_MUL + 4 * C_W8
+    else:           # per output pair: 6 limb products a term and part, the shifts and the sums
         H = (R - 1) // 2
-        d = 3 * H * C_ADD + H * (4 * H * DF_FMA + 2 * C_ADD)
-    return d + ((R - 1) * C_MUL if twiddled else 0)
+        d = 3 * H * C_ADD + 4 * H * 2 + H * (12 * H + 16 + 2 * C_ADD)
+    return d + (R - 1) * twiddle
 
 
 def pruned_split_py(M, n, tile=2048):
@@ -222,18 +221,19 @@ def pruned_split_py(M, n, tile=2048):
 
 
 def pruned_instr(kind, M, n_split, n_work):
-    """Algorithmic FP32 instructions of one k_pr_eval (n_work entries) or
+    """Algorithmic instructions of one k_pr_eval (n_work entries) or
     k_pr_fwd (n_work outputs) launch."""
     P, Q, w, rad = pruned_split_py(M, n_split, 2048)
-    if P in (128, 256):   # double-float kernels with 4096-value tiles: a radix-16 pass, then one of radix P / 16
-        w, rad = 4096 // P, [16, P // 16]
+    tw = C_MUL
+    if P in (128, 256):   # 4096-value tiles: a radix-16 pass, then one of radix P / 16
+        w, rad, tw = 4096 // P, [16, P // 16], C_MULQ
     col, Ns = 0, 1
     for R in rad:
-        col += (P // R) * butterfly_instr(R, Ns > 1)
+        col += (P // R) * butterfly_instr(R, tw if Ns > 1 else 0)
         Ns *= R
     tiles = -(-Q // w)
     if kind == "eval":   # per entry: table product and value product, then w multiply-adds
-        per_tile = w * col + n_work * 2 * C_MUL + n_work * w * (C_MUL + C_ADD)
+        per_tile = w * col + n_work * (C_MUL + C_MULQ) + n_work * w * (C_MULQ + C_ADD)
     else:                # per output: w - 1 Horner steps, table product, twist, accumulate
         per_tile = w * col + n_work * ((w - 1) * (C_MUL + C_ADD) + 2 * C_MUL + C_ADD)
     return tiles * per_tile, {"P": P, "Q": Q, "W": w, "radices": rad, "tiles": tiles}
@@ -243,7 +243,7 @@ def pruned_instr(kind, M, n_split, n_work):
 # ncu captures summarised under profiles/, with the hash of the kernel's
 # source file at capture time; a record whose source has changed since is not
 # used (traffic null).
-_PR_SOURCES = ["paper_2302_00752_gb300/csrc/fft_pruned.cu", "paper_2302_00752_gb300/csrc/dfc.cuh",
+_PR_SOURCES = ["paper_2302_00752_gb300/csrc/fft_pruned.cu", "paper_2302_00752_gb300/csrc/fxc.cuh",
                "paper_2302_00752_gb300/csrc/df.cuh"]
 KERNEL_TRAFFIC = {
     "k_pr_eval": {"sources": _PR_SOURCES, "source_sha16": "9dba2b952b8e144a", "dram_bytes_per_launch": 583.52e6,
@@ -287,9 +287,9 @@ def roofline_of(name, ms, ctx, rates):
         kind = "eval" if name == "k_pr_eval" else "fwd"
         n_split, n_work = (ctx["entries_max"], ctx["entries"]) if kind == "eval" else (ctx["outputs"], ctx["outputs"])
         instr, split = pruned_instr(kind, ctx["M"], n_split, n_work)
-        peak = rates["fp32_tflops"] / 2.0                  # FP32 instructions per second (x 1e12)
+        peak = rates["fp32_tflops"] / 2.0                  # issued instructions per second (x 1e12)
         ach = instr / (ms / 1e3) / 1e12
-        out.update({"bound": "alu", "achieved": ach, "peak": peak, "unit": "T FP32 instructions/s", "frac": ach / peak,
+        out.update({"bound": "alu", "achieved": ach, "peak": peak, "unit": "T instructions/s", "frac": ach / peak,
                     "algorithmic_instructions": instr, "split": split,
                     "peak_source": "measured: FP32 FMA rate of libss_peaks.so (instructions = flops / 2)"})
     elif name.startswith("k_solve"):
@@ -783,7 +783,7 @@ def proxy_section(B, gp, flush, Q=1000):
                      "pairs_per_s": pairs / (mc_ms / 1e3),
                      "mc_fp32_frac": pairs * DF_OPS_PER_PAIR / (mc_ms / 1e3) / peak,
                      "note": "mc_ms: whole proxy_mc call (operator, export, three kernels); fraction of the "
-                             "FP32 instruction peak at 150 double-float instructions per pair"}
+                             "FP32 instruction peak at 18 FP32 instructions per pair"}
         res.stamp.destroy()
     return out
 
@@ -884,7 +884,7 @@ def cfg2_section(B, gp, flush, steps=5):
     """The d = 10 plain-FP64 workload: a with 10 cosines in [-8,8]^10 (s_a =
     21), manufactured u with 20 +-pairs, f_hat = L[a_hat] u_hat (|supp f| =
     840), N = 3 (|S| = 334,440), CBC lattice M = 10^6: one sparse_spectral_solve
-    per step (FP64 recovery by the full double-float transform, FP64 CG to
+    per step (FP64 recovery by the full fixed-point transform, FP64 CG to
     1e-12), its error against the exact manufactured solution."""
     import torch
     inst = W.make_cfg2()
