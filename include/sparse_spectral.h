@@ -194,10 +194,15 @@ ss_status sft_recover_samples(const ss_lattice* lat, const void* samples, ss_pre
 /* lattice_sample followed by sft_recover_samples (library-owned sample and
  * FFT buffers).  In FP64 on a 7-smooth M up to 2^22 both transforms (the
  * inverse one that samples g and the forward one that recovers it) run in the
- * library's fixed-point FFT instead of cuFFT.  Its rounding is about 2^-56 of
- * sum |coef| in every bin.  On a shorter M with another prime factor (M up to
- * 2^15, at most 4096 candidates, M times the candidates and M times the terms
- * up to 2^22) samples and bins are direct FP64 sums.  The thresholding and output are as in sft_recover_samples.
+ * library's fixed-point FFT instead of cuFFT.  Beside its rounding to FP64 a bin
+ * carries about 2^-58 M^(-1/4) of sum |coef| and 2^-58 of what shares its row or
+ * column of the transform (one bin in about M^(1/2) does).  A bin that rounds to
+ * nothing there is 0 and passes a threshold of zero, as the rounding of a
+ * floating-point transform would (not where zero is exact: a sum of residues
+ * that are multiples of M / 4, a constant for one).  On a shorter M with another
+ * prime factor (M up to 2^15, at most 4096 candidates, M times the candidates and
+ * M times the terms up to 2^22) samples and bins are direct FP64 sums.  The
+ * thresholding and output are as in sft_recover_samples.
  * Synchronises `stream`. */
 ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_precision prec, const int32_t* cand,
                       int64_t n_cand, int64_t s_max, double tau, int32_t* freq_out, double* val_out,

@@ -13,13 +13,23 @@
 // applies the R-point DFT and writes output r to out[(j / Ns) Ns R + j mod Ns + r Ns]
 // (the Stockham autosort formulation, e.g. Govindaraju et al., SC 2008).
 //
-// Range (units of 2^-58).  An inverse transform (sign +1) sums inputs whose
-// moduli add up to less than 2^60: no partial sum exceeds that.  A forward
-// transform divides by a power of two at or above the radix after every pass
+// Range.  An inverse transform (sign +1, units of 2^-60) sums inputs whose
+// moduli add up to less than 2^62: no partial sum exceeds that (limb products:
+// see mul).  Launch A's
+// columns are classes of bins (mod L2), mostly with a small part of the sum or
+// none: a column counts in units finer by its own power of two (fx_column_lift)
+// and is brought to the common unit as it leaves, where its rounding averages
+// over the L1 values of the column instead of standing in one bin.  The
+// forward transform (units of 2^-58, the samples rounded to them) divides by a power of two at or above the radix after every pass
 // (the plan keeps the running growth at most 1), so values enter a pass below
 // 2^59.5, a product's operands stay below 2^61 and a radix-8 or radix-10 sum
 // below 2^63.  The last pass keeps its sums undivided: its rounding is then the
 // average of its inputs' (0.2 units where a final division would leave 0.7).
+// Launch B's rows hold the classes of bins mod L1, each lifted by its own power
+// of two (fx_row_lift).  So a bin carries a unit averaged over L1 or L2 values,
+// and a unit of what its own row and column hold (all in the common unit: 6 to
+// 20 times as much at M = 10^5 to 4 10^6, and more than in double-float, whose
+// rounding follows the values).
 //
 // On this part an FP64 instruction issues at 1/64 of the FP32 rate, which puts
 // the FP64 library transform of length 10^6 at 205 us; a double-float
@@ -58,7 +68,13 @@ struct FxBlock {
   const int4* tw;      // exp(2 pi i m / L), m < L, in shared memory
   int M, col0;         // col0: first column
   int L, L1, L2;
+  int lift[2];         // left shifts of the block's columns (inverse A) or rows (forward B)
 };
+
+// The double x in units of 2^-(kFxInvFrac + lift).
+__device__ __forceinline__ i64 to_fixed(i64 bits, int lift) {
+  return bits ? __double2ll_rn(__longlong_as_double(bits) * __hiloint2double((1023 + kFxInvFrac + lift) << 20, 0)) : 0;
+}
 
 // One pass: from global memory when `first`, to it (with the twist in launch
 // A) when `last`.  In place (INPL) every thread has at most one butterfly and
@@ -85,6 +101,17 @@ __device__ __forceinline__ void pass(const FxBlock& B, int Ns, int sh, bool firs
 #pragma unroll
         for (int r = 0; r < R; ++r)
           v[r] = ld(__ldcg(B.in + at<SECOND>(B.col0 + c, j + r * nb, B.L2)));
+        const int up = c ? B.lift[1] : B.lift[0];
+        if (SIGN > 0 && !SECOND) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r] = CX{to_fixed(v[r].re, up), to_fixed(v[r].im, up)};
+        } else if (SIGN < 0 && SECOND) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r] = CX{v[r].re << up, v[r].im << up};
+        } else if (SIGN < 0) {   // samples
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r] = scale_down(v[r], kFxInvFrac - kFxFrac);
+        }
       } else {
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = ld(B.a[(j + r * nb) * C + c]);
@@ -101,14 +128,18 @@ __device__ __forceinline__ void pass(const FxBlock& B, int Ns, int sh, bool firs
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int i = base + r * Ns;
-        CX y = SIGN > 0 ? v[r] : scale_down(v[r], sh);
+        const bool twist = last && !SECOND;
+        // a twist that divides by four rounds once, at a finer unit
+        CX y = SIGN > 0 ? v[r] : scale_down(v[r], twist && sh >= 2 ? sh - 2 : sh);
         if (!last) {
           B.b[i * C + c] = st(y);
         } else if (SECOND) {
           B.out[B.col0 + c + B.L1 * i] = st(y);
         } else {   // twist by w_M^{j2 k1} (j2 k1 < M)
-          B.out[at<false>(B.col0 + c, i, B.L2)] =
-              st(mul_t<SIGN>(y, ld_tw(__ldg(B.tab + (B.col0 + c) * i))));
+          const TW w = ld_tw(__ldg(B.tab + (B.col0 + c) * i));
+          if (SIGN > 0) y = scale_down(mul(y, w), c ? B.lift[1] : B.lift[0]);
+          else y = sh >= 2 ? mulq(y, conj(w)) : mul(y, conj(w));
+          B.out[at<false>(B.col0 + c, i, B.L2)] = st(y);
         }
       }
     }
@@ -118,7 +149,8 @@ __device__ __forceinline__ void pass(const FxBlock& B, int Ns, int sh, bool firs
 template <int SIGN, bool SECOND, int C, bool INPL, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_fft_fx(const longlong2* __restrict__ in, longlong2* __restrict__ out,
                                                 const int4* __restrict__ tab, const int4* __restrict__ roots,
-                                                int64_t M, int L1, int L2, FxPasses rad) {
+                                                const int2* __restrict__ classes, int64_t M, int L1, int L2,
+                                                FxPasses rad) {
   extern __shared__ __align__(16) longlong2 sbuf[];
   FxBlock B;
   B.L = SECOND ? L2 : L1;
@@ -133,6 +165,20 @@ __global__ void __launch_bounds__(MAXT, MINB) k_fft_fx(const longlong2* __restri
   B.col0 = (int)blockIdx.x * C;
   B.L1 = L1;
   B.L2 = L2;
+  if constexpr (SIGN > 0 ? !SECOND : SECOND) {
+    bool any = false;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const int2 k = __ldg(classes + B.col0 + c);
+      any |= k.x != 0;
+      B.lift[c] = SECOND ? fx_row_lift(k) : fx_column_lift(k);
+    }
+    if (SIGN > 0 && !any) {   // columns without a bin
+      for (int u = threadIdx.x; u < B.L * C; u += blockDim.x)
+        out[at<false>(B.col0 + u % C, u / C, L2)] = make_longlong2(0, 0);
+      return;
+    }
+  }
   for (int i = threadIdx.x; i < B.L; i += blockDim.x) tw[i] = __ldg(roots + i);   // read from the second pass on
   int Ns = 1;
   for (int p = 0; p < rad.n; ++p) {
@@ -158,18 +204,25 @@ __global__ void __launch_bounds__(MAXT, MINB) k_fft_fx(const longlong2* __restri
   }
 }
 
-// exp(2 pi i r / M) for r < M, then the L1-th and the L2-th roots.
-__global__ void k_fx_table(int64_t M, int L1, int L2, int4* tab) {
+// exp(2 pi i r / M) for r < M, then the L1-th and the L2-th roots: r = r1 L2 +
+// r0 turns by exp(2 pi i r1 / L1) and exp(2 pi i r0 / M), each to a unit.
+__global__ void k_fx_roots(int64_t M, int L1, int L2, int4* part) {   // L1, then L2 entries
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < L1) part[i] = st_tw(exact_root(i, L1));
+  else if (i < L1 + L2) part[i] = st_tw(exact_root(i - L1, M));
+}
+__global__ void k_fx_table(int64_t M, int L1, int L2, const int4* __restrict__ part, int4* tab) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M + L1 + L2) return;
-  const int64_t n = i < M ? M : (i < M + L1 ? L1 : L2), r = i < M ? i : (i < M + L1 ? i - M : i - M - L1);
-  double s, c;
-  sincospi(2.0 * (double)r / (double)n, &s, &c);
-  tab[i] = st_tw(to_tw(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * 0x1p62)));
+  const int64_t r = i < M ? i : (i < M + L1 ? (i - M) * L2 : (i - M - L1) * L1);
+  const TW u = ld_tw(__ldg(part + r / L2));
+  const CX w = mul(CX{((i64)u.rh << 32) + u.rl, ((i64)u.ih << 32) + u.il}, ld_tw(__ldg(part + L1 + r % L2)));
+  tab[i] = st_tw(to_tw(w.re, w.im));
 }
 
 template <int SIGN, bool SECOND, int C>
-ss_status launch_c(const FxFftPlan& F, const int4* tab, const longlong2* in, longlong2* out, cudaStream_t st) {
+ss_status launch_c(const FxFftPlan& F, const int4* tab, const longlong2* in, longlong2* out, const int2* classes,
+                   cudaStream_t st) {
   const int L = SECOND ? F.L2 : F.L1;
   const DfRadices& rad = SECOND ? F.rad2 : F.rad1;
   FxPasses ps;
@@ -190,18 +243,19 @@ ss_status launch_c(const FxFftPlan& F, const int4* tab, const longlong2* in, lon
                     : (threads <= 256 ? k_fft_fx<SIGN, SECOND, C, true, 256, 2> : k_fft_fx<SIGN, SECOND, C, true, 512, 1>);
   if (sm > 48 * 1024) SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   ProfScope prof_("k_fft_fx", st, true);
-  kern<<<(SECOND ? F.L1 : F.L2) / C, threads, sm, st>>>(in, out, tab, tab + F.M + (SECOND ? F.L1 : 0), F.M, F.L1, F.L2,
-                                                        ps);
+  kern<<<(SECOND ? F.L1 : F.L2) / C, threads, sm, st>>>(in, out, tab, tab + F.M + (SECOND ? F.L1 : 0),
+                                                        classes, F.M, F.L1, F.L2, ps);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
 
 template <int SIGN, bool SECOND>
-ss_status launch(const FxFftPlan& F, const int4* tab, const longlong2* in, longlong2* out, cudaStream_t st) {
+ss_status launch(const FxFftPlan& F, const int4* tab, const longlong2* in, longlong2* out, const int2* classes,
+                 cudaStream_t st) {
   // two columns a block where their number is even and five buffers of L values fit
   const int L = SECOND ? F.L2 : F.L1, cols = SECOND ? F.L1 : F.L2;
-  if (cols % 2 == 0 && L <= 2048) return launch_c<SIGN, SECOND, 2>(F, tab, in, out, st);
-  return launch_c<SIGN, SECOND, 1>(F, tab, in, out, st);
+  if (cols % 2 == 0 && L <= 2048) return launch_c<SIGN, SECOND, 2>(F, tab, in, out, classes, st);
+  return launch_c<SIGN, SECOND, 1>(F, tab, in, out, classes, st);
 }
 
 // Radices of the fixed-point passes: 10 while both 2 and 5 divide L (a pass and
@@ -272,19 +326,24 @@ bool fx_fft_plan(int64_t M, FxFftPlan* out) {
 }
 
 ss_status fx_fft_table(const FxFftPlan& F, int4* tab, cudaStream_t st) {
-  k_fx_table<<<(unsigned)((F.M + F.L1 + F.L2 + 255) / 256), 256, 0, st>>>(F.M, F.L1, F.L2, tab);
+  DevBuf<int4> part;
+  SS_TRY(part.alloc_tmp(F.L1 + F.L2, st));
+  k_fx_roots<<<(F.L1 + F.L2 + 63) / 64, 64, 0, st>>>(F.M, F.L1, F.L2, part.get());
+  k_fx_table<<<(unsigned)((F.M + F.L1 + F.L2 + 255) / 256), 256, 0, st>>>(F.M, F.L1, F.L2, part.get(), tab);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
 
-ss_status fx_fft(const FxFftPlan& F, const int4* tab, const longlong2* in, longlong2* tmp, longlong2* out, int sign,
-                 cudaStream_t st) {
-  if (sign > 0) {
-    SS_TRY((launch<1, false>(F, tab, in, tmp, st)));
-    return launch<1, true>(F, tab, tmp, out, st);
-  }
-  SS_TRY((launch<-1, false>(F, tab, in, tmp, st)));
-  return launch<-1, true>(F, tab, tmp, out, st);
+ss_status fx_inverse(const FxFftPlan& F, const int4* tab, const double2* in, const int2* classes, longlong2* tmp,
+                     longlong2* out, cudaStream_t st) {
+  SS_TRY((launch<1, false>(F, tab, reinterpret_cast<const longlong2*>(in), tmp, classes + F.L1, st)));
+  return launch<1, true>(F, tab, tmp, out, nullptr, st);
+}
+
+ss_status fx_forward(const FxFftPlan& F, const int4* tab, const longlong2* in, const int2* classes, longlong2* tmp,
+                     longlong2* out, cudaStream_t st) {
+  SS_TRY((launch<-1, false>(F, tab, in, tmp, nullptr, st)));
+  return launch<-1, true>(F, tab, tmp, out, classes, st);
 }
 
 }  // namespace ss

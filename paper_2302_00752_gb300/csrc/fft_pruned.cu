@@ -359,58 +359,10 @@ struct PrShifts {
   int pass[kDfFftMaxPasses] = {}, col = 0;
 };
 
-// exp(2 pi i r / M) in units of 2^-62, to about one unit (Horner's sums raise an
-// output's root to the W-th power, so FP64's 2^-54 would show): the angle
-// reduced to [0, pi/4] by integers, the series in pairs of doubles.
-struct D2 {
-  double h, l;
-};
-__device__ __forceinline__ D2 d2_norm(double h, double l) {
-  const double s = h + l;
-  return D2{s, l - (s - h)};
-}
-__device__ __forceinline__ D2 d2_mul(const D2 a, const D2 b) {
-  const double p = a.h * b.h;
-  return d2_norm(p, fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
-}
-__device__ __forceinline__ D2 d2_div(const D2 a, double n) {
-  const double q = a.h / n;
-  return d2_norm(q, (fma(-q, n, a.h) + a.l) / n);
-}
-__device__ __forceinline__ D2 d2_one_minus(const D2 a) {
-  const double s = 1.0 - a.h;   // |a| < 1
-  return d2_norm(s, (1.0 - s) - a.h - a.l);
-}
-__device__ long long d2_q62(const D2 a) {
-  const double x = a.h * 0x1p62, y = rint(x);
-  return (long long)y + __double2ll_rn((x - y) + a.l * 0x1p62);
-}
-__device__ fxc::TW exact_root(int64_t r, int64_t M) {
-  const int64_t q = 8 * r / M, rem = 8 * r - q * M, y = q & 1 ? M - rem : rem;
-  const double t = (double)y / (double)M, m = (double)M;
-  const D2 x = d2_mul(D2{0.78539816339744830962, 3.0616169978683830e-17}, D2{t, fma(-t, m, (double)y) / m});
-  const D2 x2 = d2_mul(x, x);
-  D2 c{1.0, 0.0}, sn{1.0, 0.0};
-  for (int k = 12; k > 0; --k) {   // x^26 / 26! < 2^-95
-    c = d2_one_minus(d2_div(d2_mul(x2, c), (double)((2 * k - 1) * (2 * k))));
-    sn = d2_one_minus(d2_div(d2_mul(x2, sn), (double)((2 * k) * (2 * k + 1))));
-  }
-  sn = d2_mul(x, sn);
-  long long a = d2_q62(c), b = d2_q62(sn);   // octant 0
-  if ((q + 1) & 2) {                         // octants 1, 2, 5, 6: nearer to the imaginary axis
-    const long long v = a;
-    a = b;
-    b = v;
-  }
-  if (q >= 2 && q <= 5) a = -a;
-  if (q >= 4) b = -b;
-  return fxc::to_tw(a, b);
-}
-
 __global__ void k_tl_table_fx(int64_t M, int b, int64_t n1, float4* t0, float4* t1) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < (1ll << b)) t0[i] = ArFX::unbits(fxc::st_tw(exact_root(i, M)));
-  if (i < n1) t1[i] = ArFX::unbits(fxc::st_tw(exact_root(i << b, M)));
+  if (i < (1ll << b)) t0[i] = ArFX::unbits(fxc::st_tw(fxc::exact_root(i, M)));
+  if (i < n1) t1[i] = ArFX::unbits(fxc::st_tw(fxc::exact_root(i << b, M)));
 }
 
 __global__ void k_tl_table(int64_t M, int b, int64_t n1, float4* t0, float4* t1) {

@@ -497,10 +497,10 @@ struct SftPlan {
   // fixed-point complex FFT (FP64 recovery of two real sums at once)
   bool has_fx = false;
   FxFftPlan fx;
-  DevBuf<longlong2> fxz, fxtmp;
+  DevBuf<longlong2> fxz, fxtmp;   // fxz: M values, then the classes of its bins (fx_classes)
   DevBuf<int4> fxtab;
   DevBuf<double2> roots;    // exp(2 pi i r / M), r < M, of the direct sums (kDirectMaxM)
-  DevBuf<double> fxscale;   // the two sums' scales and floors of the last round trip
+  DevBuf<double> fxscale;   // the two sums' scales and marks of the last round trip (pair_scale)
   // pruned transforms (on a 7-smooth M above the full table's limit;
   // double-float arithmetic in FP64, FP32 in FP32): two-level twiddle table,
   // the complex sample vector s_a / sigma_a + i s_f / sigma_f and the two
@@ -593,7 +593,7 @@ ss_status get_plan(int64_t M, ss_precision prec, cudaStream_t st, std::shared_pt
     SS_LAUNCH_CHECK();
     p->df = !native_fp64_sampling();
     if (p->df && fx_fft_plan(M, &p->fx)) {
-      SS_TRY(p->fxz.alloc(M, st));
+      SS_TRY(p->fxz.alloc(M + (p->fx.L1 + p->fx.L2 + 1) / 2, st));
       SS_TRY(p->fxtmp.alloc(M, st));
       SS_TRY(p->fxtab.alloc(M + p->fx.L1 + p->fx.L2, st));
       SS_TRY(p->fxscale.alloc(4, st));
@@ -720,11 +720,12 @@ __global__ void k_bin_terms(const int64_t* __restrict__ q, const double2* __rest
 // scale[w] = the power of two at or below sum_t |c_t| of sum w (1 if zero):
 // the two sums share one transform at comparable magnitudes, so each keeps its
 // own relative rounding error; powers of two scale exactly.
-// UNITS (fixed-point spectra, scale[4]): scale[2 + w] is what a bin of sum w
-// that rounds to zero units is read as: a quarter of a unit, so that a
-// threshold of zero keeps every candidate of a nonzero sum, 0 for a sum that
-// is zero, NaN where a coefficient of either sum is not finite or a scale has
-// no reciprocal (integers would hide it).
+// UNITS (fixed-point spectra, scale[4]): scale[2 + w] is NaN where a coefficient
+// of either sum is not finite or a scale has no reciprocal (integers would hide
+// it); else what the threshold takes a bin of sum w for that rounds to nothing:
+// 0 where zero is exact (every residue a multiple of M / 4, where the roots have
+// no rounding), else next to nothing, so that a threshold of zero keeps such a
+// bin (with its value, zero) as it keeps the others' rounding.
 constexpr int kScaleThreads = 512;
 // |c|: hypot, which costs thirty FP64 instructions more, only where squares leave the range
 __device__ __forceinline__ double magnitude(const double2 c) {
@@ -733,14 +734,21 @@ __device__ __forceinline__ double magnitude(const double2 c) {
 }
 
 template <bool UNITS = false>
-__device__ void pair_scale(const double2* const c[2], const int64_t n[2], double* scale) {
+__device__ void pair_scale(const double2* const c[2], const int64_t* const q[2], const int64_t n[2], int64_t M,
+                           double* scale) {
   double total[2];
+  int rounds[2] = {0, 0};   // some nonzero term's residue is no multiple of M / 4
   __shared__ double s_part[kScaleThreads];
   for (int w = 0; w < 2; ++w) {
     double acc = 0.0;
-    for (int64_t t = threadIdx.x; t < n[w]; t += kScaleThreads) acc += magnitude(c[w][t]);
+    for (int64_t t = threadIdx.x; t < n[w]; t += kScaleThreads) {
+      const double m = magnitude(c[w][t]);
+      acc += m;
+      if (UNITS && m > 0.0 && 4 * q[w][t] % M) rounds[w] = 1;
+    }
     s_part[threadIdx.x] = acc;
-    __syncthreads();
+    if (UNITS) rounds[w] = __syncthreads_or(rounds[w]);
+    else __syncthreads();
     for (int o = kScaleThreads / 2; o > 0; o >>= 1) {
       if (threadIdx.x < o) s_part[threadIdx.x] += s_part[threadIdx.x + o];
       __syncthreads();
@@ -751,7 +759,7 @@ __device__ void pair_scale(const double2* const c[2], const int64_t n[2], double
   }
   if (!UNITS || threadIdx.x) return;
   const double bad = 0.0 * (total[0] + 1.0 / scale[0]) + 0.0 * (total[1] + 1.0 / scale[1]);
-  for (int w = 0; w < 2; ++w) scale[2 + w] = bad + (total[w] > 0.0 ? 0.25 : 0.0);
+  for (int w = 0; w < 2; ++w) scale[2 + w] = bad + (rounds[w] ? ldexp(scale[w], -100) : 0.0);
 }
 
 // term counts on the device (merged sums)
@@ -759,10 +767,14 @@ template <bool UNITS>
 __global__ void __launch_bounds__(kScaleThreads) k_pair_scale(const double2* __restrict__ ca,
                                                               const int64_t* __restrict__ na_dev,
                                                               const double2* __restrict__ cf,
-                                                              const int64_t* __restrict__ nf_dev, double* scale) {
+                                                              const int64_t* __restrict__ nf_dev,
+                                                              const int64_t* __restrict__ qa,
+                                                              const int64_t* __restrict__ qf, int64_t M,
+                                                              double* scale) {
   const double2* c[2] = {ca, cf};
+  const int64_t* q[2] = {qa, qf};
   const int64_t n[2] = {*na_dev, *nf_dev};
-  pair_scale<UNITS>(c, n, scale);
+  pair_scale<UNITS>(c, q, n, M, scale);
 }
 
 // term counts from the host (the sums as given)
@@ -771,7 +783,8 @@ __global__ void __launch_bounds__(kScaleThreads) k_pair_scale_n(const double2* _
                                                                 double* scale) {
   const double2* c[2] = {ca, cf};
   const int64_t n[2] = {na, nf};
-  pair_scale(c, n, scale);
+  const int64_t* q[2] = {nullptr, nullptr};
+  pair_scale(c, q, n, 0, scale);
 }
 
 // z[j] = s_a[j] / scale[0] + i s_f[j] / scale[1] (FP32, exact scaling)
@@ -812,7 +825,8 @@ __global__ void k_extract_pair32(const int32_t* __restrict__ cand, int64_t n, La
 __global__ void k_bin_pair(const int64_t* __restrict__ qa, const double2* __restrict__ ca,
                            const int64_t* __restrict__ na_dev, const int64_t* __restrict__ qf,
                            const double2* __restrict__ cf, const int64_t* __restrict__ nf_dev,
-                           const double* __restrict__ scale, int64_t M, longlong2* __restrict__ Z) {
+                           const double* __restrict__ scale, int64_t M, int L1, int L2, double2* __restrict__ Z,
+                           int2* __restrict__ classes) {
   const int64_t na = *na_dev, n = na + *nf_dev;
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -844,41 +858,73 @@ __global__ void k_bin_pair(const int64_t* __restrict__ qa, const double2* __rest
   if (lane) return;
   const double ia = 1.0 / scale[0], jf = 1.0 / scale[1];   // exact: powers of two
   are *= ia; aim *= ia; fre *= jf; fim *= jf;
-  const double un = ldexp(1.0, kFxFrac);
+  auto put = [&](int64_t at, double re, double im) {
+    Z[at] = make_double2(re, im);
+    const int e = (__double2hiint(fabs(re) + fabs(im)) >> 20) & 0x7ff;
+    if (e == 0) return;   // zero, or too small to show
+    int2* k[2] = {classes + at % L1, classes + L1 + at % L2};
+    for (int w = 0; w < 2; ++w) {
+      atomicMax(&k[w]->x, e);
+      atomicAdd(&k[w]->y, 1);
+    }
+  };
   if (b == 0 || 2 * b == M) {
-    Z[b] = make_longlong2(__double2ll_rn(un * are), __double2ll_rn(un * fre));
+    put(b, are, fre);
     return;
   }
   are *= 0.5; aim *= 0.5; fre *= 0.5; fim *= 0.5;
-  Z[b] = make_longlong2(__double2ll_rn(un * (are - fim)), __double2ll_rn(un * (aim + fre)));
-  Z[M - b] = make_longlong2(__double2ll_rn(un * (are + fim)), __double2ll_rn(un * (fre - aim)));
+  put(b, are - fim, aim + fre);
+  put(M - b, are + fim, fre - aim);
 }
 
 // Recovery from the forward transform Zh of s_a + i s_f: with x = Zh[b] and
 // y = Zh[M - b], the bin of the real sum a is (x + conj(y)) / 2 and that of f
 // is (x - conj(y)) / (2 i), each scaled by 1 / M.
-// floor: pair_scale's scale[2 + WHICH].
-template <int WHICH>
-__device__ __forceinline__ double2 pair_bin(const longlong2 x, const longlong2 y, double floor) {
-  const int64_t re = WHICH == 0 ? x.x + y.x : x.y + y.y, im = WHICH == 0 ? x.y - y.y : y.x - x.x;
-  const double f = (re | im) == 0 ? floor : 0.0 * floor;
-  return make_double2((double)re + f, (double)im);
+// A row b mod L1 of the spectrum is lifted by its own power of two (fx_forward),
+// so the two meet in 128 bits: both are below 2^63, the shifts at most 41.
+struct FxSpectrum {
+  const longlong2* Z;
+  const int2* classes;
+  int64_t M;
+  int L1;
+};
+
+// x 2^-a + y 2^-b
+__device__ __forceinline__ double lifted_sum(long long x, int a, long long y, int b) {
+  const int h = max(a, b);
+  const __int128 v = ((__int128)x << (h - a)) + ((__int128)y << (h - b));
+  const unsigned __int128 u = v < 0 ? -(unsigned __int128)v : (unsigned __int128)v;
+  const double r = fma((double)(unsigned long long)(u >> 64), 0x1p64, (double)(unsigned long long)u);
+  return ldexp(v < 0 ? -r : r, -h);
 }
 
-// unit: value of one unit of Zh (2^(shift - kFxFrac)).
+template <int WHICH>
+__device__ __forceinline__ double2 pair_bin(const FxSpectrum& S, int64_t b) {
+  const int64_t nb = b ? S.M - b : 0;
+  const longlong2 x = S.Z[b], y = S.Z[nb];
+  const int hx = fx_row_lift(S.classes[b % S.L1]), hy = fx_row_lift(S.classes[nb % S.L1]);
+  return WHICH == 0 ? make_double2(lifted_sum(x.x, hx, y.x, hy), lifted_sum(x.y, hx, -y.y, hy))
+                    : make_double2(lifted_sum(x.y, hx, y.y, hy), lifted_sum(-x.x, hx, y.x, hy));
+}
+
+// mark: pair_scale's scale[2 + w]
+__device__ __forceinline__ double2 marked(double2 v, double mark) { return make_double2(v.x + 0.0 * mark, v.y); }
+__device__ __forceinline__ double marked_abs(const double2 v, double mark) {
+  return v.x == 0.0 && v.y == 0.0 ? mark : hypot(v.x, v.y);
+}
+
+// unit: value of one unit of an unlifted row (2^(shift - kFxFrac)).
 template <int WHICH>
 __global__ void k_extract_pair(const int32_t* __restrict__ cand, int64_t n, LatticeDev L,
-                               const longlong2* __restrict__ Zh, double unit, const double* __restrict__ scale,
-                               double2* val, double* mag, unsigned long long* maxbits) {
+                               FxSpectrum S, double unit, const double* __restrict__ scale, double2* val,
+                               double* mag, unsigned long long* maxbits) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int64_t b = residue_of(cand + i * L.d, L.d, L);
-  const int64_t nb = (L.M - b) % L.M;
   const double sc = 0.5 / (double)L.M * unit * scale[WHICH];
-  const double2 z = pair_bin<WHICH>(Zh[b], Zh[nb], scale[2 + WHICH]);
-  const double2 v = make_double2(z.x * sc, z.y * sc);
+  const double2 z = pair_bin<WHICH>(S, residue_of(cand + i * L.d, L.d, L));
+  const double2 v = marked(make_double2(z.x * sc, z.y * sc), scale[2 + WHICH]);
   val[i] = v;
-  const double m = hypot(v.x, v.y);
+  const double m = marked_abs(v, scale[2 + WHICH]);
   mag[i] = m;
   atomicMax(maxbits, (unsigned long long)__double_as_longlong(m));
 }
@@ -1251,12 +1297,20 @@ ss_status sample_into(const SftPlan& P, const LatticeDev& L, const ss_trig* g, v
 // Value of one unit of the spectrum that fx_round_trip leaves.
 double fx_unit(const SftPlan& P) { return std::ldexp(1.0, P.fx.shift - kFxFrac); }
 
+// The classes of the bins of P.fxz, behind its M values.
+int2* fx_classes(const SftPlan& P) { return reinterpret_cast<int2*>(P.fxz.get() + P.M); }
+// Bytes that k_bin_pair wants zeroed from P.fxz on.
+size_t fx_zero_bytes(const SftPlan& P) { return P.M * sizeof(longlong2) + (P.fx.L1 + P.fx.L2) * sizeof(int2); }
+
 // The samples of the spectrum in P.fxz, and their spectrum again.
 ss_status fx_round_trip(const SftPlan& P, cudaStream_t st) {
   longlong2* Z = P.fxz.get();
-  SS_TRY(fx_fft(P.fx, P.fxtab.get(), Z, P.fxtmp.get(), Z, +1, st));
-  return fx_fft(P.fx, P.fxtab.get(), Z, P.fxtmp.get(), Z, -1, st);
+  const int2* k = fx_classes(P);
+  SS_TRY(fx_inverse(P.fx, P.fxtab.get(), reinterpret_cast<const double2*>(Z), k, P.fxtmp.get(), Z, st));
+  return fx_forward(P.fx, P.fxtab.get(), Z, k, P.fxtmp.get(), Z, st);
 }
+
+FxSpectrum fx_spectrum(const SftPlan& P) { return FxSpectrum{P.fxz.get(), fx_classes(P), P.M, P.fx.L1}; }
 
 // FP64 plans with the fixed-point transform: the sums a and f (f may be
 // null) are sampled by one inverse transform of Z = S_a + i S_f and the
@@ -1267,14 +1321,16 @@ ss_status fx_recover_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* 
   if (!f) f = &none;
   Terms ta, tf;
   SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
-  longlong2* Z = P.fxz.get();
-  SS_CUDA(cudaMemsetAsync(Z, 0, P.M * sizeof(longlong2), st));
+  double2* Z = reinterpret_cast<double2*>(P.fxz.get());
+  SS_CUDA(cudaMemsetAsync(Z, 0, fx_zero_bytes(P), st));
   double* scale = P.fxscale.get();
-  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
+  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(),
+                                                  ta.q.get(), tf.q.get(), P.M, scale);
   SS_LAUNCH_CHECK();
   if (a->n_terms + f->n_terms > 0) {
     k_bin_pair<<<nblk((a->n_terms + f->n_terms) * 32), 256, 0, st>>>(ta.q.get(), ta.coef.get(), ta.total.get(), tf.q.get(),
-                                                              tf.coef.get(), tf.total.get(), scale, P.M, Z);
+                                                              tf.coef.get(), tf.total.get(), scale, P.M, P.fx.L1, P.fx.L2, Z,
+                                                              fx_classes(P));
     SS_LAUNCH_CHECK();
   }
   return fx_round_trip(P, st);
@@ -1291,7 +1347,8 @@ ss_status pr_sample_pair(const SftPlan& P, const LatticeDev& L, const ss_trig* a
   SS_TRY(prep_terms_pair(L, a, f, &ta, &tf, st));
   double* scale = P.prscale.get();
   const auto pair_scale_of = P.prec == SS_FP64 ? k_pair_scale<true> : k_pair_scale<false>;
-  pair_scale_of<<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), scale);
+  pair_scale_of<<<1, kScaleThreads, 0, st>>>(ta.coef.get(), ta.total.get(), tf.coef.get(), tf.total.get(), ta.q.get(),
+                                             tf.q.get(), P.M, scale);
   SS_LAUNCH_CHECK();
   return pruned_eval_pair(P.prt, ta.q.get(), ta.coef.get(), ta.total.get(), a->n_terms, tf.q.get(), tf.coef.get(),
                           tf.total.get(), f->n_terms, scale, P.prz.get(),
@@ -1320,9 +1377,9 @@ struct BinPr {
     const double sc = 0.5 / (double)M * (scale ? scale[k] : 1.0);
     double2 v = k == 0 ? make_double2((x.x + y.x) * sc, (x.y - y.y) * sc)
                        : make_double2((x.y + y.y) * sc, (y.x - x.x) * sc);
-    if (fx) v.x += 0.0 * scale[2 + k];   // not a number where a coefficient is not
-    return v;
+    return fx ? marked(v, scale[2 + k]) : v;
   }
+  __device__ double mark(int k) const { return fx ? scale[2 + k] : 0.0; }
 };
 
 template <int WHICH>
@@ -1331,7 +1388,7 @@ __global__ void k_extract_pr(BinPr bin, int64_t n, double2* val, double* mag, un
   if (i >= n) return;
   const double2 v = bin(i, WHICH);
   val[i] = v;
-  const double m = hypot(v.x, v.y);
+  const double m = marked_abs(v, bin.mark(WHICH));
   mag[i] = m;
   atomicMax(maxbits, (unsigned long long)__double_as_longlong(m));
 }
@@ -1345,18 +1402,16 @@ constexpr int kExtractRounds = 4;
 constexpr int kExtractSmall = 1024 * kExtractRounds;
 
 struct BinFx {       // k_extract_pair
-  const longlong2* Z;
+  FxSpectrum S;
   const int64_t* res;
   const double* scale;
   double unit;
-  int64_t M;
   __device__ double2 operator()(int64_t i, int k) const {
-    const int64_t b = res[i];
-    const longlong2 x = Z[b], y = Z[b ? M - b : 0];
-    const double2 z = k == 0 ? pair_bin<0>(x, y, scale[2]) : pair_bin<1>(x, y, scale[3]);
-    const double sc = 0.5 / (double)M * unit * scale[k];
-    return make_double2(z.x * sc, z.y * sc);
+    const double2 z = k == 0 ? pair_bin<0>(S, res[i]) : pair_bin<1>(S, res[i]);
+    const double sc = 0.5 / (double)S.M * unit * scale[k];
+    return marked(make_double2(z.x * sc, z.y * sc), scale[2 + k]);
   }
+  __device__ double mark(int k) const { return scale[2 + k]; }
 };
 struct BinDirect {   // the parts of k_direct_bins
   const double2* part;
@@ -1376,6 +1431,7 @@ struct BinDirect {   // the parts of k_direct_bins
     if (bb == 0 || 2 * bb == M) im = 0.0;
     return make_double2(re * sc, (b != bb ? -im : im) * sc);
   }
+  __device__ double mark(int) const { return 0.0; }
 };
 
 template <class Bin>
@@ -1385,7 +1441,7 @@ __global__ void k_extract_bins(Bin bin, int64_t n, double2* __restrict__ val, do
   if (i >= n) return;
   const double2 v = bin(i, k);
   val[k * n + i] = v;
-  mag[k * n + i] = hypot(v.x, v.y);
+  mag[k * n + i] = marked_abs(v, bin.mark(k));
 }
 
 __global__ void __launch_bounds__(1024) k_keep_compact(const double2* __restrict__ val, const double* __restrict__ mag,
@@ -1604,14 +1660,14 @@ ss_status pr_transform(const SftPlan& P, const void* s, bool real, const int64_t
 // Bins, threshold and compaction in candidate order; the reconstructing and
 // symmetry checks run on the device beside them and are read back with the
 // kept count in one synchronisation at the end.
-// zh non-null: the bins come from the fixed-point spectrum zh (real part
-// sum, as left by fx_recover_pair) instead of a transform of samples.
+// zh: the bins come from the plan's fixed-point spectrum (real part sum, as
+// left by fx_recover_pair) instead of a transform of samples.
 // pr != 0: the pruned forward transform of P.prz (pr = 1: complex samples of
 // one sum, scale P.prscale) or of the real FP64 samples (pr = 2).
 // direct non-null: that sum by direct_recover_pair.
 ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* samples, const int32_t* cand, int64_t n_cand,
                        int64_t s_max, double tau, int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st,
-                       const longlong2* zh = nullptr, int pr = 0, const ss_trig* direct = nullptr) {
+                       bool zh = false, int pr = 0, const ss_trig* direct = nullptr) {
   DevBuf<int64_t> res, total;
   DevBuf<unsigned long long> table, maxbits;
   DevBuf<int32_t> flags, flag, pos;
@@ -1655,14 +1711,14 @@ ss_status recover_from(const SftPlan& P, const LatticeDev& L, const void* sample
     SS_TRY(extract_keep(bin_pr, 1, n_cand, tau, cand, L.d, fo, vo,
                         total.get(), st));
   } else if (zh && n_cand <= kExtractSmall) {
-    SS_TRY(extract_keep(BinFx{zh, res.get(), P.fxscale.get(), fx_unit(P), L.M}, 1, n_cand, tau, cand, L.d, fo, vo,
+    SS_TRY(extract_keep(BinFx{fx_spectrum(P), res.get(), P.fxscale.get(), fx_unit(P)}, 1, n_cand, tau, cand, L.d, fo, vo,
                         total.get(), st));
   } else {
     SS_CUDA(cudaMemsetAsync(maxbits.get(), 0, sizeof(unsigned long long), st));
     if (pr)
       k_extract_pr<0><<<nblk(n_cand), 256, 0, st>>>(bin_pr, n_cand, val.get(), mag.get(), maxbits.get());
     else if (zh)
-      k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, zh, fx_unit(P), P.fxscale.get(), val.get(),
+      k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, fx_spectrum(P), fx_unit(P), P.fxscale.get(), val.get(),
                                                       mag.get(), maxbits.get());
     else if (P.prec == SS_FP64)
       k_extract<double2><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, reinterpret_cast<const double2*>(P.spectrum.get()),
@@ -1758,25 +1814,24 @@ __global__ void k_identify_coord(const T2* __restrict__ spec, const int64_t* __r
 // The same from the transform Z of two rows s_i + i s_j (coordinates i and j;
 // below zero: that half is not wanted).  Only the argument counts, so the
 // units and the rows' common scale drop out.
-__global__ void k_identify_coord_pair(const longlong2* __restrict__ Z, int64_t M, const int64_t* __restrict__ bins,
-                                      const double2* __restrict__ x0, int64_t nb, int d, int i, int j, int P,
-                                      int32_t* kf) {
+__global__ void k_identify_coord_pair(FxSpectrum S, const int64_t* __restrict__ bins, const double2* __restrict__ x0,
+                                      int64_t nb, int d, int i, int j, int P, int32_t* kf) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nb) return;
-  const int64_t b = bins[t];
-  const longlong2 x = Z[b], y = Z[b ? M - b : 0];
-  if (i >= 0) kf[t * d + i] = coord_of(pair_bin<0>(x, y, 0.0), x0[t], P);
-  if (j >= 0) kf[t * d + j] = coord_of(pair_bin<1>(x, y, 0.0), x0[t], P);
+  if (i >= 0) kf[t * d + i] = coord_of(pair_bin<0>(S, bins[t]), x0[t], P);
+  if (j >= 0) kf[t * d + j] = coord_of(pair_bin<1>(S, bins[t]), x0[t], P);
 }
 
-// The half spectrum of the first row of Z, X_0[b] (unnormalised).
-__global__ void k_pair_spectrum(const longlong2* __restrict__ Z, int64_t M, int64_t nh, double unit,
-                                const double* __restrict__ scale, double2* __restrict__ spec) {
+// The half spectrum of the first row, X_0[b] (unnormalised; a bin that rounds to
+// nothing as its mark: a threshold of zero does not pass it over).
+__global__ void k_pair_spectrum(FxSpectrum S, int64_t nh, double unit, const double* __restrict__ scale,
+                                double2* __restrict__ spec) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nh) return;
-  const double2 z = pair_bin<0>(Z[b], Z[b ? M - b : 0], scale[2]);
+  double2 z = pair_bin<0>(S, b);
+  if (z.x == 0.0 && z.y == 0.0) z.x = scale[2];
   const double sc = 0.5 * unit * scale[0];
-  spec[b] = make_double2(z.x * sc, z.y * sc);
+  spec[b] = marked(make_double2(z.x * sc, z.y * sc), scale[2]);
 }
 
 // Merged coefficients of the rows i0 and i1 (0: the lattice itself, i >= 1:
@@ -2022,21 +2077,23 @@ ss_status identify_pairs(const SftPlan& P, const LatticeDev& L, const ss_trig* g
   SS_TRY(c1.alloc_tmp(g->n_terms, st));
   double* scale = P.fxscale.get();
   // every row has the same l1 norm: one scale for all
-  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(T.coef.get(), T.total.get(), T.coef.get(), T.total.get(), scale);
+  k_pair_scale<true><<<1, kScaleThreads, 0, st>>>(T.coef.get(), T.total.get(), T.coef.get(), T.total.get(), T.q.get(),
+                                                  T.q.get(), P.M, scale);
   SS_LAUNCH_CHECK();
   auto transform = [&](int i0, int i1) -> ss_status {   // i1 > d: the last row again, unused
     k_rotate_pair<<<nblk(g->n_terms), 256, 0, st>>>(g->freq, T.lead.get(), T.coef.get(), T.total.get(), L.d, i0,
                                                     std::min(i1, L.d), Pp, c0.get(), c1.get());
-    SS_CUDA(cudaMemsetAsync(P.fxz.get(), 0, P.M * sizeof(longlong2), st));
+    SS_CUDA(cudaMemsetAsync(P.fxz.get(), 0, fx_zero_bytes(P), st));
     k_bin_pair<<<nblk(2 * g->n_terms * 32), 256, 0, st>>>(T.q.get(), c0.get(), T.total.get(), T.q.get(), c1.get(),
-                                                           T.total.get(), scale, P.M, P.fxz.get());
+                                                           T.total.get(), scale, P.M, P.fx.L1, P.fx.L2,
+                                                           reinterpret_cast<double2*>(P.fxz.get()), fx_classes(P));
     SS_LAUNCH_CHECK();
     return fx_round_trip(P, st);
   };
   auto first = [&]() -> ss_status {
     SS_TRY(transform(0, 1));
     const int64_t nh = L.M / 2 + 1;
-    k_pair_spectrum<<<nblk(nh), 256, 0, st>>>(P.fxz.get(), L.M, nh, fx_unit(P), scale,
+    k_pair_spectrum<<<nblk(nh), 256, 0, st>>>(fx_spectrum(P), nh, fx_unit(P), scale,
                                               reinterpret_cast<double2*>(P.spectrum.get()));
     SS_LAUNCH_CHECK();
     return SS_OK;
@@ -2044,8 +2101,7 @@ ss_status identify_pairs(const SftPlan& P, const LatticeDev& L, const ss_trig* g
   auto coords = [&](const int64_t* bins, const double2* x0, int64_t nb, int32_t* kf) -> ss_status {
     for (int i = 0; i <= L.d; i += 2) {   // rows i and i + 1 hold the coordinates i - 1 and i
       if (i > 0) SS_TRY(transform(i, i + 1));
-      k_identify_coord_pair<<<nblk(nb), 256, 0, st>>>(P.fxz.get(), L.M, bins, x0, nb, L.d, i - 1, i < L.d ? i : -1, Pp,
-                                                      kf);
+      k_identify_coord_pair<<<nblk(nb), 256, 0, st>>>(fx_spectrum(P), bins, x0, nb, L.d, i - 1, i < L.d ? i : -1, Pp, kf);
       SS_LAUNCH_CHECK();
     }
     return SS_OK;
@@ -2128,11 +2184,10 @@ ss_status sft_recover_both(const ss_lattice* lat, const ss_trig* a, const ss_tri
     // FP64: both sums sampled by one inverse and recovered by one forward
     // fixed-point transform of length M
     SS_TRY(fx_recover_pair(P, L, a, f, st));
-    const longlong2* Z = P.fxz.get();
+    const FxSpectrum Z = fx_spectrum(P);
     const double un = fx_unit(P);
     if (n_cand <= kExtractSmall)
-      SS_TRY(extract_keep(BinFx{Z, res.get(), P.fxscale.get(), un, L.M}, 2, n_cand, tau, cand, L.d, fo, vo, total.get(),
-                          st));
+      SS_TRY(extract_keep(BinFx{Z, res.get(), P.fxscale.get(), un}, 2, n_cand, tau, cand, L.d, fo, vo, total.get(), st));
     for (int k = 0; k < 2 && n_cand > kExtractSmall; ++k) {
       if (k == 0)
         k_extract_pair<0><<<nblk(n_cand), 256, 0, st>>>(cand, n_cand, L, Z, un, P.fxscale.get(), val.get(), mag.get(),
@@ -2244,7 +2299,7 @@ extern "C" ss_status sft_recover_samples(const ss_lattice* lat, const void* samp
   std::shared_ptr<SftPlan> P;
   SS_TRY(get_plan(L.M, prec, st, &P));
   if (P->has_pr)
-    return recover_from(*P, L, samples, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, nullptr, 2);
+    return recover_from(*P, L, samples, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, false, 2);
   return recover_from(*P, L, samples, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st);
 }
 
@@ -2262,13 +2317,13 @@ extern "C" ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_pre
   SS_TRY(get_plan(L.M, prec, st, &P));
   if (P->has_fx) {
     SS_TRY(fx_recover_pair(*P, L, g, nullptr, st));
-    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, P->fxz.get());
+    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, true);
   }
   if (use_direct(*P, g->n_terms, n_cand))
-    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, nullptr, 0, g);
+    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, false, 0, g);
   if (P->has_pr) {
     SS_TRY(pr_sample_pair(*P, L, g, nullptr, st));
-    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, nullptr, 1);
+    return recover_from(*P, L, nullptr, cand, n_cand, s_max, tau, freq_out, val_out, n_out, st, false, 1);
   }
   SS_TRY(sample_into(*P, L, g, P->samples.get(), st));
   return recover_from(*P, L, P->samples.get(), cand, n_cand, s_max, tau, freq_out, val_out, n_out, st);
