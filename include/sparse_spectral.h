@@ -221,8 +221,9 @@ ss_status sft_recover(const ss_lattice* lat, const ss_trig* g, ss_precision prec
  * than s_max terms is SS_ERR_INVALID; a k that does not map back to its bin
  * (k.z mod M != b: the lattice is not reconstructing for the support) is
  * SS_ERR_NOT_RECONSTRUCTING.  Costs d + 1 samplings and FFTs of length M (in
- * FP64 where sft_recover takes the fixed-point FFT: one complex transform each
- * way for two of them).
+ * FP64 where sft_recover takes the fixed-point FFT, for up to 2^20 / M^(1/2)
+ * terms: one complex transform each way for two of them; longer sums keep the
+ * floating-point transforms, whose rounding grows less with their number).
  * Synchronises `stream`. */
 ss_status sft_identify(const ss_lattice* lat, const ss_trig* g, ss_precision prec, int32_t P, int64_t s_max,
                        double tau, int32_t* freq_out, double* val_out, int64_t* n_out, void* stream);

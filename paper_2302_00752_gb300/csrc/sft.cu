@@ -2068,6 +2068,19 @@ ss_status identify_rows(const SftPlan& P, const LatticeDev& L, Rows row, int Pp,
 // two rows at a time as the real and imaginary part of one complex transform
 // each way.  d = 10, 840 terms, M = 10^6: 5.3 ms row by row through cuFFT's
 // FP64 transforms (205 us each way, 11 rows), 1.3 ms so.
+//
+// The fixed-point rounding of a bin follows the l1 norm (2^-58 M^(-1/4) of it),
+// a floating-point transform's the l2 norm (2^-53 log2(M)^(1/2) M^(-1/2) of it),
+// and the l1 norm is at most T^(1/2) l2 norms: up to T M^(1/2) = 2^20 the first
+// is the smaller one or of its size.  T terms of magnitudes over nine decades,
+// median relative error, pairs against rows: 3.3e-14 and 3.1e-14 at T = 420,
+// M = 10^6; 1.0e-13 and 3.3e-14 at T = 2000, M = 2^22 (beyond: rows).
+constexpr double kIdentifyPairs = 1048576.0;
+
+bool identify_by_pairs(const SftPlan& P, int64_t n_terms) {
+  return P.has_fx && n_terms > 0 && (double)n_terms * std::sqrt((double)P.M) <= kIdentifyPairs;
+}
+
 ss_status identify_pairs(const SftPlan& P, const LatticeDev& L, const ss_trig* g, int Pp, int64_t s_max, double tau,
                          int32_t* freq_out, double* val_out, int64_t* n_out, cudaStream_t st) {
   Terms T;
@@ -2343,7 +2356,7 @@ extern "C" ss_status sft_identify(const ss_lattice* lat, const ss_trig* g, ss_pr
   std::shared_ptr<SftPlan> Pl;
   SS_TRY(get_plan(L.M, prec, st, &Pl));
   const SftPlan& PP = *Pl;
-  if (PP.has_fx && g->n_terms > 0)
+  if (identify_by_pairs(PP, g->n_terms))
     return identify_pairs(PP, L, g, P, s_max, tau, freq_out, val_out, n_out, st);
   DevBuf<double2> rot;
   SS_TRY(rot.alloc(std::max<int64_t>(g->n_terms, 1), st));
