@@ -61,16 +61,16 @@ __device__ __forceinline__ float conj_if(float y, bool conj, uint32_t ent) {
 // (REAL: their imaginary parts are exactly 0, so the two dropped products add
 // exact zeros).  GB300 retires two FP64 FMAs per SM clock, so the FP64 operator
 // counts its FP64 instructions.  SKIP leaves out the entries of column `self`
-// (the row's own record is read as zero).
+// (the row's own record is read as zero); the sum starts at acc.
 template <bool CG, bool REAL, bool SKIP>
 __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, int lane,
-                                                 const double2* rec, uint32_t self) {
+                                                 const double2* rec, uint32_t self, const double2 acc) {
   const int32_t w0 = __ldg(op.woff + s), w1 = __ldg(op.woff + s + 1);
   const int64_t base = (int64_t)w0 * kSlice + lane;
   const uint32_t* e = op.ent + base;
   const double2* cf = op.ecoef + base;
   const double* cfr = reinterpret_cast<const double*>(op.ecoef) + base;   // real coefficients
-  double ar = 0.0, ai = 0.0;
+  double ar = acc.x, ai = acc.y;
   int t = 0;
   const int w = w1 - w0;
   for (; t + 4 <= w; t += 4) {
@@ -119,9 +119,9 @@ __device__ __forceinline__ double2 row_apply64_t(const OpView& op, int64_t s, in
 
 template <bool CG = false, bool SKIP = false>
 __device__ __forceinline__ double2 row_apply64(const OpView& op, int64_t s, int lane, const double2* rec,
-                                               uint32_t self = 0) {
-  return op.realc ? row_apply64_t<CG, true, SKIP>(op, s, lane, rec, self)
-                  : row_apply64_t<CG, false, SKIP>(op, s, lane, rec, self);
+                                               uint32_t self = 0, const double2 acc = double2{0.0, 0.0}) {
+  return op.realc ? row_apply64_t<CG, true, SKIP>(op, s, lane, rec, self, acc)
+                  : row_apply64_t<CG, false, SKIP>(op, s, lane, rec, self, acc);
 }
 
 // The same on an array u of n values, taken as zero from n on (padding entries

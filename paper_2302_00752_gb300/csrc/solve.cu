@@ -16,6 +16,10 @@
 // red ones; the black solution D_B^-1 (f_B - C^H u_R) follows once at the end.
 // A set without colours (N = 0, more than 16 levels, ADR operators) has only
 // red rows and skips the black phases: plain CG.
+// The CG's stopping test needs the red rows alone (S u_R = ... has that residual
+// when the black rows are solved for u_R); the residual reported at the end is
+// evaluated on all rows, the black ones' rounding included where it can show
+// (BlackRow).
 //
 // The rows of one or many instances form one row space cut into 32-row slices
 // (one warp each); the slices that hold rows of a colour are listed in order,
@@ -333,7 +337,8 @@ __device__ __forceinline__ void owner_done(const SolveParams& P, InstState& st, 
 // the vector updates, phase B the black half pass and phase Y the red one with
 // the three inner products (gamma, delta, |r|^2): three grid barriers per
 // iteration (two without colours).  Partial slot q3 holds |f|^2.
-// r is also the residual of the whole system: the black rows' is zero.
+// r is also the residual of the whole system, up to the rounding of the black
+// rows' solution.
 
 struct Coeffs {
   double alpha, beta;
@@ -402,18 +407,57 @@ __device__ __forceinline__ Coeffs cg_scalars(const SolveParams& P, int i, int it
 // phase just run; batches read the owners' count (after the grid barrier).
 __device__ __forceinline__ bool one_done(const SolveParams& P, const Smem& sm) { return !P.slice_inst && !sm.flag[0]; }
 
-// End of the FP64 modes: every instance's residual norm (the black rows are
-// solved exactly: the red slots hold all of it).
+// End of the FP64 modes: every instance's residual norm, both colours.
 __device__ void final_rr(const SolveParams& P) {
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
   for (int i = blockIdx.x * nw + (threadIdx.x >> 5); i < P.n_inst; i += gridDim.x * nw) {
-    double t[kNQ];
+    double t[kNQ], b[kNQ] = {};
     inst_sums(P, i, 0, t);
+    if (P.black) inst_sums(P, i, 1, b);
     if (lane == 0) {
-      P.state[i].rr = t[2];
+      P.state[i].rr = t[2] + b[2];
       P.state[i].applies += 1;
     }
   }
+}
+
+// Residual f - (L x)_g of a black row: its product with the red rows, added up
+// from start() on (the solution was formed from the bare product; added to the
+// diagonal's term it rounds anew, as in any evaluation of the row).  A scaled
+// table's black rows hold -D^-1 C^H: there the sum is -x + D^-1 (-C^H x).  What
+// the row needs beside its entries is loaded by start, ahead of the sum.  That is
+// one more FP64 pass over the black rows (d = 100: 18 us, a batch of 128: 80),
+// and rounding stands 2^10 times and more below a red residual above 2^-43 ||f||:
+// then the black rows are not evaluated.
+constexpr double kShow = 0x1p-86, kShowDf = 0x1p-72;   // squared; double-float rounds at 2^-47
+struct BlackRow {
+  double2 f;
+  int64_t nk;
+  __device__ __forceinline__ double2 start(const SolveParams& P, const SolveInst& in, int64_t g, double2 x) {
+    f = f_at(in, g);
+    nk = __ldg(P.norm + g);
+    if (P.op.scaled) return make_double2(-x.x, -x.y);
+    const double d = diag(in);
+    return make_double2(d * x.x, d * x.y);
+  }
+  __device__ __forceinline__ double diag(const SolveInst& in) const { return nk > 0 ? in.dscale * (double)nk : 1.0; }
+  __device__ __forceinline__ double norm2(const SolveParams& P, const SolveInst& in, double2 s) const {
+    const double m = P.op.scaled ? diag(in) : -1.0, rx = fma(m, s.x, f.x), ry = fma(m, s.y, f.y);
+    return fma(rx, rx, ry * ry);
+  }
+};
+// The general phases' sum of them into q2 (0 where it cannot show); the state
+// holds the instances' last red residuals.
+__device__ void black_rr(const SolveParams& P, Smem& sm) {
+  run_phase(P, sm, kBlack, 0b0100u, [&](const Chunk&, int k, int i, bool, int lane) {
+    if (lane == 0) sm.flag[k] = __ldcg(&P.state[i].rr) <= kShow * __ldcg(&P.state[i].bb);
+  }, [&](int64_t g, int64_t s, int lane, int i, int k, double* v) {
+    if (!sm.flag[k]) return;
+    const SolveInst& in = P.inst[i];
+    BlackRow r;
+    const double2 a = r.start(P, in, g, P.xrec[g]);
+    v[2] += r.norm2(P, in, row_apply64<true, true>(P.op, s, lane, P.xrec, (uint32_t)g, a));
+  });
 }
 
 // D^-1 (f - C^H x_R) of a black row from its product y with x_R (a scaled
@@ -536,8 +580,7 @@ __device__ void solve_fp64(const SolveParams& P, Smem& sm) {
     if (P.slice_inst && block_counter(P, 0) >= P.n_inst) break;
     if (!apply((it & 1) ^ 1)) return;
   }
-  // x_B = D^-1 (f_B - C^H x_R), the output, and the true residual f - L x of the
-  // red rows in FP64 (the black rows are solved exactly)
+  // x_B = D^-1 (f_B - C^H x_R), the output, and the true residual f - L x in FP64
   if (colours) {
     run_phase(P, sm, kBlack, 0u, nullptr, [&](int64_t g, int64_t s, int lane, int i, int, double*) {
       const SolveInst& in = P.inst[i];
@@ -547,6 +590,7 @@ __device__ void solve_fp64(const SolveParams& P, Smem& sm) {
       if (l < in.rows) in.u[l] = x;
     });
     if (!grid_sync(P, sm)) return;
+    black_rr(P, sm);
   }
   run_phase(P, sm, kRed, 0b0100u, nullptr, [&](int64_t g, int64_t s, int lane, int i, int, double* v) {
     const SolveInst& in = P.inst[i];
@@ -754,6 +798,16 @@ __device__ void solve_refined(const SolveParams& P, Smem& sm) {
       P.xrec[g] = x;
     });
     if (!grid_sync(P, sm)) return;
+  }
+  if (colours) {   // the black rows' part of the residual
+    black_rr(P, sm);
+    if (!grid_sync(P, sm)) return;
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * nw + (threadIdx.x >> 5); i < P.n_inst; i += gridDim.x * nw) {
+      double b[kNQ];
+      inst_sums(P, i, 1, b);
+      if (lane == 0) P.state[i].rr += b[2];
+    }
   }
   auto put = [&](int64_t g, int64_t, int, int i, int, double*) {
     const SolveInst& in = P.inst[i];
@@ -1006,6 +1060,10 @@ struct K64R {   // FP64, real coefficients
     ai = fma(c, v.y, ai);
   }
   static __device__ __forceinline__ V pack(A ar, A ai) { return make_double2(ar, ai); }
+  static __device__ __forceinline__ void set(A& ar, A& ai, V v) {
+    ar = v.x;
+    ai = v.y;
+  }
 };
 struct K64C : K64R {   // FP64, complex coefficients
   using C = double2;
@@ -1073,6 +1131,10 @@ struct KDF {   // double-float
     }
   }
   static __device__ __forceinline__ V pack(A ar, A ai) { return cdf(ar, ai); }
+  static __device__ __forceinline__ void set(A& ar, A& ai, V v) {
+    ar = re_of(v);
+    ai = im_of(v);
+  }
 };
 
 // Entry words of one batch, and where its coefficients and row are.
@@ -1082,13 +1144,14 @@ struct Words {
   int64_t at;          // first coefficient of the lane
   int32_t row;         // the lane's row
   int32_t left;        // entries of the lane's row from this batch's first on
-  bool on, last, ok;   // row of the phase's colour; last batch of its unit; there is a batch
+  bool on, first, last, ok;   // row of the phase's colour; first, last batch of its unit; there is a batch
 };
 
-// row(g, y) receives every row's product, on one lane per row.
-template <class K, bool SKIP, class Row>
+// row(g, y) receives every row's product, on one lane per row.  The sum starts
+// at start(g, x), x the row's own record (nullptr: at zero).
+template <class K, bool SKIP, class Row, class Start = std::nullptr_t>
 __device__ __forceinline__ void op_phase(const SolveParams& P, const SmemS& sm, const Units& U, int tab,
-                                         const typename K::V* rec, Row row) {
+                                         const typename K::V* rec, Row row, Start start = nullptr) {
   using V = typename K::V;
   using W = Words<K::NB>;
   const OpView& op = P.op;
@@ -1115,6 +1178,7 @@ __device__ __forceinline__ void op_phase(const SolveParams& P, const SmemS& sm, 
 #pragma unroll
     for (int q = 0; q < K::NB; ++q)
       b.e[q] = q * ns < b.left ? __ldg(op.ent + b.at + (int64_t)q * ns * kSlice) : op.pad;
+    b.first = t == tfirst;
     t += K::NB * ns;
     b.last = t >= u.z;   // warp-uniform
     if (b.last) {
@@ -1148,6 +1212,9 @@ __device__ __forceinline__ void op_phase(const SolveParams& P, const SmemS& sm, 
     } else {
       gather(b0, v0, c0);
       b1 = fetch();
+    }
+    if constexpr (!std::is_same<Start, std::nullptr_t>::value) {
+      if (b0.first && b0.on && lane < rows) K::set(ar, ai, start((int64_t)b0.row, __ldcg(rec + b0.row)));
     }
 #pragma unroll
     for (int q = 0; q < K::NB; ++q) {
@@ -1188,6 +1255,26 @@ __device__ __forceinline__ void put_stats(const SolveParams& P, const SmemS& sm,
   st.outer_iters = outer;
   st.applies = applies;
   st.status = status;
+}
+
+// The sum over the black rows into v[2].
+template <class K64>
+__device__ __forceinline__ void one_black_rr(const SolveParams& P, const SmemS& sm, const Units& U, double* v) {
+  const SolveInst& in = P.inst[0];
+  BlackRow r;
+  op_phase<K64, true>(P, sm, U, kOpB, P.xrec, [&](int64_t, double2 s) { v[2] += r.norm2(P, in, s); },
+                      [&](int64_t g, double2 x) { return r.start(P, in, g, x); });
+}
+// The residual of all rows in FP64.
+template <class K64>
+__device__ __forceinline__ void one_rr(const SolveParams& P, const SmemS& sm, const Units& U, bool show, double* v) {
+  const SolveInst& in = P.inst[0];
+  if (show) one_black_rr<K64>(P, sm, U, v);
+  op_phase<K64, false>(P, sm, U, kOpR, P.xrec, [&](int64_t g, double2 y) {
+    const double2 f = f_at(in, g);
+    const double rx = f.x - y.x, ry = f.y - y.y;
+    v[2] = fma(rx, rx, fma(ry, ry, v[2]));
+  });
 }
 
 template <class K64>
@@ -1310,8 +1397,9 @@ __device__ __forceinline__ void one_fp64(const SolveParams& P, SmemS& sm) {
     if (!sync_all(P, sm)) return;
   }
   if (sm.go == 2) status = SS_ERR_NOT_CONVERGED;
-  // x_B, the output, and the true residual f - L x of the red rows in FP64
-  // (the black rows are solved exactly)
+  // x_B, the output, and the true residual f - L x in FP64
+  double v[kNQ] = {};
+  const bool show = sm.t[2] <= kShow * sm.bb;
   if (colours) {
     op_phase<K64, true>(P, sm, U, kOpB, P.xrec, [&](int64_t g, double2 y) {
       const double2 x = black_x(g, y);
@@ -1320,8 +1408,8 @@ __device__ __forceinline__ void one_fp64(const SolveParams& P, SmemS& sm) {
       if (l < in.rows) in.u[l] = x;
     });
     if (!sync_all(P, sm)) return;
+    if (show) one_black_rr<K64>(P, sm, U, v);
   }
-  double v[kNQ] = {};
   op_phase<K64, false>(P, sm, U, kOpR, P.xrec, [&](int64_t g, double2 y) {
     const double2 f = f_at(in, g);
     const double2 r = make_double2(f.x - y.x, f.y - y.y);
@@ -1473,25 +1561,19 @@ __device__ __forceinline__ void one_df64(const SolveParams& P, SmemS& sm) {
     if (!sync_all(P, sm)) return;
   }
   if (sm.go == 2) status = SS_ERR_NOT_CONVERGED;
-  auto put = [&](int64_t g, float4 x) {
+  const bool show = colours && sm.t[2] <= kShowDf * sm.bb;
+  auto put = [&](int64_t g, float4 x4) {   // the output, and the FP64 record of the residual
+    const double2 x = make_double2(df_to_double(re_of(x4)), df_to_double(im_of(x4)));
+    P.xrec[g] = x;
     const int64_t l = g - in.row0;
-    if (l < in.rows) in.u[l] = make_double2(df_to_double(re_of(x)), df_to_double(im_of(x)));
+    if (l < in.rows) in.u[l] = x;
   };
-  if (colours) {
-    op_phase<KDF, true>(P, sm, U, kOpB, P.xdf, [&](int64_t g, float4 y) {
-      const float4 x = black_x(g, y);
-      P.xdf[g] = x;
-      put(g, x);
-    });
-    if (!sync_all(P, sm)) return;
-  }
+  if (colours) op_phase<KDF, true>(P, sm, U, kOpB, P.xdf, [&](int64_t g, float4 y) { put(g, black_x(g, y)); });
+  rows_phase(P, sm, U, kVec, [&](int64_t g) { put(g, P.xdf[g]); });
+  if (!sync_all(P, sm)) return;
   double v[kNQ] = {};
-  op_phase<KDF, false>(P, sm, U, kOpR, P.xdf, [&](int64_t g, float4 y) {
-    const double2 f = f_at(in, g);
-    const double rx = f.x - df_to_double(re_of(y)), ry = f.y - df_to_double(im_of(y));
-    v[2] = fma(rx, rx, fma(ry, ry, v[2]));
-    put(g, __ldcg(P.xdf + g));
-  });
+  if (P.op.realc) one_rr<K64R>(P, sm, U, show, v);
+  else one_rr<K64C>(P, sm, U, show, v);
   if (!sync_sum(P, sm, par, v)) return;
   if (blockIdx.x == 0) {
     all_sums(P, sm, par);
@@ -1669,6 +1751,15 @@ __device__ __forceinline__ void one_refined(const SolveParams& P, SmemS& sm) {
   if (colours) rows_phase(P, sm, U, kOpB, put);
   rows_phase(P, sm, U, kVec, put);
   if (sm.go == 2) status = SS_ERR_NOT_CONVERGED;
+  if (colours && rr <= kShow * sm.bb) {   // the black rows' part of the residual
+    double v[kNQ] = {};
+    one_black_rr<K64>(P, sm, U, v);
+    if (!sync_sum(P, sm, par, v)) return;
+    if (blockIdx.x == 0) {
+      all_sums(P, sm, par);
+      rr += sm.t[2];
+    }
+  }
   put_stats(P, sm, rr, 0, inner, ot, applies, status);
 }
 
