@@ -364,6 +364,8 @@ static ss_status batch_create_impl(ss_batch_s* b, int32_t n, const ss_stamp* sta
     c0 += s->s_a;
   }
   SS_CUDA(cudaMemsetAsync(b->norm.get() + (b->rows_total - 1), 0, sizeof(int64_t), st));
+  // no instance with black rows: no masks (plain CG)
+  if (std::all_of(b->cmask_h.begin(), b->cmask_h.end(), [](uint32_t m) { return m == 0; })) b->cmask_h.clear();
   SS_TRY(work_alloc(b->work, b->rows_total, b->norm.get(), wide_rows.get(), false, st));
   SS_CUDA(cudaStreamSynchronize(st));
   b->norm.settle(); b->woff.settle(); b->slice_inst.settle(); b->ent.settle();

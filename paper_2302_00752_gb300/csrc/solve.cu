@@ -14,8 +14,9 @@
 // application of S is one pass over the entries of L in two half passes:
 //   v_B = -D_B^-1 (C^H u_R)  on the black rows, then  w_R = (L (u_R, v_B))_R  on the
 // red ones; the black solution D_B^-1 (f_B - C^H u_R) follows once at the end.
-// A set without colours (N = 0, more than 16 levels, ADR operators) has only
-// red rows and skips the black phases: plain CG.
+// A set without colours (N = 0, more than 16 levels, ADR operators, or too few
+// black rows to pay: colours_pay in the build) has only red rows and skips the
+// black phases: plain CG.
 // The CG's stopping test needs the red rows alone (S u_R = ... has that residual
 // when the black rows are solved for u_R); the residual reported at the end is
 // evaluated on all rows, the black ones' rounding included where it can show
@@ -356,10 +357,16 @@ __device__ __forceinline__ Coeffs cg_coeffs(int it, double gam, double del, doub
   return c;
 }
 
+// Black rows to eliminate (one instance: its masks may have been dropped on the
+// device; a batch without any has no masks).
+__device__ __forceinline__ bool has_black(const SolveParams& P) {
+  return P.black && (!P.n_items || __ldg(P.n_items + 1) > 0);
+}
+
 // |f|^2 of instance i from the two colours' slots (all lanes).
 __device__ __forceinline__ double sum_bb(const SolveParams& P, int i, const double t[kNQ]) {
   double b[kNQ];
-  if (!P.black) return t[3];
+  if (!has_black(P)) return t[3];
   inst_sums(P, i, 1, b);
   return t[3] + b[3];
 }
@@ -413,7 +420,7 @@ __device__ void final_rr(const SolveParams& P) {
   for (int i = blockIdx.x * nw + (threadIdx.x >> 5); i < P.n_inst; i += gridDim.x * nw) {
     double t[kNQ], b[kNQ] = {};
     inst_sums(P, i, 0, t);
-    if (P.black) inst_sums(P, i, 1, b);
+    if (has_black(P)) inst_sums(P, i, 1, b);
     if (lane == 0) {
       P.state[i].rr = t[2] + b[2];
       P.state[i].applies += 1;
@@ -473,7 +480,7 @@ __device__ __forceinline__ double2 black_x(const SolveParams& P, const SolveInst
 
 __device__ void solve_fp64(const SolveParams& P, Smem& sm) {
   const double tol2 = P.tol * P.tol;
-  const bool colours = P.black != nullptr, scaled = P.op.scaled;
+  const bool colours = has_black(P), scaled = P.op.scaled;
   // The residual is kept as r = D u (D the Jacobi diagonal, u = D^-1 r the
   // preconditioned residual and the gathered record): the vector phase
   // updates u = u - alpha D^-1 s directly, and the apply phase forms
@@ -609,7 +616,7 @@ __device__ void solve_fp64(const SolveParams& P, Smem& sm) {
 
 __device__ void solve_refined(const SolveParams& P, Smem& sm) {
   const double tol2 = P.tol * P.tol, itol2 = P.inner_tol * P.inner_tol;
-  const bool colours = P.black != nullptr;
+  const bool colours = has_black(P);
   float* rd32 = reinterpret_cast<float*>(P.dlt);   // 1 / D in FP32
   for (int ot = 0;; ++ot) {
     const int ocur = ot & 1, onxt = ocur ^ 1;
@@ -1280,7 +1287,7 @@ __device__ __forceinline__ void one_rr(const SolveParams& P, const SmemS& sm, co
 template <class K64>
 __device__ __forceinline__ void one_fp64(const SolveParams& P, SmemS& sm) {
   const double tol2 = P.tol * P.tol;
-  const bool colours = P.black != nullptr, scaled = P.op.scaled;
+  const bool colours = has_black(P), scaled = P.op.scaled;
   const SolveInst& in = P.inst[0];
   // r = D u (D the Jacobi diagonal, u = D^-1 r the gathered record): the
   // vector phase updates u directly, the apply phase forms <r, u> = sum D |u|^2
@@ -1426,7 +1433,7 @@ __device__ __forceinline__ void one_fp64(const SolveParams& P, SmemS& sm) {
 
 __device__ __forceinline__ void one_df64(const SolveParams& P, SmemS& sm) {
   const double tol2 = P.tol * P.tol;
-  const bool colours = P.black != nullptr, scaled = P.op.scaled;
+  const bool colours = has_black(P), scaled = P.op.scaled;
   const SolveInst& in = P.inst[0];
   float4* r4 = reinterpret_cast<float4*>(P.r);
   float4* w4 = reinterpret_cast<float4*>(P.w64);
@@ -1586,7 +1593,7 @@ __device__ __forceinline__ void one_df64(const SolveParams& P, SmemS& sm) {
 template <class K64, class K32>
 __device__ __forceinline__ void one_refined(const SolveParams& P, SmemS& sm) {
   const double tol2 = P.tol * P.tol, itol2 = P.inner_tol * P.inner_tol;
-  const bool colours = P.black != nullptr, scaled = P.op.scaled;
+  const bool colours = has_black(P), scaled = P.op.scaled;
   const SolveInst& in = P.inst[0];
   float* rd32 = reinterpret_cast<float*>(P.dlt);         // 1 / D in FP32
   float2* rec = reinterpret_cast<float2*>(P.urec32);     // u on the red rows, v on the black ones

@@ -735,6 +735,15 @@ __device__ __forceinline__ uint64_t sym_label(uint64_t lin, uint64_t lin_bias) {
   return c < m ? c : m;
 }
 
+// Colours are kept when at most a quarter of the rows of the levels N, N - 2, ...
+// turned red (lost of cand).  In general position none does and CG needs half the
+// iterations; in a set where the steps meet (few dimensions) the rows left black
+// are too few: with a fifth to two thirds of them left, 13 to 15 iterations stood
+// against 15 to 17, and the black half pass and its barrier made batches of such
+// sets slower than plain CG (13,231 rows of 34 entries, 6 instances: 680 us
+// against 496).
+__host__ __device__ inline bool colours_pay(int32_t lost, int32_t cand) { return 4ll * lost <= cand; }
+
 // Row i has the larger label than each of its neighbours of the same level
 // (rows [own0, own0 + own_n)); called for the few rows that have one.
 __device__ __noinline__ bool black_wins(NbrView nb, int64_t i, int32_t own0, uint32_t own_n,
@@ -754,7 +763,8 @@ __device__ __noinline__ bool black_wins(NbrView nb, int64_t i, int32_t own0, uin
 // coefficient).  Also stores the FP64 coefficient of every entry,
 // (|k|^2 + |l|^2 - |p_j|^2) * 2 pi^2 a_hat_j = 4 pi^2 (k.l) a_hat_j (eq. GF), so
 // that the FP64 operator spends four FP64 FMAs per nonzero.
-// With levels given, also the solver's colour mask of the slice: black rows lie
+// With levels given, also the solver's colour mask of the slice and the number of
+// rows that turned red (lost): black rows lie
 // in level N, N - 2, ... and have no black neighbour.  Of two neighbours in
 // those levels the one with the smaller label turns red (both when the labels
 // agree), so k and -k keep one colour and what stays black is independent.
@@ -778,7 +788,7 @@ __global__ void __launch_bounds__(32 * kFillWarps) k_fill_slices(
     NbrView nb, int64_t size, int64_t rows_pad, int j0, const int32_t* __restrict__ woff, int colbits,
     const int64_t* __restrict__ norm, const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64,
     uint32_t* __restrict__ ent, double2* __restrict__ ecoef, bool real, const uint64_t* __restrict__ hl,
-    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask) {
+    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask, int32_t* __restrict__ lost) {
   constexpr int kStride = kFillWords / 4 + 1;   // 16-byte words of a staged row (odd: no bank conflicts)
   __shared__ int4 s_words[kFillWarps][32 * kStride];
   double* ecoef_re = reinterpret_cast<double*>(ecoef);
@@ -846,8 +856,11 @@ __global__ void __launch_bounds__(32 * kFillWarps) k_fill_slices(
   bool blk = i >= size || own_n > 0;
   if (near) blk = black_wins(nb, i, own0, own_n, hl, lin_bias);
   if (lv.n > 0) {
-    const uint32_t m = __ballot_sync(0xffffffffu, blk);
-    if (lane == 0) cmask[s] = m;
+    const uint32_t m = __ballot_sync(0xffffffffu, blk), red = __ballot_sync(0xffffffffu, own_n > 0 && !blk);
+    if (lane == 0) {
+      cmask[s] = m;
+      if (red) atomicAdd(lost, __popc(red));
+    }
   }
   const uint32_t pad = (uint32_t)rows_pad | ((uint32_t)j0 << colbits);
   for (; t < w; ++t) {
@@ -861,7 +874,7 @@ __global__ void __launch_bounds__(32 * kFillWarps) k_fill_dense(
     NbrView nb, int64_t size, int64_t rows_pad, int s_a, int j0, const int32_t* __restrict__ woff, int colbits,
     const int64_t* __restrict__ norm, const int64_t* __restrict__ pnorm, const double2* __restrict__ ca64,
     uint32_t* __restrict__ ent, double2* __restrict__ ecoef, bool real, const uint64_t* __restrict__ hl,
-    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask) {
+    uint64_t lin_bias, int64_t zero_idx, LevelStarts lv, uint32_t* __restrict__ cmask, int32_t* __restrict__ lost) {
   extern __shared__ int4 sm_words[];   // per warp: 32 rows of Ls lo words, then 32 rows of Hs hi words
   __shared__ double2 s_ca[kFillWords];
   __shared__ int64_t s_pn[kFillWords];
@@ -905,8 +918,11 @@ __global__ void __launch_bounds__(32 * kFillWarps) k_fill_dense(
   bool blk = i >= size || own_n > 0;
   if (near) blk = black_wins(nb, i, own0, own_n, hl, lin_bias);
   if (lv.n > 0) {
-    const uint32_t m = __ballot_sync(0xffffffffu, blk);
-    if (lane == 0) cmask[s] = m;
+    const uint32_t m = __ballot_sync(0xffffffffu, blk), red = __ballot_sync(0xffffffffu, own_n > 0 && !blk);
+    if (lane == 0) {
+      cmask[s] = m;
+      if (red) atomicAdd(lost, __popc(red));
+    }
   }
   const int32_t* lw = reinterpret_cast<const int32_t*>(w4) + lane * nb.Ls;
   const int32_t* hw = reinterpret_cast<const int32_t*>(h4) + lane * nb.Hs;
@@ -1383,8 +1399,9 @@ __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plu
                             const double2* __restrict__ ecoef, uint32_t colmask, int colbits, int64_t pad_col,
                             int colbits_h, int j0, const int32_t* __restrict__ hpos,
                             const int32_t* __restrict__ woff_h, uint32_t* ent_h, double2* ecoef_h, bool real,
-                            const int32_t* __restrict__ err, const uint32_t* __restrict__ cmask, uint32_t* cmask_h,
-                            const int64_t* __restrict__ norm_h, double dscale) {
+                            const int32_t* __restrict__ err, uint32_t* cmask, uint32_t* cmask_h,
+                            const int64_t* __restrict__ norm_h, double dscale, const int32_t* __restrict__ lost,
+                            int32_t cand, int64_t n_slices) {
   const double* ecoef_re = reinterpret_cast<const double*>(ecoef);
   double* ecoef_h_re = reinterpret_cast<double*>(ecoef_h);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1397,8 +1414,12 @@ __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plu
   int t = 0;
   bool blk = false;
   if (cmask) {   // the rows' colours (null: none)
-    const int64_t g = i < n_plus ? plus_rows[i] : -1;
-    blk = g < 0 || ((__ldg(cmask + g / kSlice) >> (g % kSlice)) & 1u);
+    if (colours_pay(__ldg(lost), cand)) {
+      const int64_t g = i < n_plus ? plus_rows[i] : -1;
+      blk = g < 0 || ((__ldg(cmask + g / kSlice) >> (g % kSlice)) & 1u);
+    } else if (i < n_slices) {   // every row red, in both tables (more threads than slices)
+      cmask[i] = 0u;
+    }
     const uint32_t m = __ballot_sync(0xffffffffu, blk);
     if (i % kSlice == 0) cmask_h[sh] = m;
   }
@@ -1457,7 +1478,17 @@ __global__ void k_half_fill(const int32_t* __restrict__ plus_rows, int64_t n_plu
 
 // Queue the half system of the current set (no synchronisation; the caller's
 // read-back returns woff_h and the mirror error flag).
-static ss_status build_half(ss_stamp_s* S, cudaStream_t st) {
+// Rows that turned red, behind the colour masks.
+static int32_t* colours_lost(const ss_stamp_s* S) { return S->slice_off.get() + 2 * S->n_slices + 1; }
+
+// The colour masks of a set without a half table, dropped where they do not pay.
+__global__ void k_drop_colours(uint32_t* cmask, int64_t n_slices, const int32_t* __restrict__ lost, int32_t cand) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n_slices && !colours_pay(__ldg(lost), cand)) cmask[i] = 0u;
+}
+
+// cand: rows that could be black.
+static ss_status build_half(ss_stamp_s* S, int32_t cand, cudaStream_t st) {
   S->half_ok = false;
   const int64_t n_plus = (S->size - (S->zero_idx >= 0 ? 1 : 0)) / 2;
   if (!S->half_cand || n_plus < 1 || 2 * n_plus + (S->zero_idx >= 0 ? 1 : 0) != S->size) return SS_OK;
@@ -1521,7 +1552,8 @@ static ss_status build_half(ss_stamp_s* S, cudaStream_t st) {
                                                      S->rows_pad, S->colbits_h, S->j0, S->hpos.get(), S->woff_h.get(),
                                                      S->ent_h.get(), S->ecoef_h.get(), S->a_real, S->err_dev.get(),
                                                      S->colours ? S->cmask.get() : nullptr, S->cmask_h.get(),
-                                                     S->norm_h.get(), 2.0 * kTwoPiSq * S->a0);
+                                                     S->norm_h.get(), 2.0 * kTwoPiSq * S->a0, colours_lost(S), cand,
+                                                     S->n_slices);
   }
   SS_LAUNCH_CHECK();
   S->woff_h_host.clear();   // host copy on demand (stamp_host_tables)
@@ -1579,7 +1611,10 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   SS_TRY(d_nnz.alloc_tmp(1, st));
   SS_TRY(d_wmax.alloc_tmp(1, st));
   SS_TRY(d_total.alloc_tmp(1, st));
+  SS_TRY(S->slice_off.alloc(2 * S->n_slices + 2, st));   // and the colour masks, and the rows they lost
+  S->cmask.view(reinterpret_cast<uint32_t*>(S->slice_off.get() + S->n_slices + 1), S->n_slices);
   SS_TRY(fill_small(st, {{S->norm.get() + S->size, (S->rows_pad + 1 - S->size) * sizeof(int64_t), 0},
+                         {colours_lost(S), sizeof(int32_t), 0},
                          {d_nnz.get(), sizeof(unsigned long long), 0},
                          {d_wmax.get(), sizeof(int32_t), 0},
                          {slice_w.get(), (S->n_slices + 1) * sizeof(int32_t), 0}}));
@@ -1598,8 +1633,6 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
                                                       d_wmax.get());
   }
   SS_LAUNCH_CHECK();
-  SS_TRY(S->slice_off.alloc(2 * S->n_slices + 1, st));   // and the colour masks
-  S->cmask.view(reinterpret_cast<uint32_t*>(S->slice_off.get() + S->n_slices + 1), S->n_slices);
   SS_TRY(scan_lookback(LbRead{slice_w.get()}, LbWrite{S->slice_off.get()}, S->n_slices + 1, d_total.get(),
                        S->err_dev.get(), st));
   int64_t total_w = 0;
@@ -1620,13 +1653,15 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   SS_TRY(S->ecoef64.alloc(S->n_ent + 1, st));
   LevelStarts lv;
   S->colours = false;
+  int32_t cand = 0;   // rows of the levels N, N - 2, ... apart from k = 0
   if (!S->adr && S->N >= 1 && S->N <= kColourLevels) {
-    int64_t red = 0;   // rows of the other levels, apart from k = 0
-    for (int t = 0; t <= S->N; ++t)
-      if ((S->N - t) & 1) {
-        const int64_t a = S->level_start[t], b = S->level_start[t + 1];
-        red += b - a - (S->zero_idx >= a && S->zero_idx < b);
-      }
+    int64_t red = 0;   // rows of the other levels, likewise
+    for (int t = 0; t <= S->N; ++t) {
+      const int64_t a = S->level_start[t], b = S->level_start[t + 1];
+      const int64_t n = b - a - (S->zero_idx >= a && S->zero_idx < b);
+      if ((S->N - t) & 1) red += n;
+      else cand += (int32_t)n;
+    }
     if (red > 0) {
       S->colours = true;
       lv.n = S->N;
@@ -1653,12 +1688,12 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
         k_fill_dense<<<fb, 32 * kFillWarps, (size_t)kFillWarps * 8 * (nb.Ls + nb.Hs) * sizeof(int4), st>>>(
             nb, S->size, S->rows_pad, s_a, S->j0, S->slice_off.get(), colbits_of(S->jbits), S->norm.get(),
             S->pnorm.get(), S->ca64.get(), S->ent.get(), S->ecoef64.get(), S->a_real, S->hl.get(), P.lin_bias,
-            S->zero_idx, lv, S->cmask.get());
+            S->zero_idx, lv, S->cmask.get(), colours_lost(S));
       else
         k_fill_slices<<<fb, 32 * kFillWarps, 0, st>>>(
             nb, S->size, S->rows_pad, S->j0, S->slice_off.get(), colbits_of(S->jbits), S->norm.get(), S->pnorm.get(),
             S->ca64.get(), S->ent.get(), S->ecoef64.get(), S->a_real, S->hl.get(), P.lin_bias, S->zero_idx, lv,
-            S->cmask.get());
+            S->cmask.get(), colours_lost(S));
     }
   }
   SS_LAUNCH_CHECK();
@@ -1667,7 +1702,11 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   k_init_records<<<nblk(S->rows_pad + 1), 256, 0, st>>>(S->norm.get(), S->rows_pad + 1, S->wide, S->nw32.get(),
                                                         S->rec64.get());
   SS_LAUNCH_CHECK();
-  SS_TRY(build_half(S, st));
+  SS_TRY(build_half(S, cand, st));
+  if (S->colours && !S->half_ok) {
+    k_drop_colours<<<nblk(S->n_slices), 256, 0, st>>>(S->cmask.get(), S->n_slices, colours_lost(S), cand);
+    SS_LAUNCH_CHECK();
+  }
   if (defer) {
     S->check_pending = true;
   } else {
