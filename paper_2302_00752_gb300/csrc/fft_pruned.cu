@@ -309,6 +309,9 @@ struct ArFX {
     return C{a.re + h, a.im + h};
   }
   static __device__ __forceinline__ C shr(const C a, int s) { return C{a.re >> s, a.im >> s}; }
+  static __device__ __forceinline__ C shfl(const C a, int m) {
+    return C{__shfl_xor_sync(0xffffffffu, a.re, m), __shfl_xor_sync(0xffffffffu, a.im, m)};
+  }
   static __device__ __forceinline__ T ldt(const TV v) { return fxc::ld_tw(v); }
   static __device__ __forceinline__ TV stt(const T w) { return fxc::st_tw(w); }
   static __device__ __forceinline__ T conjt(const T w) { return fxc::conj(w); }
@@ -353,10 +356,9 @@ struct ArFX {
   static __device__ __forceinline__ double real_out(const V) { return 0.0; }
 };
 
-// Shifts of the general forward transform: after pass p, and of a column's value
-// where Horner's sums take it up.
+// Shifts of the general forward transform after pass p.
 struct PrShifts {
-  int pass[kDfFftMaxPasses] = {}, col = 0;
+  int pass[kDfFftMaxPasses] = {};
 };
 
 __global__ void k_tl_table_fx(int64_t M, int b, int64_t n1, float4* t0, float4* t1) {
@@ -550,14 +552,14 @@ __global__ void k_pr_kout(const int64_t* __restrict__ bins, int64_t n, int P, in
 }
 
 // Evaluation: s[q + Q p] for every tile of W columns (grid-stride over tiles).
+// Fixed point: 80 registers and three blocks an SM (M = 3^16, 300 terms: 1.69 ms,
+// 102 registers and two blocks: 1.89).
 template <class A, bool OUT_REAL>
-__global__ void __launch_bounds__(kPrThreads) k_pr_eval(int64_t M, int P, int64_t Q, int wsh, DfRadices rad,
-                                                        const float4* __restrict__ t0, const float4* __restrict__ t1,
-                                                        int b, const int64_t* __restrict__ er,
-                                                        const float4* __restrict__ ev,
-                                                        const int32_t* __restrict__ boff_g,
-                                                        const float4* __restrict__ estep, int n_stage,
-                                                        int64_t n_tiles, void* __restrict__ out) {
+__global__ void __launch_bounds__(kPrThreads, A::kFixed ? 3 : 0)
+    k_pr_eval(int64_t M, int P, int64_t Q, int wsh, DfRadices rad, const float4* __restrict__ t0,
+              const float4* __restrict__ t1, int b, const int64_t* __restrict__ er, const float4* __restrict__ ev,
+              const int32_t* __restrict__ boff_g, const float4* __restrict__ estep, int n_stage, int64_t n_tiles,
+              void* __restrict__ out) {
   using V = typename A::V;
   using C = typename A::C;
   using TV = typename A::TV;
@@ -724,16 +726,17 @@ __global__ void __launch_bounds__(kPrThreads, 2) k_pr_eval_col(int64_t M, int64_
 // columns, then every output o accumulates
 //   w^{-q0 b_o} sum_i Y[b_o mod P][q0 + i] z_o^i,   z_o = w^{-b_o},
 // the sum over the tile's columns by Horner's scheme (thread o mod blockDim
-// owns output o for the whole launch).
-template <class A, bool IN_REAL>
-__global__ void __launch_bounds__(kPrThreads) k_pr_fwd(int64_t M, int P, int64_t Q, int wsh, DfRadices rad,
-                                                       PrShifts shifts,
-                                                       const float4* __restrict__ t0, const float4* __restrict__ t1,
-                                                       int b, const void* __restrict__ in,
-                                                       const int64_t* __restrict__ ob,
-                                                       const int32_t* __restrict__ kout, int n_out,
-                                                       const float4* __restrict__ oz, int64_t n_tiles,
-                                                       typename A::AccV* __restrict__ partial) {
+// owns output o for the whole launch).  FEW (fixed point, at most a thread per
+// output): lanes share the columns of an output and three blocks an SM hide what
+// is left of the chains; with more outputs the work is in them and two blocks
+// with all registers take less (M = 2^26, 2400 bins: 3.52 ms against 3.77).
+// M = 2^26, 4 bins: 805 us (one lane: 2164), 84 bins: 967 (1143).
+template <class A, bool IN_REAL, bool FEW>
+__global__ void __launch_bounds__(kPrThreads, FEW ? 3 : 0)
+    k_pr_fwd(int64_t M, int P, int64_t Q, int wsh, DfRadices rad, PrShifts shifts, const float4* __restrict__ t0,
+             const float4* __restrict__ t1, int b, const void* __restrict__ in, const int64_t* __restrict__ ob,
+             const int32_t* __restrict__ kout, int n_out, const float4* __restrict__ oz, int64_t n_tiles,
+             typename A::AccV* __restrict__ partial) {
   using V = typename A::V;
   using C = typename A::C;
   using TV = typename A::TV;
@@ -747,6 +750,8 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_fwd(int64_t M, int P, int64_t
   TV* tw = reinterpret_cast<TV*>(Bf + W * CS);
   AccV* acc = reinterpret_cast<AccV*>(tw + P);
   const uint64_t Mu = (uint64_t)M, inv = ~0ull / Mu;
+  int G = 1;   // lanes per output
+  while (2 * G * n_out <= kPrThreads && G < 32 && 2 * G <= W) G *= 2;
   for (int m = threadIdx.x; m < P; m += blockDim.x)
     tw[m] = A::stt(A::template root<1>(t0, t1, b, (uint64_t)m * (uint64_t)Q));
   for (int o = threadIdx.x; o < n_out; o += blockDim.x) acc[o] = A::acc_zero();
@@ -766,12 +771,34 @@ __global__ void __launch_bounds__(kPrThreads) k_pr_fwd(int64_t M, int P, int64_t
     __syncthreads();
     const V* res = columns_dft<A, -1>(Av, Bf, P, wsh, CS, rad, shifts, tw);
     const int wl = Q - q0 < (int64_t)W ? (int)(Q - q0) : W;
+    if constexpr (FEW) {
+      // G lanes an output, each with its W / G columns (zero beyond Q): Horner's
+      // chain of fixed-point products is long where the outputs are few
+      const int cols = W / G, g = threadIdx.x & (G - 1);
+      for (int o0 = 0; o0 < n_out; o0 += kPrThreads / G) {
+        const int o = o0 + threadIdx.x / G;
+        C s = A::zero();
+        if (o < n_out) {
+          const uint64_t q = (uint64_t)(q0 + g * cols);
+          const T w = A::template root<-1>(t0, t1, b, mulmod(q, (uint64_t)ob[o], Mu, inv));
+          const T z = A::step(__ldg(oz + 2 * o));
+          const V* r = res + (g * cols) * CS + kout[o];
+          s = A::ld(r[(cols - 1) * CS]);
+          for (int i = cols - 2; i >= 0; --i) s = A::add(A::mul(s, z), A::ld(r[i * CS]));
+          s = A::mul(s, w);
+        }
+        for (int m = G / 2; m > 0; m >>= 1) s = A::add(s, A::shfl(s, m));
+        if (g == 0 && o < n_out) acc[o] = A::acc_add(acc[o], s);
+      }
+      __syncthreads();
+      continue;
+    }
     for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
       const int k = kout[o];
       const T w = A::template root<-1>(t0, t1, b, mulmod((uint64_t)q0, (uint64_t)ob[o], Mu, inv));
       const T z = A::step(__ldg(oz + 2 * o));   // oz: stride 2 (the step table of width 2, entry 1)
-      C s = A::down(A::ld(res[(wl - 1) * CS + k]), shifts.col);
-      for (int i = wl - 2; i >= 0; --i) s = A::add(A::mul(s, z), A::down(A::ld(res[i * CS + k]), shifts.col));
+      C s = A::ld(res[(wl - 1) * CS + k]);
+      for (int i = wl - 2; i >= 0; --i) s = A::add(A::mul(s, z), A::ld(res[i * CS + k]));
       acc[o] = A::acc_add(acc[o], A::mul(s, w));
     }
     __syncthreads();
@@ -1135,12 +1162,16 @@ ss_status launch_fwd(const TwoLevelTable& T, const PrunedSplit& S, int wsh, cons
   const int64_t n_tiles = (S.Q + S.W - 1) / S.W;
   const size_t smem = fwd_smem<A>(S, nc);
   int grid = 0;
-  SS_TRY(grid_for(k_pr_fwd<A, IN_REAL>, smem, n_tiles, &grid));
+  auto kern = k_pr_fwd<A, IN_REAL, false>;
+  if constexpr (A::kFixed) {
+    if (nc <= kPrThreads) kern = k_pr_fwd<A, IN_REAL, true>;
+  }
+  SS_TRY(grid_for(kern, smem, n_tiles, &grid));
   DevBuf<typename A::AccV> partial;
   SS_TRY(partial.alloc_tmp((size_t)grid * nc, st));
   {
     ProfScope prof_("k_pr_fwd", st, true);
-    k_pr_fwd<A, IN_REAL><<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, shifts, table0<A>(T), table1<A>(T), T.b, in,
+    kern<<<grid, kPrThreads, smem, st>>>(T.M, S.P, S.Q, wsh, S.rad, shifts, table0<A>(T), table1<A>(T), T.b, in,
                                                          ob, kout, nc, oz, n_tiles, partial.get());
     SS_LAUNCH_CHECK();
   }
@@ -1150,20 +1181,20 @@ ss_status launch_fwd(const TwoLevelTable& T, const PrunedSplit& S, int wsh, cons
 }
 
 // Samples stay below 2^56.5; a value enters a pass below 2^59.5 (a radix-8 sum
-// then stays below 2^62.5), and 2^wsh columns add up to less than 2^60.5.
-// Returns the sum of the shifts.
+// then stays below 2^62.5), and 2^wsh columns add up to less than 2^60.5: the
+// last pass divides for them, once per value.  Returns the sum of the shifts.
 int fwd_shifts(const PrunedSplit& S, int wsh, PrShifts* out) {
   double g = -3.0;   // log2 of a value, less 59.5
   int sum = 0;
   for (int p = 0; p < S.rad.n; ++p) {
     g += std::log2((double)S.rad.r[p]);
-    const int sh = p + 1 < S.rad.n && g > 0.0 ? (int)std::ceil(g) : 0;
+    if (p + 1 == S.rad.n) g += wsh - 1.0;
+    const int sh = g > 0.0 ? (int)std::ceil(g) : 0;
     out->pass[p] = sh;
     sum += sh;
     g -= sh;
   }
-  out->col = std::max(0, (int)std::ceil(g + wsh - 1.0));
-  return sum + out->col;
+  return sum;
 }
 
 }  // namespace

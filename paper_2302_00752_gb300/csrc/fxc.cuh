@@ -190,6 +190,16 @@ __device__ __forceinline__ void dft(CX (&v)[R], const TW* cs) {
     v[6] = sub(e2, o2);
     v[3] = add(e3, o3);
     v[7] = sub(e3, o3);
+  } else if constexpr (R == 3) {
+    // cos 120 = -1/2: halves to even (a one-sided rounding would add up in the
+    // bins that all butterflies feed alike), one product per part
+    const CX t = add(v[1], v[2]), d = sub(v[1], v[2]);
+    auto half = [](i64 x) { return (x + ((x >> 1) & 1)) >> 1; };
+    const CX m = CX{v[0].re - half(t.re), v[0].im - half(t.im)};
+    const CX b = mul_si<SIGN>(CX{rmul(d.re, cs[0].ih, cs[0].il), rmul(d.im, cs[0].ih, cs[0].il)});
+    v[0] = add(v[0], t);
+    v[1] = add(m, b);
+    v[2] = sub(m, b);
   } else if constexpr (R == 5) {
     // cos and sin of 72 and 144 degrees; (cos72 + cos144) / 2 = -1/4 exactly, so
     // the real parts need one product, by (cos72 - cos144) / 2 = sqrt 5 / 4
