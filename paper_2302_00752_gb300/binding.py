@@ -222,9 +222,10 @@ def lattice_cbc(freq, raw, M_min):
 
 # A pageable copy waits for the stream; small arrays go through a pinned one
 # (PyTorch's cache of them), so that the host can queue a call while the last
-# one runs: proxy_mc at 1000 points of d = 10, one call after another, 476 us ->
-# 400 us.  Above the limit the copy itself is what counts.
-_PIN_MAX = 1 << 20
+# one runs: proxy_mc at 1000 points of d = 10 (40 KB), one call after another,
+# 476 us -> 400 us.  The detour itself takes 15 us at 40 KB and 30 us from 160 KB
+# on, which a call alone pays for, and there the kernels are long against the wait.
+_PIN_MAX = 1 << 16
 
 
 def _to_dev(a):

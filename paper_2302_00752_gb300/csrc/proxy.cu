@@ -261,26 +261,28 @@ __global__ void __launch_bounds__(kMcThreads, 1) k_mc_terms(const McWork W) {
 }
 
 // f[q] = sum of the first n_f rows of part, r[q] = f[q] + the others (which
-// hold -f^{s,N}).  32 points a block, their rows dealt out to the warps; the
-// order of the additions depends on the sizes alone.
+// hold -f^{s,N}).  32 points a block, their rows dealt out to the warps, as many
+// as there are rows (the whole call at 300,000 points and 6 frequencies: 381 us
+// with 32 warps always, 280 so);
+// the order of the additions depends on the sizes alone.
 constexpr int kFinWarps = 32;
 __global__ void __launch_bounds__(32 * kFinWarps) k_mc_finish(const double* __restrict__ part, int64_t n_f, int64_t n,
                                                               int64_t Q, double* __restrict__ r,
                                                               double* __restrict__ f) {
   __shared__ double sf[kFinWarps][32], sg[kFinWarps][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t q = (int64_t)blockIdx.x * 32 + lane;
   double a = 0.0, b = 0.0;
   if (q < Q) {
-    for (int64_t c = w; c < n_f; c += kFinWarps) a += part[c * Q + q];
+    for (int64_t c = w; c < n_f; c += nw) a += part[c * Q + q];
 #pragma unroll 4
-    for (int64_t c = n_f + w; c < n; c += kFinWarps) b += part[c * Q + q];
+    for (int64_t c = n_f + w; c < n; c += nw) b += part[c * Q + q];
   }
   sf[w][lane] = a;
   sg[w][lane] = b;
   __syncthreads();
   if (w || q >= Q) return;
-  for (int i = 1; i < kFinWarps; ++i) a += sf[i][lane], b += sg[i][lane];
+  for (int i = 1; i < nw; ++i) a += sf[i][lane], b += sg[i][lane];
   f[q] = a;
   r[q] = a + b;
 }
@@ -304,7 +306,9 @@ McKernel mc_kernel(int d) {
 // The tiles and chunks: every block (one per SM, the table fills its shared
 // memory) gets the same number of equal units where there are few tiles, about
 // eight units each where there are many.  Fewer than kMcMinTerms terms do not
-// pay for a row of threads of their own.
+// pay for a row of threads of their own, unless that leaves fewer units than SMs
+// (few terms at many points): then the tiles take fewer points and the rows few
+// terms (the whole call at 56 frequencies, 3000 points, d = 10: 169 -> 129 us).
 constexpr int64_t kMcMinTerms = 32;
 void mc_split(McWork* W) {
   const int64_t sm = sm_count(), n_g = W->n - W->n_f, pts = mc_pts(W->d);
@@ -313,10 +317,17 @@ void mc_split(McWork* W) {
   W->tiles = (W->Q + pts * W->qt - 1) / (pts * W->qt);
   const int64_t want = W->tiles <= sm / 8 ? sm / W->tiles : (8 * sm + W->tiles - 1) / W->tiles;
   W->L = std::max<int64_t>((W->n + want - 1) / want, kMcMinTerms * W->groups);
+  const bool few = W->L > (W->n + want - 1) / want;
   auto chunks = [&](int64_t n) { return (n + W->L - 1) / W->L; };
   while (chunks(W->n_f) + chunks(n_g) > std::max<int64_t>(want, 2)) W->L += W->L / 64 + 1;
   W->chunks_f = chunks(W->n_f);
   W->chunks = W->chunks_f + chunks(n_g);
+  if (few && W->tiles * W->chunks < sm) {
+    const int64_t tiles = (sm + W->chunks - 1) / W->chunks, qt = (W->Q + tiles * pts - 1) / (tiles * pts);
+    W->qt = (int)std::min<int64_t>(W->qt, std::max<int64_t>(32, (qt + 31) / 32 * 32));
+    W->groups = kMcThreads / W->qt;
+    W->tiles = (W->Q + pts * W->qt - 1) / (pts * W->qt);
+  }
 }
 
 }  // namespace
@@ -388,7 +399,9 @@ extern "C" ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, c
     kern<<<(unsigned)std::min<int64_t>(sm_count(), W.tiles * W.chunks), kMcThreads, kTabBytes, st>>>(W);
     SS_LAUNCH_CHECK();
   }
-  k_mc_finish<<<nblk(Q, 32), 32 * kFinWarps, 0, st>>>(part.get(), W.chunks_f * W.groups, W.chunks * W.groups, Q, r_out, f_out);
+  const int64_t rows_f = W.chunks_f * W.groups, rows = W.chunks * W.groups;
+  const int fw = (int)std::max<int64_t>(1, std::min<int64_t>(kFinWarps, std::max(rows_f, rows - rows_f)));
+  k_mc_finish<<<nblk(Q, 32), 32 * fw, 0, st>>>(part.get(), rows_f, rows, Q, r_out, f_out);
   SS_LAUNCH_CHECK();
   return SS_OK;
 }
