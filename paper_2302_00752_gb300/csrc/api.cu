@@ -1,5 +1,6 @@
 // Library-wide helpers behind the C ABI: per-thread error text, version,
 // device properties.
+#include <set>
 #include <atomic>
 #include <map>
 #include <mutex>
@@ -279,6 +280,22 @@ ss_status fill_small(cudaStream_t st, std::initializer_list<FillPart> parts) {
   const size_t blocks = std::min<size_t>((total / 16 + 255) / 256 + 1, 4 * (size_t)sm_count());
   k_fill_small<<<(unsigned)blocks, 256, 0, st>>>(a);
   SS_LAUNCH_CHECK();
+  return SS_OK;
+}
+
+ss_status allow_smem(const void* kernel) {
+  static std::mutex mu;
+  static std::set<std::pair<const void*, int>> done;
+  int dev = 0;
+  SS_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  if (done.count({kernel, dev})) return SS_OK;
+  cudaFuncAttributes at;
+  int most = 0;
+  SS_CUDA(cudaFuncGetAttributes(&at, kernel));
+  SS_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  SS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes));
+  done.insert({kernel, dev});
   return SS_OK;
 }
 

@@ -241,7 +241,7 @@ ss_status launch_c(const FxFftPlan& F, const int4* tab, const longlong2* in, lon
   const size_t sm = ((inpl ? 1 : 2) * (size_t)C + 1) * L * sizeof(longlong2);
   auto kern = !inpl ? k_fft_fx<SIGN, SECOND, C, false, 512, 1>
                     : (threads <= 256 ? k_fft_fx<SIGN, SECOND, C, true, 256, 2> : k_fft_fx<SIGN, SECOND, C, true, 512, 1>);
-  if (sm > 48 * 1024) SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  if (sm > 48 * 1024) SS_TRY(allow_smem(kern));
   ProfScope prof_("k_fft_fx", st, true);
   kern<<<(SECOND ? F.L1 : F.L2) / C, threads, sm, st>>>(in, out, tab, tab + F.M + (SECOND ? F.L1 : 0),
                                                         classes, F.M, F.L1, F.L2, ps);

@@ -1070,7 +1070,7 @@ size_t fwd_smem(const PrunedSplit& S, int n_out) {
 
 template <typename K>
 ss_status grid_for(K kernel, size_t smem, int64_t n_tiles, int* grid) {
-  SS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SS_TRY(allow_smem(kernel));
   int per_sm = 0;
   SS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPrThreads, smem));
   if (per_sm < 1) SS_FAIL(SS_ERR_CUDA, "pruned transform: a block of %zu bytes of shared memory does not fit", smem);

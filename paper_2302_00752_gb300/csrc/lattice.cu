@@ -526,8 +526,7 @@ extern "C" ss_status lattice_cbc(const int32_t* freq, int64_t n, int32_t d, int6
   while (hash_cap < 2 * n) hash_cap <<= 1;
   const size_t hash_smem = (size_t)n * sizeof(int64_t) + (size_t)hash_cap * sizeof(int32_t);
   if (hash_smem <= 200 * 1024) {
-    if (hash_smem > 48 * 1024)
-      SS_CUDA(cudaFuncSetAttribute(k_cbc_try_hash, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hash_smem));
+    if (hash_smem > 48 * 1024) SS_TRY(allow_smem(k_cbc_try_hash));
     SS_TRY(scratch.alloc_tmp(1, st));
   } else {
     SS_TRY(scratch.alloc_tmp((size_t)n_cand * n, st));
@@ -548,7 +547,7 @@ extern "C" ss_status lattice_cbc(const int32_t* freq, int64_t n, int32_t d, int6
   int per_sm = 0;
   bool fused = all_smem <= 200 * 1024 && d > 1;
   if (fused) {
-    SS_CUDA(cudaFuncSetAttribute(k_cbc_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)all_smem));
+    SS_TRY(allow_smem(k_cbc_all));
     SS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cbc_all, kCbcThreads, all_smem));
     fused = (int64_t)per_sm * sm_count() >= n_cand;
   }

@@ -345,7 +345,7 @@ extern "C" ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, c
     SS_FAIL(SS_ERR_INVALID, "proxy_mc: bad sizes");
   if (Q == 0) return SS_OK;
   const McKernel kern = mc_kernel(s->d);
-  SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTabBytes));
+  SS_TRY(allow_smem(kern));
   cudaStream_t st = as_stream(stream);
   DevBuf<float4> tab;
   DevBuf<int4> rec;

@@ -935,7 +935,7 @@ ss_status launch_sample(const SftPlan& P, unsigned grid, size_t sm, const int64_
   using T2 = typename C2<R>::T;
   auto lo = reinterpret_cast<const T2*>(TAB == 2 ? P.full.get() : P.lo.get());
   auto hi = reinterpret_cast<const T2*>(P.hi.get());
-  SS_CUDA(cudaFuncSetAttribute(k_sample<R, TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  SS_TRY((allow_smem(k_sample<R, TAB>)));
   k_sample<R, TAB><<<grid, kSampThreads, sm, st>>>(P.M, P.bl, P.H, lo, hi, q, step, coef, n_dev,
                                                    reinterpret_cast<R*>(out));
   SS_LAUNCH_CHECK();
@@ -1284,7 +1284,7 @@ ss_status sample_into(const SftPlan& P, const LatticeDev& L, const ss_trig* g, v
     SS_TRY(W.alloc_tmp(n * kSampPerThread, st));
     k_term_powers32<<<nblk(n), 256, 0, st>>>(step.get(), total.get(), P.M, W.get());
     const size_t sm = tab_sm + w_sm;
-    SS_CUDA(cudaFuncSetAttribute(k_sample32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    SS_TRY(allow_smem(k_sample32));
     k_sample32<<<grid, kSampThreads, sm, st>>>(P.M, P.n2, P.t3[0].get(), P.t3[1].get(), P.t3[2].get(), q.get(),
                                                W.get(), coef.get(), total.get(), reinterpret_cast<float*>(out));
     SS_LAUNCH_CHECK();

@@ -322,6 +322,13 @@ ss_status ensure_ecoefdf_half(ss_stamp_s* s, cudaStream_t st);
 // FP32 copy of the full or half table's entry coefficients (asynchronous).
 ss_status ensure_ecoef32(ss_stamp_s* s, bool half, cudaStream_t st);
 
+// Raise a kernel's dynamic shared memory limit to what a block may have, once
+// per kernel and device.  The limit is the process's: set to every launch's own
+// size, one thread's launch could find it lowered by another's.
+ss_status allow_smem(const void* kernel);
+template <class... P>
+ss_status allow_smem(void (*kernel)(P...)) { return allow_smem(reinterpret_cast<const void*>(kernel)); }
+
 int sm_count();
 
 // Row replaced by the identity in the operator (the pinned zero frequency of
