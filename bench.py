@@ -295,15 +295,18 @@ def roofline_of(name, ms, ctx, rates):
     elif name.startswith("k_solve"):
         st = ctx["solve_stats"]
         half, realc = bool(st.get("half_system")), bool(st.get("real_coefficients"))
-        nnz_p = ctx["nnz"] / 2 if half else ctx["nnz"]
-        rows_p = (ctx["size"] - (1 if ctx["zero_index"] >= 0 else 0)) // 2 if half else ctx["size"]
+        # CG on the red rows (levels N - 1, N - 3, ...; the workload's points are in
+        # general position, so no row of the others turns red): its vectors live
+        # there, and an application skips the black rows' diagonal
+        share = 0.5 if half else 1.0
+        red, black = share * ctx["red_rows"], share * (ctx["size"] - ctx["red_rows"])
         flops_nnz = 4.0 if realc else 8.0
-        flops = flops_nnz * nnz_p * st["applies"] + 30.0 * rows_p * st["inner_iters"]
+        flops = flops_nnz * (share * ctx["nnz"] - black) * st["applies"] + 30.0 * red * st["inner_iters"]
         peak = rates["fp64_tflops"] * 1e3
         ach = flops / (ms / 1e3) / 1e9
         out.update({"bound": "alu", "achieved": ach, "peak": peak, "unit": "GFLOP/s (FP64)", "frac": ach / peak,
-                    "algorithmic_flops": flops, "half_system": half, "real_coefficients": realc,
-                    "peak_source": "measured: FP64 FMA rate of libss_peaks.so"})
+                    "algorithmic_flops": flops, "red_rows": ctx["red_rows"], "half_system": half,
+                    "real_coefficients": realc, "peak_source": "measured: FP64 FMA rate of libss_peaks.so"})
     elif name == "k_neighbors":
         # pair-symmetric lookups: j0 = (s_a - 1) / 2 per row, one slot probe
         # each; every found pair reads the stored key once (16-byte loads)
@@ -1106,10 +1109,12 @@ def main():
     r_all = step(prep, keep=True)
     e1.record()
     e1.synchronize()
-    r_all["stamp"].destroy()
     all_ms = e0.elapsed_time(e1)
     totals_all = B.profile_totals()
     B.profile(False)
+    level = r_all["stamp"].export()[1].cpu().numpy().astype(np.int64)
+    red_rows = int(((inst.N - level) % 2 == 1).sum())
+    r_all["stamp"].destroy()
     total_ms = sum(step_ms)
     if world > 1:
         tt = torch.tensor([total_ms], dtype=torch.float64, device=dev)
@@ -1198,7 +1203,7 @@ def main():
     n_cand = int(prep.cand.shape[0])
     ctx = {"M": int(prep.M), "entries": 2 * (len(inst.a.freq) + len(inst.f.freq)) - 1,
            "entries_max": 2 * (len(inst.a.freq) + len(inst.f.freq)), "outputs": 2 * n_cand, "size": size,
-           "nnz": nnz, "zero_index": r["zero_index"], "s_a": 2 * len(inst.a.freq) - 1,
+           "nnz": nnz, "red_rows": red_rows, "s_a": 2 * len(inst.a.freq) - 1,
            "key_words": key_words(inst.d, maxabs_f + (inst.N + 1) * maxabs_a), "solve_stats": r["stats"]}
     roofline = roofline_of(dom, kernels[dom]["ms_per_launch"], ctx, rates) if dom else None
     if roofline:
