@@ -71,7 +71,9 @@ typedef struct { int32_t d; int64_t n_terms; const int32_t* freq; const double* 
 typedef struct { int32_t d; int64_t n; const int32_t* freq; const double* val; } ss_sparse;
 
 /* Opaque stamping set: owns its hash table, packed keys, levels, neighbour
- * table and operator scratch until stamp_destroy. */
+ * table and operator scratch until stamp_destroy.  The first refined solve adds
+ * the FP32 copy of its table's entry coefficients (4 bytes an entry, 8 where
+ * a_hat is not real), which is kept as long. */
 typedef struct ss_stamp_s* ss_stamp;
 
 /* Opaque batch of stamping sets prepared for one persistent solve. */
@@ -351,7 +353,7 @@ ss_status proxy_residual(ss_stamp s, const double* u_prefix, int64_t n_u, const 
  * sqrt(sum r^2 / sum f^2).  Phases k.X mod 2^32 are exact integers; each
  * term is evaluated in double-float arithmetic (about 2e-14 of |coef| per
  * term).  r_out, f_out: device FP64 [Q].  Deterministic; asynchronous on
- * `stream`; uses the stamp's operator scratch. */
+ * `stream`. */
 ss_status proxy_mc(ss_stamp s, const double* u_prefix, int64_t n_u, const ss_trig* f, const uint32_t* X, int64_t Q,
                    double* r_out, double* f_out, void* stream);
 
@@ -415,9 +417,10 @@ ss_status solve_set_config(ss_stamp s, int32_t block, int32_t blocks_per_sm, int
  * address does not survive cudaDeviceReset (or any other teardown of the
  * device's primary context): do not call solve_noalloc on a device after
  * resetting it.  Unlike solve() it always solves the full system (never the
- * Hermitian half system), with the work split solve() uses for the full
- * system at its default tile shape.  Every call uses the whole array and leaves its contents
- * there (the next call re-initialises what must start at zero), so calls whose
+ * Hermitian half system), by the phases that batches use, in blocks of 1024
+ * threads, the FP32 operator's entry coefficients formed as it goes; results may
+ * differ from solve()'s in rounding and in iterations, both within tol.  Every
+ * call uses the whole array and leaves its contents there (the next call re-initialises what must start at zero), so calls whose
  * GPU work overlaps - on different streams or threads - race and must be
  * serialised by the caller.  Synchronises `stream`; stats as solve() (without
  * kernel_ms). */

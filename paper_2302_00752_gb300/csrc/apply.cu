@@ -4,7 +4,7 @@
 // gathered straight from the caller's array.  FP64: beside the stored entry
 // coefficients.  FP32: the coefficient is formed from the stamp's norm words.
 //
-// FP64, 334,440 rows: 18.4 us (two or eight entries in flight: 22.0, 18.4);
+// FP64, 334,440 rows: 18 to 19 us (two or eight entries in flight: 22.0, 18.4);
 // with the values copied into a record array first 23 us.  Bound: the gathers'
 // L2 sectors (32 bytes for 16).
 #include <algorithm>

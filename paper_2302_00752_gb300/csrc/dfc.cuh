@@ -34,13 +34,6 @@ __device__ __forceinline__ C4 mul_si(const C4 a) {
   return SIGN > 0 ? C4{df_neg(a.im), a.re} : C4{a.im, df_neg(a.re)};
 }
 
-// exp(sign 2 pi i m / M) from the table of exp(+2 pi i r / M)
-template <int SIGN>
-__device__ __forceinline__ C4 twiddle(const float4* __restrict__ tab, int64_t m) {
-  const float4 e = __ldg(tab + m);
-  return SIGN > 0 ? C4{DF{e.x, e.y}, DF{e.z, e.w}} : C4{DF{e.x, e.y}, DF{-e.z, -e.w}};
-}
-
 // 4-point DFT; the first level's sums are left unnormalised, the outputs are
 // renormalised unless LAZY (then the caller's next level renormalises).
 template <int SIGN, bool LAZY = false>

@@ -275,10 +275,16 @@ struct ArF32 {
   static __device__ __forceinline__ float real_out(const V v) { return v.x; }
 };
 
-// Fixed-point complex values.  An entry (below 1 in modulus, all of them below
-// 4) counts units of 2^-61; its products with the tile's and the column's root
-// divide by four each (mulq), and so does the evaluation's second pass (or its
-// end): samples count units of 2^-55 and stay below 2^56.5.  A sample's rounding
+// Fixed-point complex values.  An entry counts units of 2^-61.  Each sum's scale
+// is the power of two at or below its l1 norm: its entries' moduli add up to less
+// than 2, both sums' to less than 4.  A residue of 0 or M/2 takes the whole real
+// coefficient, below 2 (the constant 1 of a, for instance), the others half of
+// theirs, below 1.  So an entry is one component below 2^62, or two of modulus
+// below 2^61, and the products with the tile's and the column's root divide by
+// four each (mulq): the middle products of the first are below 2^62 (one
+// component) or 2^61.5 + 2^60.5 (two), the second's arguments below 2^60, a
+// column's sum below 2^59.  The evaluation's second pass (or its end) divides by
+// four as well: samples count units of 2^-55 and stay below 2^56.5.  A sample's rounding
 // (a few units) is averaged over the M samples of a bin.  Forward, 4096-value
 // tiles: 2^60.5 after the first pass, divided by four by the second's roots,
 // 2^62.5 (P = 256) or 2^61.5 after it, divided by 2^6: Horner's sums over the

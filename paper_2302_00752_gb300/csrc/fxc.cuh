@@ -65,7 +65,6 @@ __device__ __forceinline__ CX ld(const longlong2 v) { return CX{v.x, v.y}; }
 __device__ __forceinline__ longlong2 st(const CX c) { return make_longlong2(c.re, c.im); }
 __device__ __forceinline__ CX add(const CX a, const CX b) { return CX{a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ CX sub(const CX a, const CX b) { return CX{a.re - b.re, a.im - b.im}; }
-__device__ __forceinline__ CX conj(const CX a) { return CX{a.re, -a.im}; }
 template <int SIGN>
 __device__ __forceinline__ CX mul_si(const CX a) {   // a * (sign i)
   return SIGN > 0 ? CX{-a.im, a.re} : CX{a.im, -a.re};

@@ -1167,10 +1167,6 @@ ss_status prep_terms(const LatticeDev& L, const ss_trig* g, Terms* T, cudaStream
     return SS_OK;
   }
   SS_TRY(T->total.alloc_tmp(1, st));
-  if (n == 0) {
-    SS_CUDA(cudaMemsetAsync(T->total.get(), 0, sizeof(int64_t), st));
-    return SS_OK;
-  }
   if (n > 46340) SS_FAIL(SS_ERR_INVALID, "lattice_sample: more than 46340 terms");
   DevBuf<int32_t> flag, pos, imag, first, sgn;
   DevBuf<double2> merged;

@@ -2876,10 +2876,11 @@ extern "C" ss_status solve(ss_stamp s, const double* f_on_S, double* u_on_S, dou
 
 // ------------------------------------------------------ allocation-free solve
 //
-// solve_noalloc runs the same persistent solver as solve() (the full system,
-// never the Hermitian half system; the same work split as solve() with its
-// default tile shape) but takes all of its workspace from one file-scope
-// device array instead of allocating it.
+// solve_noalloc runs the general phases (k_solve, blocks of 1024 threads) on the
+// full system, never the Hermitian half system; its FP32 operator forms the entry
+// coefficients as it goes.  solve() runs one instance by k_solve_one with 512
+// threads and stored FP32 coefficients: the two may differ in rounding and in
+// iterations.  All of the workspace is one file-scope device array.
 // It serves callers that may not allocate device memory once they run:
 // plug-ins inside a host application that owns all device memory, code that
 // must not stall on cudaMalloc (allocation synchronises the device), or code

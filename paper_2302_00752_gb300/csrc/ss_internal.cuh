@@ -253,8 +253,8 @@ struct ss_stamp_s {
   ss::DevBuf<double2> ecoef64;        // [n_ent] 2 pi^2 (|k|^2 + |l|^2 - |p_j|^2) a_hat_j per entry (FP64 operator)
   ss::DevBuf<float4> ecoefdf;         // [n_ent + 1] the same as double-float, built on first DF64 solve
   ss::DevBuf<int32_t> nw32;           // [rows_pad + 1] FP32 norm words of |k|^2 (norm_word; 0 on padding)
-  // scratch for galerkin_apply (FP64)
-  ss::DevBuf<double2> rec64;          // [rows_pad + 1] scratch of the FP64 operator in place
+  ss::DevBuf<double2> rec64;          // [rows_pad + 1] the input's copy where galerkin_apply (FP64) runs in place;
+                                      // allocated with the set, written by such calls only
   // build state kept for stamp_extend
   int maxabs_f = 0, maxabs_a = 0;     // largest |coordinate| of F and of supp a_hat
   // operator of Remark ADR (advection b.grad u and reaction c u added; not

@@ -1012,13 +1012,11 @@ __global__ void k_fill_slices_adr(KeyParams P, const uint64_t* __restrict__ keys
   }
 }
 
-__global__ void k_init_records(const int64_t* __restrict__ norm, int64_t n, bool wide, int32_t* nw32,
-                               double2* rec64) {
+__global__ void k_init_records(const int64_t* __restrict__ norm, int64_t n, bool wide, int32_t* nw32) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t nr = norm[i];
   nw32[i] = norm_word(nr, wide);
-  rec64[i] = make_double2(0.0, 0.0);
 }
 
 // One thread per coordinate: whole lines of the output (100,000 rows, d = 30:
@@ -1698,9 +1696,8 @@ static ss_status build_operator(ss_stamp_s* S, cudaStream_t st, bool defer) {
   }
   SS_LAUNCH_CHECK();
   SS_TRY(S->nw32.alloc(S->rows_pad + 1, st));
-  SS_TRY(S->rec64.alloc(S->rows_pad + 1, st));
-  k_init_records<<<nblk(S->rows_pad + 1), 256, 0, st>>>(S->norm.get(), S->rows_pad + 1, S->wide, S->nw32.get(),
-                                                        S->rec64.get());
+  SS_TRY(S->rec64.alloc(S->rows_pad + 1, st));   // here: an apply in place may run under stream capture
+  k_init_records<<<nblk(S->rows_pad + 1), 256, 0, st>>>(S->norm.get(), S->rows_pad + 1, S->wide, S->nw32.get());
   SS_LAUNCH_CHECK();
   SS_TRY(build_half(S, cand, st));
   if (S->colours && !S->half_ok) {
