@@ -611,7 +611,7 @@ def apply_section(B, gp, flush, peaks, reps=10):
             res[prec] = d
         st.destroy()
         out[name] = res
-    out["note"] = ("CUDA events around one galerkin_apply call (FP32: one kernel; FP64: pack + operator) after "
+    out["note"] = ("CUDA events around one galerkin_apply call (one kernel) after "
                    "a 512 MB L2 flush (write, "
                    "then read so that no dirty line is written back inside the timed call), all calls queued "
                    "before the first wait; fraction of the measured HBM copy bandwidth")
@@ -686,7 +686,7 @@ def identify_section(B, gp, flush):
         if it:
             times.append(a.elapsed_time(b))
     return {"workload": "cfg2 forcing (d=10, M=10^6)", "P": P, "identified": int(len(f)),
-            "ms": statistics.median(times), "samplings_and_ffts": inst.d + 1}
+            "ms": statistics.median(times), "rows": inst.d + 1, "transform_round_trips": (inst.d + 2) // 2}
 
 
 

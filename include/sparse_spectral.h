@@ -84,7 +84,9 @@ typedef struct {
     int32_t outer_iters;   /* refinement steps (FP32 mode), 1 in FP64 mode */
     int32_t inner_iters;   /* CG iterations in total */
     int32_t applies;       /* operator applications (FP64 + FP32) */
-    double rel_residual;   /* ||f - L u||_2 / ||f||_2 in FP64 at exit */
+    double rel_residual;   /* ||f - L u||_2 / ||f||_2 in FP64 at exit; rows that the solver
+                              eliminates are solved to rounding, which is evaluated where
+                              the other rows' part is below 2^-43 (2^-36 in double-float) */
     double kernel_ms;      /* duration of the persistent solver launch (CUDA events on the stream) */
     int32_t half_system;   /* 1 when the Hermitian half system was solved (see solve) */
     int32_t real_coefficients;   /* 1 when a_hat was real and the operator's entry

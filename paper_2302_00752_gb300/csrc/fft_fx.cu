@@ -35,8 +35,9 @@
 // the FP64 library transform of length 10^6 at 205 us; a double-float
 // addition takes eight to eleven FP32 instructions against two integer ones
 // here, and rounds at 2^-47 where this transform rounds at about 2^-56 of the
-// data's l1 norm.  Bound: integer and multiply-add issue, then shared memory.
-// M = 10^6, one complex transform: 65 us (double-float: 82 us).
+// data's l1 norm.  Bound: latency, of global loads first (12 warps an SM, issue
+// slots 21 to 35 % busy).  M = 10^6, one complex transform: 65 us, 70 with 840
+// terms (double-float: 82 us).
 #include <cmath>
 
 #include "fft_fx.cuh"

@@ -2063,7 +2063,7 @@ ss_status identify_rows(const SftPlan& P, const LatticeDev& L, Rows row, int Pp,
 // rows (a shift turns a merged coefficient like the coefficients it sums), and
 // two rows at a time as the real and imaginary part of one complex transform
 // each way.  d = 10, 840 terms, M = 10^6: 5.3 ms row by row through cuFFT's
-// FP64 transforms (205 us each way, 11 rows), 1.3 ms so.
+// FP64 transforms (205 us each way, 11 rows), 1.36 ms so.
 //
 // The fixed-point rounding of a bin follows the l1 norm (2^-58 M^(-1/4) of it),
 // a floating-point transform's the l2 norm (2^-53 log2(M)^(1/2) M^(-1/2) of it),
